@@ -13,6 +13,8 @@
 // The metrics come either from materialised arrays or, fused, from the closed-form evaluation
 // itself, walked in the tiled order of tiled.cuh so the integer task tables are built once per
 // (model, batch, TP, length) point.
+#include <algorithm>
+
 #include "select_sink.cuh"
 
 namespace guide {
@@ -905,8 +907,8 @@ static size_t topk_stream_offset(u32 k) {
 static size_t pareto_stream_offset() {
     return (256 + (size_t)SEL_MAX_BLOCKS * sizeof(u32) + (size_t)SEL_MAX_BLOCKS * GUIDE_PARETO_MAX * sizeof(P3) + 255) / 256 * 256;
 }
-size_t topk_workspace_bytes(u32 k) { return topk_stream_offset(k) + topk_stream_bytes(); }
-size_t pareto_workspace_bytes() { return pareto_stream_offset() + pareto_stream_bytes(); }
+size_t topk_workspace_bytes(u32 k) { return topk_stream_offset(k) + std::max(topk_stream_bytes(), topk_coop_bytes()); }
+size_t pareto_workspace_bytes() { return pareto_stream_offset() + std::max(pareto_stream_bytes(), pareto_coop_bytes()); }
 
 static u32 grid_for(u64 count, u32 items, u32 blocks_per_sm, u32 max_blocks) {
     // every block has fixed costs (first sorts, final sort, its list in the merge): give each at
@@ -1017,15 +1019,8 @@ int launch_topk(const DSpace &s, Range r, const guide_outputs *mat, int time_mod
     unsigned char *w = (unsigned char *)ws;
     if (mat) {
         MatSource src{*mat, make_cons(c), key, -1, mat_vec_ok(*mat)};
-        if (k <= STREAM_TOPK_MAX_K && stream_eligible(*mat, r)) {
-            // streaming path first; the accumulator kernels are queued behind it and return at once
-            // unless it raised the redo flag
-            int rc;
-            u32 *header = (u32 *)w;                         // reset by the streaming path itself
-            if ((rc = launch_topk_stream(r, *mat, c, key, k, header, w + topk_stream_offset(k), idx_out, key_out, count_out, st)))
-                return rc;
-            return run_topk_scan(src, r, k, negate, SEL_MAX_BLOCKS, w, idx_out, key_out, count_out, st, header + TK_REDO);
-        }
+        if (k <= STREAM_TOPK_MAX_K && coop_select_ok())
+            return launch_topk_coop(r, *mat, c, key, k, (u32 *)w, w + topk_stream_offset(k), idx_out, key_out, count_out, st);
         return run_topk_scan(src, r, k, negate, SEL_MAX_BLOCKS, w, idx_out, key_out, count_out, st);
     }
     TileGeom g;
@@ -1124,12 +1119,10 @@ int launch_pareto(const DSpace &s, Range r, const guide_outputs *mat, int time_m
                   unsigned *ticket, cudaStream_t st) {
     if (mat) {
         MatSource src{*mat, make_cons(c), xm, ym, mat_vec_ok(*mat)};
-        if (stream_eligible(*mat, r)) {
-            // streaming path, then the general kernel gated on the redo flag (header word 1)
-            GUIDE_CUDA(cudaMemsetAsync(ws, 0, 256, st));
-            u32 *header = (u32 *)ws;
-            int rc = launch_pareto_stream(r, *mat, c, xm, ym, header, (unsigned char *)ws + pareto_stream_offset(), idx_out, cap,
-                                          count_out, st);
+        if (coop_select_ok()) {
+            // one launch, then the general kernel gated on the redo flag (header word 1)
+            int rc = launch_pareto_coop(r, *mat, c, xm, ym, (u32 *)ws, (unsigned char *)ws + pareto_stream_offset(), idx_out, cap,
+                                        count_out, st);
             if (rc) return rc;
             return run_pareto_general(src, r, idx_out, cap, count_out, ws, st);
         }

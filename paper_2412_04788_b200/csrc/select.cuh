@@ -135,22 +135,25 @@ inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 bl
 enum { TK_TICKET = 2, TK_COUNT = 3, TK_REDO = 4, TK_SAMPLED = 5, TK_BOUND = 6, TK_TICKET2 = 10 };
 enum { PH_TICKET = 4, PH_COUNT = 5, PH_KILLERS = 6, PH_FRONT = 7, PH_TICKET2 = 8 };
 
-// ---- streaming path (select_stream.cu) -----------------------------------------------------------
-// Materialised metrics only.  A strided sample gives a bound (top-k) or a small set of dominating
-// points (Pareto); one pass at memory speed then keeps the few configs the bound cannot exclude and
-// a last small kernel finishes exactly.  When the survivors do not fit the workspace the redo flag
-// goes up and the accumulator-based kernels, queued behind and gated on that flag, redo the call.
+// ---- one-launch path over materialised metrics (select_coop.cu) ------------------------------------
+// A sample gives a bound (top-k) or a small set of dominating points (Pareto); one pass then keeps the
+// few configs those cannot exclude and a last step finishes exactly.
+static constexpr u32 STREAM_TOPK_MAX_K = 128;            // larger k goes to the accumulator kernels
+bool coop_select_ok();
+size_t topk_coop_bytes();
+size_t pareto_coop_bytes();
+int launch_topk_coop(Range r, const guide_outputs &mat, const guide_constraints &c, int key, u32 k, u32 *header,
+                     unsigned char *region, u64 *idx_out, double *key_out, u32 *count_out, cudaStream_t st);
+// raises header word 1 when the survivors do not fit its list: the general kernel queued behind is gated on it
+int launch_pareto_coop(Range r, const guide_outputs &mat, const guide_constraints &c, int xm, int ym, u32 *header,
+                       unsigned char *region, u64 *idx_out, u32 cap, u32 *count_out, cudaStream_t st);
+
+// ---- streaming path of the fused selection (select_stream.cu) --------------------------------------
+// A survivor list that overflows raises the redo flag, and the accumulator-based kernels, queued behind
+// and gated on that flag, redo the call.
 static constexpr u64 STREAM_MIN_COUNT = 1ull << 18;      // below this the accumulator kernels are as fast
-static constexpr u32 STREAM_TOPK_MAX_K = 128;
 size_t topk_stream_bytes();
 size_t pareto_stream_bytes();
-bool stream_eligible(const guide_outputs &mat, Range r);
-// Both leave *redo_flag pointing at the device word the fallback kernels must be gated on.
-int launch_topk_stream(Range r, const guide_outputs &mat, const guide_constraints &c, int key, u32 k, u32 *header,
-                       unsigned char *region, u64 *idx_out, double *key_out, u32 *count_out, cudaStream_t st);
-int launch_pareto_stream(Range r, const guide_outputs &mat, const guide_constraints &c, int xm, int ym, u32 *header,
-                         unsigned char *region, u64 *idx_out, u32 cap, u32 *count_out, cudaStream_t st);
-
 
 // Fused form (nothing materialised, whole closed-form spaces): the sample rows are evaluated into a
 // compact scratch in the workspace, the same bound / killer kernels run on that, and the filter pass

@@ -1,0 +1,924 @@
+// Selection over materialised metrics in one launch (constraint filter + top-k / Pareto front of
+// Sec. 3.2 / Sec. 4.1 on arrays written by guide_simulate).
+//
+// A selection keeps a handful of configs out of many, so what bounds it is a chain of latencies, not
+// bandwidth: on a million configs the arrays are read in 3 us, and everything else is steps that wait
+// for one another.  The steps are therefore parts of one cooperative kernel with grid barriers
+// between them instead of five launches:
+//
+//   sample : rows of 64 consecutive configs, one out of every r at a hashed position (r = 1: all of
+//            them), at most four per warp.  Their keys stay in registers.
+//   bound  : top-k: the smallest pair of every group of warps goes to the workspace; after a barrier
+//            every block works out for itself a pair that at least k of those are within (one
+//            histogram of the encoded keys).  With r > 1 the sample pairs within it are gathered and
+//            give, in the same way, a bound close to the sample's own k-th pair.  Pareto: the extreme
+//            points of eight directions, over the lane, the warp, the block and, after a barrier, all
+//            blocks ("killers").
+//   filter : a config survives if it passes the constraints and its pair is within the bound, or no
+//            killer strictly dominates it.  With r = 1 the values are still in registers, otherwise
+//            one pass over the arrays.  Survivors go to a list in the workspace.
+//   finish : the (few) survivors are ranked and the answer is written, by one block unless a front has
+//            many of them.
+//
+// Bound and killers only exclude configs that cannot be part of the answer, whatever the sample
+// looked like.  If the top-k list overflows, the bound of what it holds excludes more, and the filter
+// runs again; a Pareto list that overflows raises the redo flag and the accumulator kernel queued
+// behind (select.cu) redoes the call.
+//
+// Ranges of up to 2048 configs are one block: its barriers are block barriers and nothing goes
+// through the workspace.
+//
+// Top-k + front after a sweep on a B200, against chains of kernels (sample, refined bound, filter, rank,
+// gated fallback): 983,040 configs 14 + 21 us instead of 38 + 39; 504 configs 7 + 8 us instead of 14 + 19;
+// 16.8 M configs (one row of 14 sampled) 60 + 65 us instead of 65 + 78.
+#include <algorithm>
+#include <cmath>
+#include <cstdlib>
+
+#include <cooperative_groups.h>
+
+#include "select_src.cuh"
+
+namespace guide {
+
+static constexpr u32 CO_THREADS = 512, CO_WARPS = CO_THREADS / 32;
+static constexpr u32 CO_BLOCKS_PER_SM = 2;      // 64 registers: 32 warps per SM, and few enough blocks for a quick grid barrier
+static constexpr u32 CO_ROWS = 4;               // sample rows a warp keeps in registers
+static constexpr u32 CO_ONE_BLOCK_ROWS = 32;    // ranges up to this many rows are one block; its survivors stay in shared memory
+static constexpr u32 CO_BOUND_LIST = 1024;      // most pairs a bound is worked out from: group minima, sample pairs within the coarse bound
+static constexpr u32 CO_LIST = 2560;            // pairs the finishing block holds in shared memory (five per thread)
+static constexpr u32 CO_BINS = 2 * CO_THREADS;  // bins of a histogram
+static constexpr u32 CO_RANKED = 256;           // pairs the finishing block ranks by counting (at least two threads each)
+static constexpr u32 CO_DIRS = 8;               // killers of a Pareto call
+static constexpr u32 CO_P_DIRECT = 128;         // survivors one block compares all against all
+static constexpr u32 CO_P_CHUNK = 1024;         // survivors staged in shared memory at a time
+static constexpr u32 CO_MAX_BLOCKS = 512;       // workspace for the blocks' killer candidates
+static_assert(CO_ONE_BLOCK_ROWS * ROW <= CO_LIST && CO_LIST % CO_THREADS == 0, "one block's whole range fits its list");
+
+template <int NA>
+struct CoopSrc {
+    Arr a[NA];        // entry 0 is the key (top-k) or x (Pareto), entry 1 is y (Pareto only)
+    const uint8_t *status;
+    int vec;          // every array is 16-byte aligned (status: 2-byte)
+};
+
+// The sample: groups of r consecutive rows, one row of each, at a hashed offset so that it does not
+// lock onto a period of the config index.
+struct Walk {
+    u64 n_rows, n_slots;
+    u32 r;
+    __device__ __forceinline__ u64 row(u64 slot) const {
+        if (r == 1) return slot;
+        const u32 h = ((u32)slot * 2654435761u) >> 7;
+        return slot * r + h % r;
+    }
+};
+
+// status and values of this lane's two configs of a row; outside the range: status 0xFF
+template <int NA>
+__device__ __forceinline__ void load_row(const CoopSrc<NA> &s, u64 count, u64 row, bool live, u32 lane, u32 &st, double2 (&v)[NA]) {
+    const u64 j = row * ROW + 2 * lane;
+    if (live && s.vec && (row + 1) * ROW <= count) {
+        st = __ldcg(reinterpret_cast<const unsigned short *>(s.status + j));
+#pragma unroll
+        for (int a = 0; a < NA; a++) v[a] = __ldcg(reinterpret_cast<const double2 *>(s.a[a].p + j));
+    } else {
+        const bool in0 = live && j < count, in1 = live && j + 1 < count;
+        st = (in0 ? (u32)s.status[j] : 0xFFu) | ((in1 ? (u32)s.status[j + 1] : 0xFFu) << 8);
+#pragma unroll
+        for (int a = 0; a < NA; a++) {
+            v[a].x = in0 ? s.a[a].p[j] : 0.0;
+            v[a].y = in1 ? s.a[a].p[j + 1] : 0.0;
+        }
+    }
+}
+
+template <int NA>
+__device__ __forceinline__ void row_ok(const CoopSrc<NA> &s, u32 st, const double2 (&v)[NA], bool &ok0, bool &ok1) {
+    ok0 = (st & 0xFFu) == 0;
+    ok1 = (st >> 8) == 0;
+#pragma unroll
+    for (int a = 0; a < NA; a++) {
+        ok0 &= within(s.a[a], v[a].x);
+        ok1 &= within(s.a[a], v[a].y);
+    }
+}
+
+// A pass over everything, in chunks of CO_ROWS rows taken in turn by all warps, from the end of the range
+// backwards (when the metrics were written just before this call the end of the arrays is what the L2
+// still holds).  Neighbouring chunks go to different blocks, and a warp takes a different place in every
+// round: rows that fit come in runs, and a fixed place would share its position modulo the batch and TP
+// axes, whose lengths are powers of two as the number of warps nearly is.
+struct FilterWalk {
+    u64 n_rows, stride, base;
+    u32 pos;
+    __device__ __forceinline__ FilterWalk(u64 rows, u64 warps, u32 first) : n_rows(rows), stride(warps), base(0), pos(first) {}
+    // row u of the current chunk; past the end of the walk: a huge number
+    __device__ __forceinline__ u64 row(u32 u) const { return n_rows - 1 - ((base + pos) * CO_ROWS + u); }
+    __device__ __forceinline__ bool more() const { return base * CO_ROWS < n_rows; }
+    __device__ __forceinline__ void next() { base += stride; pos = (pos + 37u) % (u32)stride; }
+};
+
+// The status bytes of a chunk come first (asked for a round ahead); a row's values are loaded only if
+// some config of it passed its memory check, which most rows of a large sweep do not.
+template <int NA>
+__device__ __forceinline__ void load_chunk_status(const CoopSrc<NA> &s, u64 count, const FilterWalk &fw, u32 lane, u32 (&st)[CO_ROWS]) {
+#pragma unroll
+    for (u32 u = 0; u < CO_ROWS; u++) {
+        const u64 row = fw.row(u), j = row * ROW + 2 * lane;
+        st[u] = 0xFFFFu;
+        if (row < fw.n_rows) {
+            if (s.vec && (row + 1) * ROW <= count) st[u] = __ldcs(reinterpret_cast<const unsigned short *>(s.status + j));
+            else st[u] = (j < count ? (u32)s.status[j] : 0xFFu) | ((j + 1 < count ? (u32)s.status[j + 1] : 0xFFu) << 8);
+        }
+    }
+}
+// returns false when no row of the chunk has a config to look at
+template <int NA>
+__device__ __forceinline__ bool load_chunk_values(const CoopSrc<NA> &s, u64 count, const FilterWalk &fw, u32 lane,
+                                                  const u32 (&st)[CO_ROWS], double2 (&v)[CO_ROWS][NA]) {
+    u32 any = 0;
+#pragma unroll
+    for (u32 u = 0; u < CO_ROWS; u++)
+        if (__any_sync(0xFFFFFFFFu, (st[u] & 0xFFu) == 0 || (st[u] >> 8) == 0)) any |= 1u << u;
+    if (any == 0) return false;
+#pragma unroll
+    for (u32 u = 0; u < CO_ROWS; u++) {
+        const u64 row = fw.row(u), j = row * ROW + 2 * lane;
+#pragma unroll
+        for (int a = 0; a < NA; a++) {
+            v[u][a] = make_double2(0.0, 0.0);
+            if ((any >> u) & 1u) {
+                if (s.vec && (row + 1) * ROW <= count) v[u][a] = __ldcs(reinterpret_cast<const double2 *>(s.a[a].p + j));
+                else {
+                    if (j < count) v[u][a].x = s.a[a].p[j];
+                    if (j + 1 < count) v[u][a].y = s.a[a].p[j + 1];
+                }
+            }
+        }
+    }
+    return true;
+}
+
+__device__ __forceinline__ void grid_barrier() {
+    if (gridDim.x == 1) __syncthreads();
+    else cooperative_groups::this_grid().sync();
+}
+
+// ---- block-wide counting --------------------------------------------------------------------------
+
+struct CountScratch {
+    u32 part[2][CO_WARPS];
+    u64 lo[CO_WARPS], hi[CO_WARPS];
+};
+
+// Sum over the block.  Two buffers in turn: one barrier per call is enough.
+__device__ __forceinline__ u32 block_sum(u32 v, u32 (*part)[CO_WARPS], u32 &phase) {
+    const u32 lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    v = __reduce_add_sync(0xFFFFFFFFu, v);
+    if (lane == 0) part[phase][warp] = v;
+    __syncthreads();
+    const u32 t = lane < CO_WARPS ? part[phase][lane] : 0u;
+    phase ^= 1;
+    return __reduce_add_sync(0xFFFFFFFFu, t);
+}
+
+__device__ __forceinline__ void block_min_max(u64 &lo, u64 &hi, u64 *slo, u64 *shi) {
+    const u32 lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int d = 16; d > 0; d >>= 1) {
+        const u64 ol = __shfl_xor_sync(0xFFFFFFFFu, lo, d), oh = __shfl_xor_sync(0xFFFFFFFFu, hi, d);
+        lo = ol < lo ? ol : lo; hi = oh > hi ? oh : hi;
+    }
+    __syncthreads();                                   // earlier readers of the scratch are done
+    if (lane == 0) { slo[warp] = lo; shi[warp] = hi; }
+    __syncthreads();
+    for (u32 w = 0; w < CO_WARPS; w++) { lo = slo[w] < lo ? slo[w] : lo; hi = shi[w] > hi ? shi[w] : hi; }
+}
+
+// A pair (bkey, bidx) that at least k and, ties or not, at most k + slack of the block's pairs are
+// within (the total order is (key, index); indices are distinct).  A bisection on the encoded key,
+// then, if one key is shared by too many, on the index; it stops as soon as the count is in the
+// window.  Entries with an all-ones index are padding.  All-ones when there are fewer than k pairs.
+// Collective; every thread gets the result.
+template <u32 PER>
+__device__ __noinline__ void kth_bound(const u64 (&key)[PER], const u64 (&idx)[PER], u32 k, u32 slack, CountScratch &sc, u64 &bkey,
+                                       u64 &bidx) {
+    u32 phase = 0;
+    __syncthreads();                                   // the scratch is free
+    u32 n = 0;
+    u64 lo = KEY_MAX, hi = 0;
+#pragma unroll
+    for (u32 u = 0; u < PER; u++)
+        if (idx[u] != KEY_MAX) { n++; lo = key[u] < lo ? key[u] : lo; hi = key[u] > hi ? key[u] : hi; }
+    bkey = KEY_MAX; bidx = KEY_MAX;
+    if (block_sum(n, sc.part, phase) < k) return;
+    block_min_max(lo, hi, sc.lo, sc.hi);
+    while (lo < hi) {
+        const u64 mid = lo + ((hi - lo) >> 1);
+        u32 c = 0;
+#pragma unroll
+        for (u32 u = 0; u < PER; u++) c += (idx[u] != KEY_MAX && key[u] <= mid) ? 1u : 0u;
+        c = block_sum(c, sc.part, phase);
+        if (c < k) { lo = mid + 1; continue; }
+        hi = mid;
+        if (c <= k + slack) { bkey = hi; return; }
+    }
+    bkey = hi;                                         // the k-th key itself; maybe many share it
+    u32 c = 0;
+    u64 ilo = KEY_MAX, ihi = 0;
+#pragma unroll
+    for (u32 u = 0; u < PER; u++) {
+        if (idx[u] == KEY_MAX) continue;
+        c += key[u] <= bkey ? 1u : 0u;
+        if (key[u] == bkey) { ilo = idx[u] < ilo ? idx[u] : ilo; ihi = idx[u] > ihi ? idx[u] : ihi; }
+    }
+    if (block_sum(c, sc.part, phase) <= k + slack) return;
+    block_min_max(ilo, ihi, sc.lo, sc.hi);
+    while (ilo < ihi) {
+        const u64 mid = ilo + ((ihi - ilo) >> 1);
+        c = 0;
+#pragma unroll
+        for (u32 u = 0; u < PER; u++) c += (idx[u] != KEY_MAX && pair_le(key[u], idx[u], bkey, mid)) ? 1u : 0u;
+        c = block_sum(c, sc.part, phase);
+        if (c < k) { ilo = mid + 1; continue; }
+        ihi = mid;
+        if (c <= k + slack) break;
+    }
+    bidx = ihi;
+}
+
+// The same from one histogram of the keys' high halves, which as a rule decides: four barriers instead
+// of one per round.  Where the bin of the k-th pair takes the count above k + slack (many keys
+// share it) the bisection follows.  All-ones when there are fewer than k pairs.
+template <u32 PER>
+__device__ __forceinline__ void histogram_bound(const u64 (&key)[PER], const u64 (&idx)[PER], u32 k, u32 slack, u32 *bins, CountScratch &sc,
+                                                u64 &bkey, u64 &bidx) {
+    const u32 lane = threadIdx.x & 31, warp = threadIdx.x >> 5, FULL = 0xFFFFFFFFu;
+    __syncthreads();                                   // the scratch is free
+    u32 lo = FULL, hi = 0;
+#pragma unroll
+    for (u32 u = 0; u < PER; u++)
+        if (idx[u] != KEY_MAX) { const u32 h = (u32)(key[u] >> 32); lo = min(lo, h); hi = max(hi, h); }
+    lo = __reduce_min_sync(FULL, lo); hi = __reduce_max_sync(FULL, hi);
+    if (lane == 0) { sc.part[0][warp] = lo; sc.part[1][warp] = hi; }
+    for (u32 i = threadIdx.x; i < CO_BINS; i += CO_THREADS) bins[i] = 0;
+    if (threadIdx.x == 0) { sc.lo[0] = KEY_MAX; sc.hi[0] = 0; }
+    __syncthreads();
+    lo = __reduce_min_sync(FULL, sc.part[0][lane % CO_WARPS]); hi = __reduce_max_sync(FULL, sc.part[1][lane % CO_WARPS]);
+    const u32 range = hi >= lo ? hi - lo : 0, width = 32 - __clz(range | 1u), shift = width > 10 ? width - 10 : 0;   // range >> shift < 1024
+    static_assert(CO_BINS == 1024, "ten bits of the range");
+#pragma unroll
+    for (u32 u = 0; u < PER; u++)
+        if (idx[u] != KEY_MAX) atomicAdd(&bins[((u32)(key[u] >> 32) - lo) >> shift], 1u);
+    __syncthreads();
+    const u32 b0 = bins[2 * threadIdx.x], b1 = bins[2 * threadIdx.x + 1];
+    u32 incl = b0 + b1;
+    for (u32 d = 1; d < 32; d <<= 1) {
+        const u32 o = __shfl_up_sync(FULL, incl, d);
+        if (lane >= d) incl += o;
+    }
+    if (lane == 31) sc.part[0][warp] = incl;
+    __syncthreads();
+    u32 off = 0;
+    for (u32 w = 0; w < warp; w++) off += sc.part[0][w];
+    incl += off;
+    const u32 before = incl - b0 - b1;
+    if (before < k && incl >= k) {                     // one thread: the k-th pair is in one of its two bins
+        const bool first = before + b0 >= k;
+        const u64 end = (u64)lo + ((u64)(2 * threadIdx.x + (first ? 1 : 2)) << shift);
+        sc.lo[0] = end > FULL ? KEY_MAX : (end << 32) - 1;
+        sc.hi[0] = first ? before + b0 : incl;
+    }
+    __syncthreads();
+    bkey = sc.lo[0]; bidx = KEY_MAX;
+    const u32 c = (u32)sc.hi[0];
+    if (c > k + slack) kth_bound<PER>(key, idx, k, slack, sc, bkey, bidx);
+}
+
+// ... of n pairs of a list in the workspace (of PER per thread spread over it, if it is longer)
+template <u32 PER>
+__device__ __forceinline__ void list_bound(const KI *list, u32 n, u32 k, u32 *bins, CountScratch &sc, u64 &bkey, u64 &bidx) {
+    constexpr u32 MOST = PER * CO_THREADS;
+    const u32 step = n > MOST ? n / MOST : 1;
+    u64 key[PER], idx[PER];
+#pragma unroll
+    for (u32 u = 0; u < PER; u++) {
+        const u32 i = threadIdx.x + u * CO_THREADS;
+        ulonglong2 e; e.x = KEY_MAX; e.y = KEY_MAX;
+        if (i < min(n, MOST)) e = __ldcg(reinterpret_cast<const ulonglong2 *>(list + (size_t)i * step));
+        key[u] = e.x; idx[u] = e.y;
+    }
+    histogram_bound<PER>(key, idx, k, k + 8, bins, sc, bkey, bidx);
+}
+
+// the takers of a warp append to a list through one atomic; entries beyond cap are counted, not stored
+template <class T>
+__device__ __forceinline__ void warp_append(bool take, const T &e, u32 *counter, T *list, u32 cap) {
+    const u32 ballot = __ballot_sync(0xFFFFFFFFu, take);
+    if (!ballot) return;
+    const u32 lane = threadIdx.x & 31;
+    u32 base = 0;
+    if (lane == 0) base = atomicAdd(counter, __popc(ballot));
+    base = __shfl_sync(0xFFFFFFFFu, base, 0);
+    const u32 pos = base + __popc(ballot & ((1u << lane) - 1));
+    if (take && pos < cap) list[pos] = e;
+}
+
+// ---- top-k -------------------------------------------------------------------------------------------
+
+struct FinishScratch {
+    KI sl[CO_LIST];
+    u32 bins[CO_BINS];
+    u32 n;
+};
+
+// One block: the k smallest of n pairs, in order; of the list in the workspace, or (cand null) already in f.sl.
+__device__ __noinline__ void topk_finish(const KI *cand, u32 n, u32 k, FinishScratch &f, CountScratch &sc, int negate, u64 *idx_out,
+                                         double *key_out, u32 *count_out) {
+    constexpr u32 PER = CO_LIST / CO_THREADS;
+    const u32 found = min(n, k);
+    if (threadIdx.x == 0) *count_out = found;
+    for (u32 i = found + threadIdx.x; i < k; i += CO_THREADS) {
+        idx_out[i] = KEY_MAX;
+        key_out[i] = __longlong_as_double(0x7FF0000000000000LL);
+    }
+    if (n == 0) return;
+    u32 c = n;
+    u64 bkey = KEY_MAX, bidx = KEY_MAX;
+    if (cand && n <= CO_LIST) {
+        for (u32 i = threadIdx.x; i < n; i += CO_THREADS) {
+            const ulonglong2 w = __ldcg(reinterpret_cast<const ulonglong2 *>(cand + i));
+            f.sl[i].key = w.x; f.sl[i].idx = w.y;
+        }
+        __syncthreads();
+    }
+    // down to CO_RANKED pairs: those within a bound of what shared memory holds.  A list that does not fit
+    // it is gone through again with that bound, which leaves out most of what was looked at.
+    while (c > CO_RANKED) {
+        if (c > CO_LIST) {
+            __syncthreads();
+            if (threadIdx.x == 0) f.n = 0;
+            __syncthreads();
+            for (u32 i0 = 0; i0 < n; i0 += CO_THREADS) {
+                const u32 i = i0 + threadIdx.x;
+                KI e; e.key = KEY_MAX; e.idx = KEY_MAX;
+                if (i < n) {
+                    const ulonglong2 w = __ldcg(reinterpret_cast<const ulonglong2 *>(cand + i));
+                    e.key = w.x; e.idx = w.y;
+                }
+                warp_append(i < n && pair_le(e.key, e.idx, bkey, bidx), e, &f.n, f.sl, CO_LIST);
+            }
+            __syncthreads();
+            c = f.n;
+            if (c <= CO_RANKED) break;
+        }
+        u64 key[PER], idx[PER];
+#pragma unroll
+        for (u32 u = 0; u < PER; u++) {
+            const u32 i = threadIdx.x + u * CO_THREADS;
+            key[u] = KEY_MAX; idx[u] = KEY_MAX;
+            if (i < min(c, CO_LIST)) { key[u] = f.sl[i].key; idx[u] = f.sl[i].idx; }
+        }
+        histogram_bound<PER>(key, idx, found, CO_RANKED - found, f.bins, sc, bkey, bidx);
+        if (c > CO_LIST) continue;
+        __syncthreads();
+        if (threadIdx.x == 0) f.n = 0;
+        __syncthreads();
+#pragma unroll
+        for (u32 u = 0; u < PER; u++) {
+            KI e; e.key = key[u]; e.idx = idx[u];
+            warp_append(idx[u] != KEY_MAX && pair_le(key[u], idx[u], bkey, bidx), e, &f.n, f.sl, CO_LIST);
+        }
+        __syncthreads();
+        c = f.n;
+    }
+    // rank by counting: a power of two of threads per pair shares out the comparisons
+    u32 tpe = 32;
+    while (tpe * c > CO_THREADS) tpe >>= 1;            // c <= CO_RANKED: at least two
+    const u32 me_i = threadIdx.x / tpe, part = threadIdx.x % tpe;
+    const KI me = f.sl[min(me_i, c - 1)];
+    u32 ahead = 0;
+    for (u32 q = part; q < c; q += tpe) ahead += ki_less(f.sl[q], me) ? 1u : 0u;
+    for (u32 d = tpe >> 1; d > 0; d >>= 1) ahead += __shfl_xor_sync(0xFFFFFFFFu, ahead, d);
+    if (part == 0 && me_i < c && ahead < k) {
+        const double v = dec(me.key);
+        idx_out[ahead] = me.idx;
+        key_out[ahead] = negate ? 0.0 - v : v;
+    }
+}
+
+template <int NA>
+__global__ void __launch_bounds__(CO_THREADS, CO_BLOCKS_PER_SM)
+k_topk_coop(CoopSrc<NA> s, Range r, Walk w, u32 k, u32 group_log2, u32 *header, KI *minima, KI *spairs, KI *cand, int negate,
+            u64 *idx_out, double *key_out, u32 *count_out) {
+    __shared__ FinishScratch fin;
+    __shared__ CountScratch sc;
+    KI *sl = fin.sl;
+    grid_dep_wait();
+    const u32 lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // nothing reads the header before the first barrier
+    if (blockIdx.x == 0 && threadIdx.x < 64) header[threadIdx.x] = 0;
+    // ---- sample: this warp's rows; the groups of 2^group_log2 warps take rows far apart ----
+    const u32 n_groups = (gridDim.x * CO_WARPS) >> group_log2;
+    const u32 group = (blockIdx.x * CO_WARPS + warp) >> group_log2, member = warp & ((1u << group_log2) - 1);
+    u64 key[2 * CO_ROWS];
+    u32 ok = 0;
+    {
+        u32 st[CO_ROWS];
+        double2 v[CO_ROWS][NA];
+#pragma unroll
+        for (u32 u = 0; u < CO_ROWS; u++) {
+            const u64 slot = (u64)((u << group_log2) + member) * n_groups + group;
+            load_row(s, r.count, w.row(slot), slot < w.n_slots, lane, st[u], v[u]);
+        }
+#pragma unroll
+        for (u32 u = 0; u < CO_ROWS; u++) {
+            bool ok0, ok1;
+            row_ok(s, st[u], v[u], ok0, ok1);
+            key[2 * u] = metric_key(s.a[0], v[u][0].x);
+            key[2 * u + 1] = metric_key(s.a[0], v[u][0].y);
+            ok |= (ok0 ? 1u : 0u) << (2 * u) | (ok1 ? 1u : 0u) << (2 * u + 1);
+        }
+    }
+    auto index_of = [&](u32 i) {                       // config index of sample value i of this lane
+        const u64 slot = (u64)(((i >> 1) << group_log2) + member) * n_groups + group;
+        return r.first + w.row(slot) * ROW + 2 * lane + (i & 1);
+    };
+    // ---- one block: what passes is ranked where it is ----
+    if (gridDim.x == 1) {
+        if (threadIdx.x == 0) fin.n = 0;
+        __syncthreads();
+#pragma unroll
+        for (u32 i = 0; i < 2 * CO_ROWS; i++) {
+            KI e; e.key = key[i]; e.idx = index_of(i);
+            warp_append(((ok >> i) & 1u) != 0, e, &fin.n, sl, CO_LIST);
+        }
+        __syncthreads();
+        const u32 n = fin.n;
+        __syncthreads();
+        topk_finish(nullptr, n, k, fin, sc, negate, idx_out, key_out, count_out);
+        return;
+    }
+    // ---- coarse bound: the smallest pair of every group, then a pair k of them are within ----
+    {
+        u64 bk = KEY_MAX, bi = KEY_MAX;
+#pragma unroll
+        for (u32 i = 0; i < 2 * CO_ROWS; i++)
+            if ((ok >> i) & 1u) pair_min(bk, bi, key[i], index_of(i));
+        for (int d = 16; d > 0; d >>= 1)
+            pair_min(bk, bi, __shfl_xor_sync(0xFFFFFFFFu, bk, d), __shfl_xor_sync(0xFFFFFFFFu, bi, d));
+        if (lane == 0) { sl[warp].key = bk; sl[warp].idx = bi; }
+        __syncthreads();
+        if (threadIdx.x < (CO_WARPS >> group_log2)) {
+            const KI *mine = sl + (threadIdx.x << group_log2);
+            bk = mine[0].key; bi = mine[0].idx;
+            for (u32 q = 1; q < (1u << group_log2); q++) pair_min(bk, bi, mine[q].key, mine[q].idx);
+            ulonglong2 m; m.x = bk; m.y = bi;
+            *reinterpret_cast<ulonglong2 *>(minima + ((blockIdx.x * CO_WARPS) >> group_log2) + threadIdx.x) = m;
+        }
+    }
+    grid_barrier();
+    u64 bkey, bidx;
+    list_bound<CO_BOUND_LIST / CO_THREADS>(minima, n_groups, k, fin.bins, sc, bkey, bidx);
+    // ---- the sample values within it: the survivors themselves, or (r > 1) the pairs of a closer bound ----
+    const bool whole = w.r == 1;
+    u32 *count = header + TK_COUNT;
+#pragma unroll
+    for (u32 i = 0; i < 2 * CO_ROWS; i++) {
+        KI e; e.key = key[i]; e.idx = index_of(i);
+        const bool take = ((ok >> i) & 1u) && pair_le(e.key, e.idx, bkey, bidx);
+        if (whole) warp_append(take, e, count, cand, TK_CAND_CAP);
+        else warp_append(take, e, header + TK_SAMPLED, spairs, CO_BOUND_LIST);
+    }
+    grid_barrier();
+    if (!whole) {
+        // of more pairs than the list holds the stored ones still give a valid bound; fewer than k only
+        // when the coarse bound is all-ones, which then stays
+        const u32 ns = min(__ldcg(header + TK_SAMPLED), CO_BOUND_LIST);
+        if (ns >= k) list_bound<CO_BOUND_LIST / CO_THREADS>(spairs, ns, k, fin.bins, sc, bkey, bidx);
+    }
+    // ---- filter passes over everything: none when the sample was everything and its survivors fit ----
+    for (bool first_pass = !whole;; first_pass = false) {
+        if (!first_pass) {
+            const u32 n = __ldcg(count);
+            if (n <= TK_CAND_CAP) {
+                if (blockIdx.x == 0) topk_finish(cand, n, k, fin, sc, negate, idx_out, key_out, count_out);
+                return;
+            }
+            // the list overflowed: k pairs of what it holds are within a bound that excludes more
+            list_bound<CO_BOUND_LIST / CO_THREADS>(cand, TK_CAND_CAP, k, fin.bins, sc, bkey, bidx);
+            u32 *next = count == header + TK_COUNT ? header + TK_TICKET : header + TK_COUNT;   // last read two barriers ago
+            if (blockIdx.x == 0 && threadIdx.x == 0) *next = 0;
+            count = next;
+            grid_barrier();
+        }
+        const u64 stride = (u64)gridDim.x * CO_WARPS;
+        FilterWalk fw(w.n_rows, stride, warp * gridDim.x + blockIdx.x), ahead = fw;
+        u32 st[CO_ROWS], st_ahead[CO_ROWS];
+        load_chunk_status(s, r.count, ahead, lane, st_ahead);
+        for (; fw.more(); fw = ahead) {
+#pragma unroll
+            for (u32 u = 0; u < CO_ROWS; u++) st[u] = st_ahead[u];
+            ahead.next();
+            load_chunk_status(s, r.count, ahead, lane, st_ahead);
+            double2 v[CO_ROWS][NA];
+            if (!load_chunk_values(s, r.count, fw, lane, st, v)) continue;
+#pragma unroll
+            for (u32 u = 0; u < CO_ROWS; u++) {
+                bool ok0, ok1;
+                row_ok(s, st[u], v[u], ok0, ok1);
+                const u64 k0 = metric_key(s.a[0], v[u][0].x), k1 = metric_key(s.a[0], v[u][0].y);
+                ok0 = ok0 && k0 <= bkey; ok1 = ok1 && k1 <= bkey;
+                if (!__any_sync(0xFFFFFFFFu, ok0 | ok1)) continue;     // the usual case
+                KI e0, e1;
+                e0.key = k0; e0.idx = r.first + fw.row(u) * ROW + 2 * lane;
+                e1.key = k1; e1.idx = e0.idx + 1;
+                warp_append(ok0 && pair_le(e0.key, e0.idx, bkey, bidx), e0, count, cand, TK_CAND_CAP);
+                warp_append(ok1 && pair_le(e1.key, e1.idx, bkey, bidx), e1, count, cand, TK_CAND_CAP);
+            }
+        }
+        grid_barrier();
+    }
+}
+
+// ---- Pareto ------------------------------------------------------------------------------------------
+
+// The killers are the extreme points of a few directions: of the points seen, the one that minimises a
+// weighted sum of the two encoded metrics (their high halves: about the logarithms).  Every one is a
+// real point, so whatever it strictly dominates is out.  No direction is an axis: the other metric
+// decides between points that share the best value of one, as they do where it has few values.
+__device__ __forceinline__ u32 direction_weight(u32 d) { return d == 0 ? 31u : d == CO_DIRS - 1 ? 1u : 30u - 4u * d; }
+static_assert(CO_DIRS == 8, "weights 31, 26, 22, 18, 14, 10, 6, 1 of 32");
+// a missing point (all-ones twice) has the largest score there is
+__device__ __forceinline__ u32 direction_score(u64 x, u64 y, u32 w) { return (u32)(x >> 37) * w + (u32)(y >> 37) * (32u - w); }
+
+// is this the lane with the smallest score of the warp?
+__device__ __forceinline__ bool warp_best(u32 score) {
+    const u32 s = __reduce_min_sync(0xFFFFFFFFu, score);
+    return (threadIdx.x & 31) == (u32)__ffs(__ballot_sync(0xFFFFFFFFu, score == s)) - 1;
+}
+
+struct Killers8 {
+    const P2 *k;
+    // strictly dominated by one of them?  The high halves decide nearly always.
+    __device__ __forceinline__ bool kills(u64 x, u64 y) const {
+        const u32 X = (u32)(x >> 32), Y = (u32)(y >> 32);
+        bool dead = false;
+#pragma unroll
+        for (u32 q = 0; q < CO_DIRS; q++) dead |= (u32)(k[q].x >> 32) < X && (u32)(k[q].y >> 32) < Y;
+        if (dead) return true;
+#pragma unroll 1
+        for (u32 q = 0; q < CO_DIRS; q++) dead |= dominates(k[q].x, k[q].y, x, y);
+        return dead;
+    }
+};
+
+// One block: the front of n points, by all-against-all comparison shared out over the threads, in
+// ascending x (the x of a front are distinct).  flags: n bytes.
+__device__ __noinline__ void pareto_small(const P3 *sv, u32 n, unsigned char *flags, u32 lim, u64 *idx_out, u32 *count_out) {
+    u32 tpe = 32;
+    while (tpe > 1 && tpe * n > CO_THREADS) tpe >>= 1;
+    const u32 part = threadIdx.x % tpe, per_round = CO_THREADS / tpe;
+    for (u32 g0 = 0; g0 < n; g0 += per_round) {
+        const u32 g = g0 + threadIdx.x / tpe;
+        const P3 me = sv[min(g, n - 1)];
+        u32 out = 0;
+        for (u32 q = part; q < n; q += tpe) {
+            const P3 o = sv[q];
+            out |= dominates(o.x, o.y, me.x, me.y) || (o.x == me.x && o.y == me.y && o.idx < me.idx) ? 1u : 0u;
+        }
+        for (u32 d = tpe >> 1; d > 0; d >>= 1) out |= __shfl_xor_sync(0xFFFFFFFFu, out, d);
+        if (part == 0 && g < n) flags[g] = out ? 0 : 1;
+    }
+    __syncthreads();
+    for (u32 g = threadIdx.x; g < n; g += CO_THREADS) {
+        if (!flags[g]) continue;
+        u32 ahead = 0;
+        for (u32 q = 0; q < n; q++) ahead += flags[q] && sv[q].x < sv[g].x ? 1u : 0u;
+        if (ahead < lim) idx_out[ahead] = sv[g].idx;
+    }
+    u32 total = 0;
+    for (u32 g0 = 0; g0 < n; g0 += CO_THREADS) total += __syncthreads_count(g0 + threadIdx.x < n && flags[g0 + threadIdx.x]);
+    if (threadIdx.x == 0) *count_out = total > GUIDE_PARETO_MAX ? 0xFFFFFFFFu : total;
+}
+
+template <int NA>
+__global__ void __launch_bounds__(CO_THREADS, CO_BLOCKS_PER_SM)
+k_pareto_coop(CoopSrc<NA> s, Range r, Walk w, u32 *header, P2 *local, P3 *surv, KI *front_list, u64 *idx_out, u32 out_cap, u32 *count_out) {
+    __shared__ P3 sv[CO_P_CHUNK];
+    __shared__ unsigned char flags[CO_P_CHUNK];
+    __shared__ P2 best[CO_DIRS][CO_WARPS];
+    __shared__ P2 ks[CO_DIRS];
+    __shared__ u32 s_n;
+    grid_dep_wait();
+    const u32 lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (blockIdx.x == 0 && threadIdx.x < 64) header[threadIdx.x] = 0;
+    if (threadIdx.x == 0) s_n = 0;
+    // ---- sample ----
+    const u32 total_warps = gridDim.x * CO_WARPS, gwarp = blockIdx.x * CO_WARPS + warp;
+    constexpr u32 N_PTS = 2 * CO_ROWS;
+    u64 px[N_PTS], py[N_PTS];
+    {
+        u32 st[CO_ROWS];
+        double2 v[CO_ROWS][NA];
+#pragma unroll
+        for (u32 u = 0; u < CO_ROWS; u++) {
+            const u64 slot = (u64)u * total_warps + gwarp;
+            load_row(s, r.count, w.row(slot), slot < w.n_slots, lane, st[u], v[u]);
+        }
+#pragma unroll
+        for (u32 u = 0; u < CO_ROWS; u++) {
+            bool ok0, ok1;
+            row_ok(s, st[u], v[u], ok0, ok1);
+            px[2 * u] = py[2 * u] = px[2 * u + 1] = py[2 * u + 1] = KEY_MAX;       // "no point"
+            if (ok0) { px[2 * u] = metric_key(s.a[0], v[u][0].x); py[2 * u] = metric_key(s.a[1], v[u][1].x); }
+            if (ok1) { px[2 * u + 1] = metric_key(s.a[0], v[u][0].y); py[2 * u + 1] = metric_key(s.a[1], v[u][1].y); }
+        }
+    }
+    // ---- killers: per direction the best point of the lane, the warp, the block, all blocks ----
+#pragma unroll 2
+    for (u32 d = 0; d < CO_DIRS; d++) {
+        const u32 wd = direction_weight(d);
+        u32 bs = 0xFFFFFFFFu;
+        u64 bx = KEY_MAX, by = KEY_MAX;
+#pragma unroll
+        for (u32 i = 0; i < N_PTS; i++) {
+            const u32 sc = direction_score(px[i], py[i], wd);
+            if (sc < bs) { bs = sc; bx = px[i]; by = py[i]; }
+        }
+        if (warp_best(bs)) { best[d][warp].x = bx; best[d][warp].y = by; }
+    }
+    __syncthreads();
+    if (warp < CO_DIRS) {
+        P2 p; p.x = KEY_MAX; p.y = KEY_MAX;
+        if (lane < CO_WARPS) p = best[warp][lane];
+        if (warp_best(direction_score(p.x, p.y, direction_weight(warp)))) {
+            if (gridDim.x == 1) ks[warp] = p;
+            else {
+                ulonglong2 e; e.x = p.x; e.y = p.y;
+                *reinterpret_cast<ulonglong2 *>(local + (size_t)warp * CO_MAX_BLOCKS + blockIdx.x) = e;
+            }
+        }
+    }
+    if (gridDim.x > 1) {
+        static_assert(CO_WARPS == 2 * CO_DIRS, "two warps per direction");
+        constexpr u32 PER = CO_MAX_BLOCKS / 64;
+        grid_barrier();
+        const u32 d = warp >> 1, wd = direction_weight(d);
+        ulonglong2 e[PER];
+#pragma unroll
+        for (u32 u = 0; u < PER; u++) {
+            const u32 b = (warp & 1) * 32 + lane + 64 * u;
+            e[u].x = KEY_MAX; e[u].y = KEY_MAX;
+            if (b < gridDim.x) e[u] = __ldcg(reinterpret_cast<const ulonglong2 *>(local + (size_t)d * CO_MAX_BLOCKS + b));
+        }
+        u32 bs = 0xFFFFFFFFu;
+        u64 bx = KEY_MAX, by = KEY_MAX;
+#pragma unroll
+        for (u32 u = 0; u < PER; u++) {
+            const u32 sc = direction_score(e[u].x, e[u].y, wd);
+            if (sc < bs) { bs = sc; bx = e[u].x; by = e[u].y; }
+        }
+        if (warp_best(bs)) { best[d][warp & 1].x = bx; best[d][warp & 1].y = by; }
+        __syncthreads();
+        if (threadIdx.x < CO_DIRS) {
+            const P2 a = best[threadIdx.x][0], b = best[threadIdx.x][1];
+            const u32 wt = direction_weight(threadIdx.x);
+            ks[threadIdx.x] = direction_score(b.x, b.y, wt) < direction_score(a.x, a.y, wt) ? b : a;
+        }
+    }
+    __syncthreads();
+    const Killers8 K = {ks};
+    const u32 lim = min(out_cap, GUIDE_PARETO_MAX);
+    // ---- filter: the sample itself when it was everything, else one pass over the arrays ----
+    if (w.r == 1) {
+#pragma unroll
+        for (u32 i = 0; i < N_PTS; i++) {
+            const bool real = !(px[i] == KEY_MAX && py[i] == KEY_MAX);
+            if (!__any_sync(0xFFFFFFFFu, real)) continue;
+            P3 e; e.x = px[i]; e.y = py[i];
+            e.idx = r.first + ((u64)(i >> 1) * total_warps + gwarp) * ROW + 2 * lane + (i & 1);
+            const bool take = real && !K.kills(px[i], py[i]);
+            if (gridDim.x == 1) warp_append(take, e, &s_n, sv, CO_P_CHUNK);
+            else warp_append(take, e, header + PH_COUNT, surv, PA_SURV_CAP);
+        }
+    } else {
+        const u64 stride = (u64)gridDim.x * CO_WARPS;
+        FilterWalk fw(w.n_rows, stride, warp * gridDim.x + blockIdx.x), ahead = fw;
+        u32 st[CO_ROWS], st_ahead[CO_ROWS];
+        load_chunk_status(s, r.count, ahead, lane, st_ahead);
+        for (; fw.more(); fw = ahead) {
+#pragma unroll
+            for (u32 u = 0; u < CO_ROWS; u++) st[u] = st_ahead[u];
+            ahead.next();
+            load_chunk_status(s, r.count, ahead, lane, st_ahead);
+            double2 v[CO_ROWS][NA];
+            if (!load_chunk_values(s, r.count, fw, lane, st, v)) continue;
+#pragma unroll
+            for (u32 u = 0; u < CO_ROWS; u++) {
+                bool okh[2];
+                row_ok(s, st[u], v[u], okh[0], okh[1]);
+                if (!__any_sync(0xFFFFFFFFu, okh[0] | okh[1])) continue;
+                const u64 x[2] = {metric_key(s.a[0], v[u][0].x), metric_key(s.a[0], v[u][0].y)};
+                const u64 y[2] = {metric_key(s.a[1], v[u][1].x), metric_key(s.a[1], v[u][1].y)};
+#pragma unroll
+                for (u32 h = 0; h < 2; h++) {
+                    P3 e; e.x = x[h]; e.y = y[h]; e.idx = r.first + fw.row(u) * ROW + 2 * lane + h;
+                    warp_append(okh[h] && !K.kills(x[h], y[h]), e, header + PH_COUNT, surv, PA_SURV_CAP);
+                }
+            }
+        }
+    }
+    // ---- finish ----
+    if (gridDim.x == 1) {
+        __syncthreads();
+        if (s_n > CO_P_CHUNK) { if (threadIdx.x == 0) header[1] = 1; }      // the general kernel redoes the call
+        else pareto_small(sv, s_n, flags, lim, idx_out, count_out);
+        return;
+    }
+    grid_barrier();
+    const u32 n = __ldcg(header + PH_COUNT);
+    if (n > PA_SURV_CAP) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) header[1] = 1;
+        return;
+    }
+    const u64 *words = reinterpret_cast<const u64 *>(surv);
+    if (n <= CO_P_DIRECT) {
+        if (blockIdx.x != 0) return;
+        for (u32 i = threadIdx.x; i < 3 * n; i += CO_THREADS) reinterpret_cast<u64 *>(sv)[i] = __ldcg(words + i);
+        __syncthreads();
+        pareto_small(sv, n, flags, lim, idx_out, count_out);
+        return;
+    }
+    // Many: the survivors are judged by all warps, against chunks of the list staged in shared memory;
+    // those nobody rules out go to a second list.
+    const u32 flat_warp = warp * gridDim.x + blockIdx.x;
+    for (u32 g0 = 0; g0 < n; g0 += total_warps) {
+        const u32 g = g0 + flat_warp;
+        u64 mx = 0, my = 0, mi = 0;
+        if (g < n) { mx = __ldcg(words + 3 * (size_t)g); my = __ldcg(words + 3 * (size_t)g + 1); mi = __ldcg(words + 3 * (size_t)g + 2); }
+        bool out = g >= n;
+        for (u32 c0 = 0; c0 < n; c0 += CO_P_CHUNK) {
+            const u32 nc = min(CO_P_CHUNK, n - c0);
+            __syncthreads();
+            for (u32 i = threadIdx.x; i < 3 * nc; i += CO_THREADS) reinterpret_cast<u64 *>(sv)[i] = __ldcg(words + 3 * (size_t)c0 + i);
+            __syncthreads();
+            for (u32 i = lane; i < nc && !out; i += 32) {
+                const P3 o = sv[i];
+                out = dominates(o.x, o.y, mx, my) || (o.x == mx && o.y == my && o.idx < mi);
+            }
+        }
+        if (!__any_sync(0xFFFFFFFFu, out) && lane == 0) {
+            const u32 pos = atomicAdd(header + PH_FRONT, 1);                // pos < n <= PA_SURV_CAP
+            front_list[pos].key = mx; front_list[pos].idx = mi;
+        }
+    }
+    grid_barrier();
+    // a front point's place is its rank in x
+    const u32 nfr = __ldcg(header + PH_FRONT);
+    const ulonglong2 *f = reinterpret_cast<const ulonglong2 *>(front_list);
+    for (u32 g = flat_warp; g < nfr; g += total_warps) {
+        const ulonglong2 me = __ldcg(f + g);
+        u32 ahead = 0;
+        for (u32 i = lane; i < nfr; i += 32) ahead += __ldcg(f + i).x < me.x ? 1u : 0u;
+        ahead = __reduce_add_sync(0xFFFFFFFFu, ahead);
+        if (lane == 0 && ahead < lim) idx_out[ahead] = me.y;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) *count_out = nfr > GUIDE_PARETO_MAX ? 0xFFFFFFFFu : nfr;
+}
+
+// ---- host side -----------------------------------------------------------------------------------------
+
+// The arrays a call touches, each once: metric(s) first, then the bounded ones not yet listed.
+static int collect_arrays(const guide_outputs &o, const guide_constraints &c, int m0, int m1, Arr *arr) {
+    int n = 0;
+    auto add_metric = [&](int key) { arr[n++] = Arr{metric_array_of(o, key), 0.0, 0, key == GUIDE_THROUGHPUT ? 1 : 0}; };
+    add_metric(m0);
+    if (m1 >= 0) add_metric(m1);
+    auto add_bound = [&](const double *p, double bound, int cmp) {
+        for (int i = 0; i < n; i++)
+            if (arr[i].p == p && arr[i].cmp == 0) { arr[i].bound = bound; arr[i].cmp = cmp; return; }
+        arr[n++] = Arr{p, bound, cmp, 0};
+    };
+    if (c.max_ttft < INFINITY)
+        add_bound(c.ttft_stat == GUIDE_STAT_MEAN ? o.ttft : c.ttft_stat == GUIDE_STAT_P50 ? o.ttft_p50 : o.ttft_p99, c.max_ttft, 1);
+    if (c.max_latency < INFINITY) add_bound(o.latency, c.max_latency, 1);
+    if (c.max_cost_per_hr < INFINITY) add_bound(o.cost_per_hr, c.max_cost_per_hr, 1);
+    if (c.min_throughput > 0.0) add_bound(o.thr_decode, c.min_throughput, 2);
+    return n;
+}
+
+// Does the device launch cooperatively, with CO_BLOCKS_PER_SM blocks resident per SM?  Asked once per
+// device.  Setting GUIDE_NO_COOPERATIVE in the environment takes every call to the accumulator kernels
+// (the tests use it to cover both).
+bool coop_select_ok() {
+    static int cached[64] = {};                      // 0 unknown, 1 yes, 2 no
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+    if (!cached[dev]) {
+        int coop = 0, t = 0, p = 0;
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&t, k_topk_coop<MAX_ARR - 1>, CO_THREADS, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, k_pareto_coop<MAX_ARR>, CO_THREADS, 0);
+        if (getenv("GUIDE_NO_COOPERATIVE")) coop = 0;
+        cached[dev] = (coop && t >= (int)CO_BLOCKS_PER_SM && p >= (int)CO_BLOCKS_PER_SM) ? 1 : 2;
+    }
+    return cached[dev] == 1;
+}
+
+// One row per warp while that fills the machine; a range one block can hold in its registers is one block.
+static u32 coop_grid(u64 n_rows) {
+    if (n_rows <= CO_ONE_BLOCK_ROWS) return 1;
+    return (u32)std::min<u64>((n_rows + CO_WARPS - 1) / CO_WARPS, std::min<u64>((u64)num_sms() * CO_BLOCKS_PER_SM, CO_MAX_BLOCKS));
+}
+
+// All rows while the warps' registers hold them, else one out of every r, as many as they hold.
+static Walk make_walk(u64 n_rows, u32 grid) {
+    const u64 room = (u64)grid * CO_WARPS * CO_ROWS;
+    Walk w;
+    w.n_rows = n_rows;
+    w.r = (u32)std::max<u64>((n_rows + room - 1) / room, 1);
+    w.n_slots = n_rows / w.r;
+    return w;
+}
+
+template <class... KArgs, class... Args>
+static cudaError_t launch_coop(void (*kernel)(KArgs...), u32 grid, cudaStream_t st, Args... args) {
+    if (grid == 1) return launch_dependent(kernel, 1, CO_THREADS, 0, st, args...);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(CO_THREADS); cfg.dynamicSmemBytes = 0; cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+
+// workspace region of a top-k call: KI minima[CO_BOUND_LIST] | KI spairs[CO_BOUND_LIST] | KI cand[TK_CAND_CAP]
+size_t topk_coop_bytes() { return ((size_t)2 * CO_BOUND_LIST + TK_CAND_CAP) * sizeof(KI); }
+// ... and of a Pareto call: P2 local[CO_DIRS][CO_MAX_BLOCKS] | P3 surv[PA_SURV_CAP] | KI front[PA_SURV_CAP]
+size_t pareto_coop_bytes() { return (size_t)CO_DIRS * CO_MAX_BLOCKS * sizeof(P2) + (size_t)PA_SURV_CAP * (sizeof(P3) + sizeof(KI)); }
+
+template <int NA>
+static int topk_coop_na(const Arr *arr, Range r, const guide_outputs &mat, u32 k, int negate, u32 *header, unsigned char *region,
+                        u64 *idx_out, double *key_out, u32 *count_out, cudaStream_t st) {
+    CoopSrc<NA> s;
+    for (int i = 0; i < NA; i++) s.a[i] = arr[i];
+    s.status = mat.status;
+    s.vec = mat_vec_ok(mat);
+    KI *minima = reinterpret_cast<KI *>(region), *spairs = minima + CO_BOUND_LIST, *cand = spairs + CO_BOUND_LIST;
+    const u64 n_rows = (r.count + ROW - 1) / ROW;
+    const u32 grid = coop_grid(n_rows);
+    u32 group_log2 = 0;
+    while (((grid * CO_WARPS) >> group_log2) > CO_BOUND_LIST) group_log2++;
+    GUIDE_CUDA(launch_coop(k_topk_coop<NA>, grid, st, s, r, make_walk(n_rows, grid), k, group_log2, header, minima, spairs, cand, negate,
+                           idx_out, key_out, count_out));
+    return GUIDE_OK;
+}
+
+int launch_topk_coop(Range r, const guide_outputs &mat, const guide_constraints &c, int key, u32 k, u32 *header,
+                     unsigned char *region, u64 *idx_out, double *key_out, u32 *count_out, cudaStream_t st) {
+    Arr arr[MAX_ARR];
+    const int na = collect_arrays(mat, c, key, -1, arr);
+    const int negate = key == GUIDE_THROUGHPUT;
+    switch (na) {
+    case 1: return topk_coop_na<1>(arr, r, mat, k, negate, header, region, idx_out, key_out, count_out, st);
+    case 2: return topk_coop_na<2>(arr, r, mat, k, negate, header, region, idx_out, key_out, count_out, st);
+    case 3: return topk_coop_na<3>(arr, r, mat, k, negate, header, region, idx_out, key_out, count_out, st);
+    case 4: return topk_coop_na<4>(arr, r, mat, k, negate, header, region, idx_out, key_out, count_out, st);
+    case 5: return topk_coop_na<5>(arr, r, mat, k, negate, header, region, idx_out, key_out, count_out, st);
+    default: return fail(GUIDE_ERR_UNSUPPORTED, "a top-k call touches at most five arrays");
+    }
+}
+
+template <int NA>
+static int pareto_coop_na(const Arr *arr, Range r, const guide_outputs &mat, u32 *header, unsigned char *region, u64 *idx_out,
+                          u32 cap, u32 *count_out, cudaStream_t st) {
+    CoopSrc<NA> s;
+    for (int i = 0; i < NA; i++) s.a[i] = arr[i];
+    s.status = mat.status;
+    s.vec = mat_vec_ok(mat);
+    P2 *local = reinterpret_cast<P2 *>(region);
+    P3 *surv = reinterpret_cast<P3 *>(region + (size_t)CO_DIRS * CO_MAX_BLOCKS * sizeof(P2));
+    KI *front = reinterpret_cast<KI *>(region + (size_t)CO_DIRS * CO_MAX_BLOCKS * sizeof(P2) + (size_t)PA_SURV_CAP * sizeof(P3));
+    const u64 n_rows = (r.count + ROW - 1) / ROW;
+    const u32 grid = coop_grid(n_rows);
+    GUIDE_CUDA(launch_coop(k_pareto_coop<NA>, grid, st, s, r, make_walk(n_rows, grid), header, local, surv, front, idx_out, cap, count_out));
+    return GUIDE_OK;
+}
+
+int launch_pareto_coop(Range r, const guide_outputs &mat, const guide_constraints &c, int xm, int ym, u32 *header,
+                       unsigned char *region, u64 *idx_out, u32 cap, u32 *count_out, cudaStream_t st) {
+    Arr arr[MAX_ARR];
+    const int na = collect_arrays(mat, c, xm, ym, arr);
+    switch (na) {
+    case 2: return pareto_coop_na<2>(arr, r, mat, header, region, idx_out, cap, count_out, st);
+    case 3: return pareto_coop_na<3>(arr, r, mat, header, region, idx_out, cap, count_out, st);
+    case 4: return pareto_coop_na<4>(arr, r, mat, header, region, idx_out, cap, count_out, st);
+    case 5: return pareto_coop_na<5>(arr, r, mat, header, region, idx_out, cap, count_out, st);
+    case 6: return pareto_coop_na<6>(arr, r, mat, header, region, idx_out, cap, count_out, st);
+    default: return fail(GUIDE_ERR_UNSUPPORTED, "a Pareto call touches two to six arrays");
+    }
+}
+
+}  // namespace guide

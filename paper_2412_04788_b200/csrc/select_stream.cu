@@ -1,21 +1,20 @@
-// Streaming selection over materialised metrics (constraint filter + top-k / Pareto front of
-// Sec. 3.2 / Sec. 4.1 on arrays written by guide_simulate).
+// Streaming selection fused with the closed-form evaluation (constraint filter + top-k / Pareto front of
+// Sec. 3.2 / Sec. 4.1; nothing is materialised).
 //
-// A selection keeps a handful of configs out of millions, so the work is reading the arrays once at
-// memory speed; what has to be avoided is every warp of the grid building its own partial answer
-// before it can reject anything.  Three small steps do that:
+// A selection keeps a handful of configs out of millions; what has to be avoided is every warp of the
+// grid building its own partial answer before it can reject anything.  Four small steps do that:
 //
-//   sample : rows of 64 consecutive configs, one row out of every r at a hashed position, are read
-//            by a small grid.  Top-k: every block reports the smallest passing (key, index) pair it
-//            saw; the k-th smallest of those block minima is a pair that at least k passing configs
-//            reach, hence an upper bound of the k-th pair of the whole range.  A second pass over the
-//            same rows gathers the sample pairs within that bound and replaces it by their k-th
-//            smallest, the exact k-th pair of the sample.  Pareto: every block reduces its sample to
-//            its own front; the last block to finish merges those into one staircase of real points
-//            ("killers"), sorted by x.
-//   filter : one pass over everything.  A config survives if it passes the constraints and its
-//            pair is within the bound (top-k), or no killer strictly dominates it (Pareto).
-//            Survivors go to a list in the workspace through one atomic counter; there are few.
+//   sample : rows of 64 consecutive configs, one row out of every r at a hashed position, are evaluated
+//            config by config into a compact scratch in the workspace.
+//   bound  : top-k: every block reports the smallest passing (key, index) pair it saw; the k-th
+//            smallest of those block minima is a pair that at least k passing configs reach, hence an
+//            upper bound of the k-th pair of the whole range.  A second pass over the same rows gathers
+//            the sample pairs within that bound and replaces it by their k-th smallest, the exact k-th
+//            pair of the sample.  Pareto: every block reduces its sample to its own front; the last
+//            block to finish merges those into one staircase of real points ("killers"), sorted by x.
+//   filter : the model walk.  A config survives if it passes the constraints and its pair is within
+//            the bound (top-k), or no killer strictly dominates it (Pareto).  Survivors go to a list
+//            in the workspace through one atomic counter; there are few.
 //   finish : every survivor is ranked against all others by one warp (the list staged in shared
 //            memory): top-k writes the pairs of rank < k in place; Pareto keeps the survivors no
 //            other survivor rules out and orders them by x.
@@ -26,7 +25,7 @@
 // kernels queued behind this path (select.cu) redo the call.
 //
 // Loads are laid out so that a warp reads 512 contiguous bytes of each array per instruction (a
-// thread takes two consecutive configs, 16 bytes), two such rows per thread and round.
+// thread takes two consecutive configs, 16 bytes).
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
@@ -34,13 +33,9 @@
 #include <cooperative_groups.h>
 
 #include "model_walk.cuh"
-#include "select_sink.cuh"
+#include "select_src.cuh"
 
 namespace guide {
-
-static constexpr u32 ROW = 64;                  // configs per warp-wide load (32 lanes x 2)
-static constexpr u32 TILE = 1024;               // configs per block and round of the filter pass
-static constexpr int MAX_ARR = 6;               // distinct arrays a call can touch
 
 static constexpr u32 SAMPLE_BATCH = 4;          // rows a warp has in flight at once
 
@@ -58,13 +53,6 @@ static constexpr u32 PA_LOCAL_CAP = 1024;       // per-block list of sample poin
 static constexpr u32 PA_PER_BLOCK = 2;          // front points a sample block hands on
 static_assert(PA_KILLERS == PA_SAMPLE_BLOCKS * PA_PER_BLOCK, "every sample block hands on its share of the killers");
 
-// one metric array with the role it plays in this call
-struct Arr {
-    const double *p;
-    double bound;
-    int cmp;          // 0: no bound, 1: value <= bound, 2: value >= bound
-    int neg;          // used as a metric through its negation (throughput)
-};
 // arrays in use: entry 0 is the key (top-k) or x (Pareto), entry 1 is y (Pareto only)
 template <int NA>
 struct Src {
@@ -100,8 +88,6 @@ static_assert(PA_SAMPLE_BLOCKS * 4 <= 512, "local_n fits its slot");
 static constexpr size_t PA_OFF_FUSED = (PA_OFF_FRONT + (size_t)PA_SURV_CAP * sizeof(KI) + 255) / 256 * 256;
 size_t pareto_stream_bytes() { return PA_OFF_FUSED + FU_BYTES; }
 
-bool stream_eligible(const guide_outputs &mat, Range r) { return r.count >= STREAM_MIN_COUNT && mat_vec_ok(mat) != 0; }
-
 // ---- loads and the constraint filter ----------------------------------------------------------------
 
 // two consecutive configs j, j+1 (j even): status bytes and one 16-byte load per array
@@ -110,32 +96,6 @@ __device__ __forceinline__ void load_pair(const Src<NA> &s, u64 j, u32 &st, doub
     st = __ldcs(reinterpret_cast<const unsigned short *>(s.status + j));
 #pragma unroll
     for (int a = 0; a < NA; a++) v[a] = __ldcs(reinterpret_cast<const double2 *>(s.a[a].p + j));
-}
-
-__device__ __forceinline__ bool within(const Arr &a, double v) {
-    // no bound, value <= bound, or value >= bound; written so that a NaN fails an active bound
-    return a.cmp == 0 || (a.cmp == 1 ? v <= a.bound : v >= a.bound);
-}
-
-// The two pairs of a thread in a filter tile (a warp: 64 consecutive configs at j0, 64 at j1).  The
-// status bytes come first; the metric values of a 64-config group are loaded only when some config of
-// the group passed its memory check, which most groups of a large sweep do not: whole runs of the
-// length axis do not fit, and their 512 bytes per array are never read.  Returns false when both
-// groups are dead.
-template <int NA>
-__device__ __forceinline__ bool load_live_pairs(const Src<NA> &s, u64 j0, u64 j1, u32 &st0, u32 &st1, double2 (&v0)[NA],
-                                                double2 (&v1)[NA]) {
-    st0 = __ldcs(reinterpret_cast<const unsigned short *>(s.status + j0));
-    st1 = __ldcs(reinterpret_cast<const unsigned short *>(s.status + j1));
-    const bool g0 = __any_sync(0xFFFFFFFFu, (st0 & 0xFFu) == 0 || (st0 >> 8) == 0);
-    const bool g1 = __any_sync(0xFFFFFFFFu, (st1 & 0xFFu) == 0 || (st1 >> 8) == 0);
-    if (!g0 && !g1) return false;
-#pragma unroll
-    for (int a = 0; a < NA; a++) {
-        v0[a] = g0 ? __ldcs(reinterpret_cast<const double2 *>(s.a[a].p + j0)) : make_double2(0.0, 0.0);
-        v1[a] = g1 ? __ldcs(reinterpret_cast<const double2 *>(s.a[a].p + j1)) : make_double2(0.0, 0.0);
-    }
-    return true;
 }
 
 template <int NA>
@@ -147,20 +107,6 @@ __device__ __forceinline__ void eval_pair(const Src<NA> &s, u32 st, const double
         ok0 &= within(s.a[a], v[a].x);
         ok1 &= within(s.a[a], v[a].y);
     }
-}
-
-__device__ __forceinline__ u64 metric_key(const Arr &a, double v) { return enc(a.neg ? 0.0 - v : v); }
-
-// one config through scalar loads (ragged tail of the range)
-template <int NA>
-__device__ __forceinline__ bool eval_one(const Src<NA> &s, u64 j, u64 &k0, u64 &k1) {
-    bool ok = s.status[j] == 0;
-    double v[NA];
-#pragma unroll
-    for (int a = 0; a < NA; a++) { v[a] = s.a[a].p[j]; ok &= within(s.a[a], v[a]); }
-    k0 = metric_key(s.a[0], v[0]);
-    k1 = NA > 1 ? metric_key(s.a[NA > 1 ? 1 : 0], v[NA > 1 ? 1 : 0]) : 0;
-    return ok;
 }
 
 // The sample: the range is cut into groups of r consecutive rows and one row per group is read, at
@@ -197,11 +143,6 @@ __device__ __forceinline__ void load_batch(const Src<NA> &s, const Sample &sm, u
 }
 
 // ---- top-k ---------------------------------------------------------------------------------------
-//
-__device__ __forceinline__ void pair_min(u64 &key, u64 &idx, u64 okey, u64 oidx) {
-    if (okey < key || (okey == key && oidx < idx)) { key = okey; idx = oidx; }
-}
-
 // k-th smallest (k >= 1) of the n <= blockDim.x * PER pairs in shared memory, by counting: entry i
 // has rank #{entries before it in the total order}; indices are distinct, so ranks are.  The thread
 // that finds rank k-1 writes the bound.  All-ones pairs are padding and sort last.
@@ -468,45 +409,6 @@ __global__ void __launch_bounds__(SEL_THREADS) k_topk_bound(Src<NA> s, Sample sm
     }
 }
 
-// Filter pass: passing configs within the bound go to the candidate list.
-template <int NA>
-__global__ void __launch_bounds__(SEL_THREADS, 4) k_topk_filter(Src<NA> s, Range r, u32 *header, KI *cand) {
-    grid_dep_wait();
-    const u64 *bp = reinterpret_cast<const u64 *>(header + TK_BOUND);
-    const u64 bkey = __ldcg(bp), bidx = __ldcg(bp + 1);
-    const u64 tiles = r.count / TILE;
-    // from the end of the range backwards: when the metrics were written just before this call the
-    // end of the arrays is what the L2 still holds
-    for (u64 back = blockIdx.x; back < tiles; back += gridDim.x) {
-        const u64 tile = tiles - 1 - back;
-        const u64 j0 = tile * TILE + 2 * threadIdx.x, j1 = j0 + TILE / 2;
-        u32 st0, st1;
-        double2 v0[NA], v1[NA];
-        if (!load_live_pairs(s, j0, j1, st0, st1, v0, v1)) continue;
-        bool ok[4];
-        eval_pair(s, st0, v0, ok[0], ok[1]);
-        eval_pair(s, st1, v1, ok[2], ok[3]);
-        const u64 key[4] = {metric_key(s.a[0], v0[0].x), metric_key(s.a[0], v0[0].y), metric_key(s.a[0], v1[0].x),
-                            metric_key(s.a[0], v1[0].y)};
-        bool any = false;
-#pragma unroll
-        for (int u = 0; u < 4; u++) { ok[u] = ok[u] && key[u] <= bkey; any |= ok[u]; }
-        if (!__any_sync(0xFFFFFFFFu, any)) continue;        // the usual case: nothing in this warp's 128 configs
-#pragma unroll
-        for (int u = 0; u < 4; u++) {
-            const u64 idx = r.first + (u < 2 ? j0 : j1) + (u & 1);
-            if (ok[u] && pair_le(key[u], idx, bkey, bidx)) topk_keep(key[u], idx, header, cand);
-        }
-    }
-    grid_dep_launch();              // late: the rank kernel needs this block's registers only now
-    if (blockIdx.x == gridDim.x - 1) {                      // ragged tail, scalar loads
-        for (u64 j = tiles * TILE + threadIdx.x; j < r.count; j += blockDim.x) {
-            u64 k0, k1;
-            if (eval_one(s, j, k0, k1) && pair_le(k0, r.first + j, bkey, bidx)) topk_keep(k0, r.first + j, header, cand);
-        }
-    }
-}
-
 // Finish: every block stages the candidate list in shared memory; one warp per candidate counts
 // the candidates ahead of it.  Ranks are distinct (config indices are), so every output slot has
 // one writer.
@@ -719,54 +621,6 @@ __global__ void __launch_bounds__(SEL_THREADS) k_pareto_sample(Src<NA> s, Sample
     if (threadIdx.x == 0) header[PH_KILLERS] = total;
 }
 
-// Filter pass: passing configs no killer strictly dominates go to the survivor list.
-template <int NA>
-__global__ void __launch_bounds__(SEL_THREADS, 4) k_pareto_filter(Src<NA> s, Range r, u32 *header, const P2 *killers, P3 *surv) {
-    __shared__ P2 ks[PA_KILLERS];
-    grid_dep_wait();
-    KillerSet K;
-    K.k = ks;
-    K.n = min(__ldcg(header + PH_KILLERS), PA_KILLERS);
-    for (u32 i = threadIdx.x; i < K.n; i += blockDim.x) {
-        const ulonglong2 w = __ldcg(reinterpret_cast<const ulonglong2 *>(killers + i));
-        ks[i].x = w.x; ks[i].y = w.y;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 4; i++) {
-        if (K.n > 0) { const P2 p = ks[(K.n * (2 * i + 1)) / 8]; K.rx[i] = p.x; K.ry[i] = p.y; }
-        else { K.rx[i] = KEY_MAX; K.ry[i] = KEY_MAX; }
-    }
-    const u64 tiles = r.count / TILE;
-    // from the end of the range backwards: when the metrics were written just before this call the
-    // end of the arrays is what the L2 still holds
-    for (u64 back = blockIdx.x; back < tiles; back += gridDim.x) {
-        const u64 tile = tiles - 1 - back;
-        const u64 j0 = tile * TILE + 2 * threadIdx.x, j1 = j0 + TILE / 2;
-        u32 st0, st1;
-        double2 v0[NA], v1[NA];
-        if (!load_live_pairs(s, j0, j1, st0, st1, v0, v1)) continue;
-        bool ok[4];
-        eval_pair(s, st0, v0, ok[0], ok[1]);
-        eval_pair(s, st1, v1, ok[2], ok[3]);
-        if (!__any_sync(0xFFFFFFFFu, ok[0] | ok[1] | ok[2] | ok[3])) continue;
-        const Arr &ax = s.a[0], &ay = s.a[1 % NA];
-        const u64 x[4] = {metric_key(ax, v0[0].x), metric_key(ax, v0[0].y), metric_key(ax, v1[0].x), metric_key(ax, v1[0].y)};
-        const u64 y[4] = {metric_key(ay, v0[1 % NA].x), metric_key(ay, v0[1 % NA].y), metric_key(ay, v1[1 % NA].x),
-                          metric_key(ay, v1[1 % NA].y)};
-#pragma unroll
-        for (int u = 0; u < 4; u++)
-            if (ok[u] && !K.kills(x[u], y[u])) pareto_keep(x[u], y[u], r.first + (u < 2 ? j0 : j1) + (u & 1), header, surv);
-    }
-    grid_dep_launch();              // late: the rank kernel needs this block's registers only now
-    if (blockIdx.x == gridDim.x - 1) {                      // ragged tail, scalar loads
-        for (u64 j = tiles * TILE + threadIdx.x; j < r.count; j += blockDim.x) {
-            u64 x, y;
-            if (eval_one(s, j, x, y) && !K.kills(x, y)) pareto_keep(x, y, r.first + j, header, surv);
-        }
-    }
-}
-
 // Finish.  Every block stages the survivors in shared memory; one warp per survivor looks for a
 // survivor that rules it out (a dominating point, or an equal point with a lower index); those left
 // are the front and go to a second list.  The block that finishes last places each front point at
@@ -828,30 +682,6 @@ __global__ void __launch_bounds__(SEL_THREADS) k_pareto_rank(u32 *header, const 
 
 // ---- host side -----------------------------------------------------------------------------------------
 
-// The arrays a call touches, each once: metric(s) first, then the bounded ones not yet listed.
-static int collect_arrays(const guide_outputs &o, const guide_constraints &c, int m0, int m1, Arr *arr) {
-    int n = 0;
-    auto add_metric = [&](int key) { arr[n++] = Arr{metric_array_of(o, key), 0.0, 0, key == GUIDE_THROUGHPUT ? 1 : 0}; };
-    add_metric(m0);
-    if (m1 >= 0) add_metric(m1);
-    auto add_bound = [&](const double *p, double bound, int cmp) {
-        for (int i = 0; i < n; i++)
-            if (arr[i].p == p && arr[i].cmp == 0) { arr[i].bound = bound; arr[i].cmp = cmp; return; }
-        arr[n++] = Arr{p, bound, cmp, 0};
-    };
-    if (c.max_ttft < INFINITY)
-        add_bound(c.ttft_stat == GUIDE_STAT_MEAN ? o.ttft : c.ttft_stat == GUIDE_STAT_P50 ? o.ttft_p50 : o.ttft_p99, c.max_ttft, 1);
-    if (c.max_latency < INFINITY) add_bound(o.latency, c.max_latency, 1);
-    if (c.max_cost_per_hr < INFINITY) add_bound(o.cost_per_hr, c.max_cost_per_hr, 1);
-    if (c.min_throughput > 0.0) add_bound(o.thr_decode, c.min_throughput, 2);
-    return n;
-}
-
-static u32 filter_grid(u64 count) {
-    const u64 tiles = std::max<u64>(count / TILE, 1);
-    return (u32)std::min<u64>((u64)num_sms() * 4, tiles);
-}
-
 // The walk over the sample (see Sample): groups of r rows, n_slots of them visited.
 static Sample make_sample(u64 n_rows, u32 want_rows, u32 max_r) {
     Sample sm;
@@ -880,94 +710,6 @@ static bool cooperative_ok() {
         cached[dev] = (coop && (u64)per_sm * num_sms() >= TK_SAMPLE_BLOCKS) ? 1 : 2;
     }
     return cached[dev] == 1;
-}
-
-template <int NA>
-static int topk_stream_na(const Arr *arr, Range r, const guide_outputs &mat, u32 k, int negate, u32 *header,
-                          unsigned char *region, u64 *idx_out, double *key_out, u32 *count_out, cudaStream_t st) {
-    Src<NA> s;
-    for (int i = 0; i < NA; i++) s.a[i] = arr[i];
-    s.status = mat.status;
-    s.row_base = nullptr;
-    ulonglong2 *minima = reinterpret_cast<ulonglong2 *>(region);
-    ulonglong2 *spairs = reinterpret_cast<ulonglong2 *>(region + TK_OFF_SKEYS);
-    KI *cand = reinterpret_cast<KI *>(region + TK_OFF_CAND);
-    // the coarse bound needs every block to see rows: the walk covers the whole sample (all groups)
-    Sample sm = make_sample(r.count / ROW, TK_SAMPLE_ROWS, TK_SAMPLE_MAX_R);
-    sm.n_slots = sm.n_groups;
-    if (cooperative_ok<NA>()) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(TK_SAMPLE_BLOCKS); cfg.blockDim = dim3(SEL_THREADS); cfg.dynamicSmemBytes = 0; cfg.stream = st;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeCooperative;
-        at[0].val.cooperative = 1;
-        cfg.attrs = at; cfg.numAttrs = 1;
-        GUIDE_CUDA(cudaLaunchKernelEx(&cfg, k_topk_bound<NA>, s, sm, r.first, k, header, minima, spairs));
-    } else {
-        GUIDE_CUDA(cudaMemsetAsync(header, 0, 256, st));
-        k_topk_sample<NA><<<TK_SAMPLE_BLOCKS, SEL_THREADS, 0, st>>>(s, sm, r.first, k, header, minima);
-        GUIDE_CUDA(cudaGetLastError());
-        GUIDE_CUDA(launch_dependent(k_topk_refine<NA>, TK_SAMPLE_BLOCKS, SEL_THREADS, 0, st, s, sm, r.first, k, header, spairs));
-    }
-    GUIDE_CUDA(launch_dependent(k_topk_filter<NA>, filter_grid(r.count), SEL_THREADS, 0, st, s, r, header, cand));
-    const size_t smem = (size_t)TK_CAND_SMEM * sizeof(KI);
-    GUIDE_CUDA(cudaFuncSetAttribute(k_topk_rank, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    GUIDE_CUDA(launch_dependent(k_topk_rank, num_sms(), SEL_THREADS, smem, st, header, (const KI *)cand, k, negate, idx_out,
-                                key_out, count_out));
-    return GUIDE_OK;
-}
-
-int launch_topk_stream(Range r, const guide_outputs &mat, const guide_constraints &c, int key, u32 k, u32 *header,
-                       unsigned char *region, u64 *idx_out, double *key_out, u32 *count_out, cudaStream_t st) {
-    Arr arr[MAX_ARR];
-    const int na = collect_arrays(mat, c, key, -1, arr);
-    const int negate = key == GUIDE_THROUGHPUT;
-    switch (na) {
-    case 1: return topk_stream_na<1>(arr, r, mat, k, negate, header, region, idx_out, key_out, count_out, st);
-    case 2: return topk_stream_na<2>(arr, r, mat, k, negate, header, region, idx_out, key_out, count_out, st);
-    case 3: return topk_stream_na<3>(arr, r, mat, k, negate, header, region, idx_out, key_out, count_out, st);
-    case 4: return topk_stream_na<4>(arr, r, mat, k, negate, header, region, idx_out, key_out, count_out, st);
-    case 5: return topk_stream_na<5>(arr, r, mat, k, negate, header, region, idx_out, key_out, count_out, st);
-    default: return fail(GUIDE_ERR_UNSUPPORTED, "a top-k call touches at most five arrays");
-    }
-}
-
-template <int NA>
-static int pareto_stream_na(const Arr *arr, Range r, const guide_outputs &mat, u32 *header, unsigned char *region, u64 *idx_out,
-                            u32 cap, u32 *count_out, cudaStream_t st) {
-    Src<NA> s;
-    for (int i = 0; i < NA; i++) s.a[i] = arr[i];
-    s.status = mat.status;
-    s.row_base = nullptr;
-    P2 *local = reinterpret_cast<P2 *>(region);
-    P2 *killers = reinterpret_cast<P2 *>(region + PA_OFF_KILLERS);
-    u32 *local_n = reinterpret_cast<u32 *>(region + PA_OFF_LOCAL_N);
-    P3 *surv = reinterpret_cast<P3 *>(region + PA_OFF_SURV);
-    KI *front = reinterpret_cast<KI *>(region + PA_OFF_FRONT);
-    const Sample sm = make_sample(r.count / ROW, PA_SAMPLE_ROWS, 1u << 20);
-    k_pareto_sample<NA><<<PA_SAMPLE_BLOCKS, SEL_THREADS, 0, st>>>(s, sm, header, local, local_n, killers);
-    GUIDE_CUDA(cudaGetLastError());
-    GUIDE_CUDA(launch_dependent(k_pareto_filter<NA>, filter_grid(r.count), SEL_THREADS, 0, st, s, r, header, (const P2 *)killers,
-                                surv));
-    const size_t smem = (size_t)PA_SURV_CAP * 16;
-    GUIDE_CUDA(cudaFuncSetAttribute(k_pareto_rank, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    GUIDE_CUDA(launch_dependent(k_pareto_rank, num_sms(), SEL_THREADS, smem, st, header, (const P3 *)surv, front, idx_out, cap,
-                                count_out));
-    return GUIDE_OK;
-}
-
-int launch_pareto_stream(Range r, const guide_outputs &mat, const guide_constraints &c, int xm, int ym, u32 *header,
-                         unsigned char *region, u64 *idx_out, u32 cap, u32 *count_out, cudaStream_t st) {
-    Arr arr[MAX_ARR];
-    const int na = collect_arrays(mat, c, xm, ym, arr);
-    switch (na) {
-    case 2: return pareto_stream_na<2>(arr, r, mat, header, region, idx_out, cap, count_out, st);
-    case 3: return pareto_stream_na<3>(arr, r, mat, header, region, idx_out, cap, count_out, st);
-    case 4: return pareto_stream_na<4>(arr, r, mat, header, region, idx_out, cap, count_out, st);
-    case 5: return pareto_stream_na<5>(arr, r, mat, header, region, idx_out, cap, count_out, st);
-    case 6: return pareto_stream_na<6>(arr, r, mat, header, region, idx_out, cap, count_out, st);
-    default: return fail(GUIDE_ERR_UNSUPPORTED, "a Pareto call touches two to six arrays");
-    }
 }
 
 // ---- fused form: nothing materialised ---------------------------------------------------------------
