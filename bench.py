@@ -593,8 +593,8 @@ def run_ours(args):
     bytes_topk = 1 + 8 * len(cons_arrays | {key})
     bytes_pareto = 1 + 8 * len(cons_arrays | {"latency", "cost_per_hr"})
     per = {"guide_simulate (k_closed_form_memory + k_closed_form_lines)": (t_sim / args.steps, BYTES_SIM),
-           "guide_select_topk (k_topk_bound + k_topk_filter + k_topk_rank)": (t_topk / args.steps, bytes_topk),
-           "guide_pareto (k_pareto_sample + k_pareto_filter + k_pareto_rank)": (t_par / args.steps, bytes_pareto)}
+           "guide_select_topk (k_topk_coop)": (t_topk / args.steps, bytes_topk),
+           "guide_pareto (k_pareto_coop)": (t_par / args.steps, bytes_pareto)}
     calls = {}
     for name, (ms, nbytes) in per.items():
         calls[name] = hbm_roofline(nbytes * n_local, ms, hbm_peak, peak_kind, f"{nbytes} algorithmic bytes per config")

@@ -29,6 +29,7 @@ static constexpr unsigned TICKET_SLOTS = 64;
 struct DeviceTables {
     int device = -1;
     void *blob = nullptr;
+    size_t blob_bytes = 0;
     DSpace view{};
     unsigned *tickets = nullptr;     // TICKET_SLOTS slots, 32 words apart
     std::vector<void *> ticket_streams;   // slot i belongs to the calls on ticket_streams[i]
@@ -37,6 +38,7 @@ struct DeviceTables {
 struct DeviceTrace {
     int device = -1;
     void *blob = nullptr;
+    size_t blob_bytes = 0;
     DTrace view{};
 };
 
