@@ -7,9 +7,9 @@
 // do not hold back a whole block.  The clock, counters and the iteration time are warp-uniform.
 //
 // Between events a decode iteration costs O(1): nothing per request is touched.
-//   - Resident requests live in per-warp shared-memory slots in ascending request order and store
-//     invariants, not running values: with D = decode iterations done so far, a slot keeps
-//     base = cache - D and fin = D + tokens still to generate, both constant while it is resident.
+//   - Resident requests live in per-warp shared-memory slots, in no order (the last one fills the slot
+//     of one that leaves; the youngest is searched for when one is evicted), and store invariants,
+//     not running values: with D = decode iterations done so far, a slot keeps base = cache - D and fin = D + tokens still to generate, both constant while it is resident.
 //   - The number of requests whose last KV block is full comes from a histogram of
 //     (cache - D) mod block; the next completion is a countdown; the summed context grows by the
 //     running count each step.
@@ -87,9 +87,8 @@ static_assert(sizeof(DModel) <= 128 && sizeof(DRate) <= 128, "a warp copies each
 struct SlotArrays {
     double tbuf[32];    // times of the 32 iterations a run computes at once
     double dterm[32][4];   // decode terms (fixed tasks, all-reduce, head, activation bytes) of 32 neighbouring resident counts
-    double sc[32];         // the config's task-table factors as doubles (a StageConst), when its counts stay exact in them
-    double rate[10];       // its row of rate10
-    double cst[8];         // its attention and stage constants (read where they are used: they need not live in registers)
+    double task[7][16];    // what a prompt pass needs of each task, one per lane: see prompt_task (when the config's counts stay exact in doubles)
+    double cst[10];        // its attention and stage constants (read where they are used: they need not live in registers)
     DModel m;              // the config's model and (hardware, framework) rates
     DRate rt;
     u32 req[SLOTS];     // request index
@@ -98,6 +97,56 @@ struct SlotArrays {
     u32 hist[HIST];     // residents per (cache - D) mod block
     unsigned char meta[SLOTS];   // phase (6 bits) | first-ever prompt pass | waiting for its prompt pass
 };
+
+// A prompt pass with one task per lane.  Every task time is F x ic against B x im (the sum of both for the
+// all-reduce) with F = p f and B = ((w + p a) / t + p r) m for a count p (new tokens; emitting requests
+// for the LM head; summed squared lengths for attention): stage_fixed and the attention terms of
+// stage_prompt_pass, operation for operation, with zeros and ones where a task has no such term (adding
+// +0 and multiplying by 1 change nothing).  The lanes' times are then added in the fixed order.
+// All lanes working out all tasks took three times the instructions, on the unit with half the rate.
+enum { PT_F, PT_W, PT_A, PT_R, PT_M, PT_IC, PT_IM };
+enum { PT_NORM, PT_QO, PT_KV, PT_RES, PT_UP, PT_ACT, PT_DOWN, PT_HEAD, PT_QK, PT_SOFT, PT_COMM, PT_TASKS };
+__device__ __forceinline__ void prompt_task(double (*task)[16], u32 lane, const StageConst &c, const double *rate, bool flash) {
+    if (lane >= PT_TASKS) return;
+    const double icL = rate[0], icA = rate[1], icE = rate[2], imL = rate[3], imA = rate[4], imE = rate[5];
+    double f = 0.0, w = 0.0, a = 0.0, r = 0.0, m = 1.0, ic = icL, im = imL;
+    switch (lane) {
+    case PT_NORM: f = c.f1; r = c.b1; ic = icE; im = imE; break;
+    case PT_QO: f = c.f2; w = c.w2; a = c.ha; r = c.ha; break;
+    case PT_KV: f = c.f3; w = c.w3; a = c.dk; r = c.ha; m = 2.0; break;
+    case PT_RES: f = c.f5; r = c.b5; ic = icE; im = imE; break;
+    case PT_UP: f = c.f6; w = c.w6; a = c.ia; r = c.ha; m = c.mult6; break;
+    case PT_ACT: f = c.f7; r = c.b7; ic = icE; im = imE; break;
+    case PT_DOWN: f = c.f8; w = c.w6; a = c.ia; r = c.ha; break;
+    case PT_HEAD: f = c.f13; w = c.w13; a = c.va; r = c.ha; break;
+    case PT_QK: f = c.f9; a = flash ? 0.0 : c.xb; ic = icA; im = imA; break;             // w: see prompt_pass
+    case PT_SOFT: f = c.f10; r = flash ? 0.0 : (2.0 * c.xb) * c.inv_t; ic = icA; im = imA; break;
+    case PT_COMM: f = c.hops; r = c.cb; ic = rate[7]; im = rate[6]; break;               // F = hops, whatever the count
+    }
+    task[PT_F][lane] = f; task[PT_W][lane] = w; task[PT_A][lane] = a; task[PT_R][lane] = r; task[PT_M][lane] = m;
+    task[PT_IC][lane] = ic; task[PT_IM][lane] = im;
+}
+template <int TIME_SUM>
+__device__ __forceinline__ double prompt_pass(const double (*task)[16], double *out, u32 lane, double hakv_T, double Td, double Ed, double Ad,
+                                              double inv_t, double Nd, double tovh, double lf) {
+    const u32 i = lane & 15;
+    const double p = i == PT_HEAD ? Ed : i == PT_QK || i == PT_SOFT ? Ad : Td;
+    const double f = task[PT_F][i], w = i == PT_QK ? hakv_T : task[PT_W][i];
+    const double F = i == PT_COMM ? f : p * f;
+    const double B = ((w + p * task[PT_A][i]) * inv_t + p * task[PT_R][i]) * task[PT_M][i];
+    const double tc = F * task[PT_IC][i], tm = B * task[PT_IM][i];
+    __syncwarp();
+    if (lane < PT_TASKS) out[lane] = TIME_SUM || i == PT_COMM ? tc + tm : (tc > tm ? tc : tm);
+    __syncwarp();
+    const double2 *v = reinterpret_cast<const double2 *>(out);
+    const double2 a = v[0], b = v[1], c = v[2], d = v[3], e = v[4], g = v[5];
+    double s = a.x + a.y;                          // norm, q/o
+    s = s + b.x;                                   // k/v
+    s = s + a.y;
+    s = s + b.y;                                   // residual
+    s = s + c.x; s = s + c.y; s = s + d.x;         // up, activation, down
+    return combine_phase(s, (e.x + e.y) + e.x, 2.0 * g.x, d.y, 1.0, Nd, tovh, lf);
+}
 
 // Results of one simulated config: per-request values, means in request order, nearest-rank
 // percentiles (sorted in the tpot slice, which is free by then).  Called by the whole warp.
@@ -310,7 +359,6 @@ k_trace_sim(DSpace s, DTrace tr, Range r, int tp_model, u64 max_iters_opt, guide
     double *tpot = (double *)(mine + gen_bytes + first_bytes);
     const u32 n = tr.n;
     const double inf = __longlong_as_double(0x7FF0000000000000LL);
-    const u32 lt_mask = (1u << lane) - 1;
 
     for (;;) {
         u64 w = 0;
@@ -366,17 +414,17 @@ k_trace_sim(DSpace s, DTrace tr, Range r, int tp_model, u64 max_iters_opt, guide
             sl.cst[4] = (double)(2 * (u64)m.H) * inv_tt;                   // F9  = ctx * 2H / t
             sl.cst[5] = (double)((u64)m.Dkv * m.kvb + xw) * inv_tt;        // KV read + score bytes per context token / t
             sl.cst[6] = (double)(5 * (u64)m.nh) * inv_tt;                  // F10 = ctx * 5 n_h / t
+            sl.cst[8] = cvt((u64)m.Dkv * m.kvb);                           // KV bytes per token
             sl.cst[7] = (double)(2 * xw) * inv_tt;                         // B10 = ctx * 2 n_h a_b / t (0 with flash)
         }
         __syncwarp();
 
-        double clock = 0.0, dec_time = 0.0, csum_d = 0.0;   // csum_d mirrors csum when exact53
+        double clock = 0.0, dec_time = 0.0, csum_d = 0.0;   // dec_time: in the upper half of the lanes; csum_d mirrors csum when exact53
         u64 dec_tok = 0, n_iters = 0, n_req_iters = 0, free_blocks = blocks_total, csum = 0;
         u32 next = 0, high_water = 0, nrun = 0, n_new = 0;
         u32 D = 0, Dmod = 0, min_rem = NO_COMPLETION;
         const bool use_hist = blk > 1 && blk <= HIST;
         const bool burst_ok = exact53 && (blk == 1 || use_hist);
-        const u32 lmod = lane % blk, m32 = 32u % blk;     // lane and warp width modulo the block size
         // block sizes are powers of two as a rule: their divisions are shifts
         const u32 blk_shift = (blk & (blk - 1)) == 0 ? (u32)__ffs(blk) - 1 : 0xFFFFFFFFu;
         auto divb = [&](u32 x) { return blk_shift != 0xFFFFFFFFu ? x >> blk_shift : x / blk; };
@@ -389,14 +437,20 @@ k_trace_sim(DSpace s, DTrace tr, Range r, int tp_model, u64 max_iters_opt, guide
         u32 dc_w0 = 0x80000000u;         // first resident count of the window of decode terms in shared memory (none yet)
         u64 pre_T = 0, pre_A = 0;        // prompt tokens (and their squares) admitted since the last prompt pass
         // the head of the waiting queue: its arrival time and the blocks it needs
-        double arr_next = 0.0;
-        u32 need_next = 0, in_next = 0, g_next = 0;              // ... its prompt length (0: the config's) and the tokens kept from before an eviction
+        double arr_next = 0.0, pf_arr = 0.0;
+        u32 need_next = 0, in_next = 0, out_next = 0, g_next = 0;   // ... its lengths (prompt 0: the config's) and the tokens kept from before an eviction
+        u32 pf = n, pf_in = 0, pf_out = 0;                          // request pf is the one behind it, asked for when the head changed
         auto refresh_head = [&]() {
             while (next < high_water && (gen[next] & GEN_DONE)) next++;
             if (next < n) {
-                arr_next = __ldg(tr.arrival + next);
+                if (next == pf) {
+                    arr_next = pf_arr; in_next = pf_in; out_next = pf_out;
+                } else {
+                    arr_next = __ldg(tr.arrival + next); in_next = __ldg(tr.in_len + next); out_next = __ldg(tr.out_len + next);
+                }
+                pf = next + 1;
+                if (pf < n) { pf_arr = __ldg(tr.arrival + pf); pf_in = __ldg(tr.in_len + pf); pf_out = __ldg(tr.out_len + pf); }
                 g_next = next < high_water ? gen[next] : 0u;
-                in_next = __ldg(tr.in_len + next);
                 need_next = blocks_of((in_next ? in_next : Lin) + g_next);
             } else {
                 arr_next = inf; need_next = 0;
@@ -406,9 +460,8 @@ k_trace_sim(DSpace s, DTrace tr, Range r, int tp_model, u64 max_iters_opt, guide
             for (u32 i = lane; i < HIST; i += 32) sl.hist[i] = 0;
             if (sc_ok) {
                 // what a prompt pass needs, next to the warp: the (model, TP degree) factors and the pair's rates
-                const double *scg = reinterpret_cast<const double *>(s.stage_consts + (size_t)(tp_model ? s.n_t : c.t) * s.n_m + c.m);
-                sl.sc[lane] = scg[lane];
-                if (lane < 10) sl.rate[lane] = s.rate10[(size_t)(c.h * s.n_f + c.f) * 10 + lane];
+                prompt_task(sl.task, lane, s.stage_consts[(size_t)(tp_model ? s.n_t : c.t) * s.n_m + c.m], s.rate10 + (size_t)(c.h * s.n_f + c.f) * 10,
+                            rt.flash != 0);
             }
             refresh_head();
             __syncwarp();
@@ -418,10 +471,7 @@ k_trace_sim(DSpace s, DTrace tr, Range r, int tp_model, u64 max_iters_opt, guide
             // ---- 1. admit in arrival order, no overtaking ----
             if (nrun < b && arr_next <= clock && need_next <= free_blocks) {
                 do {
-                    const u32 g = g_next;
-                    u32 in = in_next, out = Lout;
-                    if (in == 0) in = Lin;
-                    else out = __ldg(tr.out_len + next);
+                    const u32 g = g_next, in = in_next ? in_next : Lin, out = in_next ? out_next : Lout;
                     free_blocks -= need_next;
                     if (lane == 0) {
                         sl.req[nrun] = next;
@@ -451,14 +501,10 @@ k_trace_sim(DSpace s, DTrace tr, Range r, int tp_model, u64 max_iters_opt, guide
                 pre_T = 0; pre_A = 0;
                 double t_iter;
                 if (sc_ok) {
-                    // the same operations on doubles (exact for this config), the factors read from shared memory as they are used
-                    const StageConst &sc = *reinterpret_cast<const StageConst *>(sl.sc);
+                    // on doubles (exact for this config), a task per lane
                     const double Td = (double)(long long)T, Ad = (double)(long long)A;
-                    const StageFixed sf = stage_fixed<TIME_SUM>(sc, sl.rate, Td, (double)n_new);
-                    const double xw = rt.flash ? 0.0 : sc.xb;
-                    const double t9 = task_time<TIME_SUM>(Ad * c_f9, ((Td * sc.ha + Td * sc.kv) + Ad * xw) * sc.inv_t, icA, imA);
-                    const double t10 = task_time<TIME_SUM>(Ad * c_f10, Ad * c_b10, icA, imA);
-                    t_iter = combine_phase(sf.fix, (t9 + t10) + t9, sf.comm, sf.head, 1.0, Nd, rt.tovh, lf);
+                    const double ha = sl.task[PT_A][PT_QO], kv = sl.cst[8];
+                    t_iter = prompt_pass<TIME_SUM>(sl.task, sl.tbuf, lane, Td * ha + Td * kv, Td, (double)n_new, Ad, inv_tt, Nd, rt.tovh, lf);
                 } else {
                     TaskTab kt;
                     build_fixed_tasks(m, tt, T, n_new, 1, kt);
@@ -510,8 +556,12 @@ k_trace_sim(DSpace s, DTrace tr, Range r, int tp_model, u64 max_iters_opt, guide
                 }
                 if (needed > free_blocks) {
                     while (needed > free_blocks) {                     // evict the youngest, recompute later
-                        const u32 v = nrun - 1;
-                        const u32 cv = sl.base[v] + D, rq = sl.req[v], rem = sl.fin[v] - D, ph = sl.meta[v] & M_PHASE;
+                        u32 young = 0;                                 // request index << 8 | slot
+                        for (u32 k = lane; k < nrun; k += 32) young = max(young, sl.req[k] << 8 | k);
+                        young = __reduce_max_sync(0xFFFFFFFFu, young);
+                        const u32 v = young & 0xFFu, tail = nrun - 1;
+                        const u32 cv = sl.base[v] + D, rq = young >> 8, rem = sl.fin[v] - D, ph = sl.meta[v] & M_PHASE;
+                        const u32 t_rq = sl.req[tail], t_bs = sl.base[tail], t_fn = sl.fin[tail], t_mt = sl.meta[tail];
                         free_blocks += blocks_of(cv);
                         if (modb(cv) == 0) needed--;
                         csum -= cv;
@@ -520,9 +570,11 @@ k_trace_sim(DSpace s, DTrace tr, Range r, int tp_model, u64 max_iters_opt, guide
                         if (lane == 0) {
                             gen[rq] = out - rem;
                             if (use_hist) sl.hist[ph] -= 1;
+                            sl.req[v] = t_rq; sl.base[v] = t_bs; sl.fin[v] = t_fn; sl.meta[v] = (unsigned char)t_mt;
                         }
-                        nrun--;
+                        nrun = tail;
                         next = rq;
+                        __syncwarp();
                     }
                     __syncwarp();
                     refresh_head();
@@ -551,107 +603,131 @@ k_trace_sim(DSpace s, DTrace tr, Range r, int tp_model, u64 max_iters_opt, guide
                     dc_nd = (double)nrun;
                 }
                 if (burst_ok) {
-                    // A run of decode iterations up to the next event.  Nothing per request is
-                    // touched; integer counters are settled once after the run.  The next
-                    // iteration's time is computed before the clock-dependent exit test so the two
-                    // dependency chains overlap.
+                    // A run of decode iterations up to the next event: nothing per request is touched, and
+                    // integer counters are settled once after the run.  The iterations depend on one
+                    // another through the clock only (the summed context of the i-th is cd0 + i * nd,
+                    // exact), so the 32 lanes work out the times of 32 consecutive ones at once; the
+                    // clock is then advanced one iteration after the other, in order.
+                    //
+                    // What bounds a run is that chain of additions (9 cycles each) and, with many warps,
+                    // instruction issue.  A full batch that nothing can cut short is one straight block:
+                    // 32 additions to the clock and the decode time from shared memory, with the next batch's
+                    // times worked out in their shadow; whether the queue head has arrived is asked once, of
+                    // the clock at the end (it only grows).
                     const u64 cap_left = max_iters - n_iters;
                     const u32 steps_max = (u32)min((u64)min_rem, cap_left);
                     const u32 fb0 = (u32)min(free_blocks, (u64)0xFFFFFFFFu);
-                    u32 fb = fb0, it = 0;
-                    u32 hidx = Dmod + 1 == blk ? 0 : blk - (Dmod + 1);     // histogram bin of the next iteration's needers
+                    const u32 hidx0 = Dmod + 1 == blk ? 0 : blk - (Dmod + 1);     // histogram bin of those who need a block before the second iteration
+                    // the bin of those who need one before iteration j + 2, and the blocks taken before the first j of those
+                    auto bin = [&](u32 j) { const u32 o = modb(j); return hidx0 >= o ? hidx0 - o : hidx0 + blk - o; };
+                    auto taken = [&](u32 j) {
+                        if (blk == 1) return j * nrun;
+                        const u32 q = divb(j), rest = j - q * blk;
+                        u32 v = 0;
+                        if (lane < rest) v = sl.hist[bin(lane)];
+                        if (lane + 32 < rest) v += sl.hist[bin(lane + 32)];
+                        return q * nrun + __reduce_add_sync(0xFFFFFFFFu, v);
+                    };
                     const bool room = nrun < b;
                     const double nd = dc_nd, cd0 = csum_d;
-                    // The iterations of a run do not depend on one another except through the clock:
-                    // the summed context of the i-th is cd0 + i * nd (exact), so the 32 lanes compute
-                    // the times of 32 consecutive iterations at once; which of them ends the run on
-                    // block counts is a prefix sum over the histogram bins, and the clock is then
-                    // advanced one iteration after the other (same order of additions as a scalar
-                    // loop), watching for the arrival of the queue head where it could come in.
+                    double ctx_k = cd0 + nd * (double)(lane + 1);
+                    double t_k = decode_time<TIME_SUM>(ctx_k, c_f9, dc_tha, c_kvx, c_f10, c_b10, icA, imA, dc_fix, dc_comm, dc_head, Nd, rt.tovh, lf);
+                    double acc = lane < 16 ? clock : dec_time;        // half of the lanes carry the clock, half the decode time: one addition for both
+                    u32 it = 0;
+                    u32 fb = fb0, fb_it = 0;                          // blocks free after the first fb_it iterations (and what they ask for)
+                    u32 used = 0xFFFFFFFFu;                           // blocks taken by the whole run, once known
                     for (;;) {
                         const u32 nb = min(32u, steps_max - it);
-                        const double t_k = decode_time<TIME_SUM>(cd0 + nd * ((double)it + (double)(lane + 1)), c_f9, dc_tha, c_kvx, c_f10, c_b10,
-                                                                 icA, imA, dc_fix, dc_comm, dc_head, Nd, rt.tovh, lf);
-                        // blocks the residents need before the iteration after lane's, and what is free by then
-                        u32 need_k = 0;
-                        if (lane < nb) need_k = blk == 1 ? nrun : sl.hist[hidx >= lmod ? hidx - lmod : hidx + blk - lmod];
-                        // Usually the free blocks cover the whole batch and the queue head's need: then only the
-                        // completion count can end the run on integers, and what is free afterwards is one sum.
-                        const u32 total = __reduce_add_sync(0xFFFFFFFFu, need_k);
-                        const bool plenty = (u64)total + need_next <= fb;
-                        u32 fb_k = 0, stops, last, watch;
-                        if (plenty) {
-                            last = nb - 1;
-                            stops = steps_max - it <= 32u ? 1u << last : 0u;
-                            watch = room ? 0xFFFFFFFFu >> (31 - last) : 0u;
-                        } else {
-                            u32 incl = need_k;
+                        u32 need_k = 0, total = 0;                    // blocks asked for after lane's iteration of the batch, and after all of them
+                        bool counted = false;
+                        u32 cnt = nb, watch = room ? 0xFFFFFFFFu : 0u;
+                        bool stop = it + nb == steps_max;             // a completion or the cap follows the batch
+                        // Blocks usually cover the batch and the queue head's need whatever their spread over the
+                        // residents (each takes one every blk iterations); then no count is needed.
+                        if ((u64)nrun * divb(it + nb + blk - 1) + (room ? need_next : 0u) > fb0) {
+                            if (fb_it != it) fb = fb0 - taken(it);
+                            counted = true;
+                            if (lane < nb) need_k = blk == 1 ? nrun : sl.hist[bin(it + lane)];
+                            total = __reduce_add_sync(0xFFFFFFFFu, need_k);
+                            if ((u64)total + (room ? need_next : 0u) > fb) {      // short somewhere, or the queue head may have to wait
+                                u32 incl = need_k;
+                                #pragma unroll
+                                for (int d = 1; d < 32; d <<= 1) {
+                                    const u32 up = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+                                    if (lane >= (u32)d) incl += up;
+                                }
+                                const u32 fb_k = fb - (incl - need_k);            // wraps only behind a lane that already stops
+                                const u32 stops = __ballot_sync(0xFFFFFFFFu, lane < nb && need_k > fb_k);
+                                if (stops) { cnt = (u32)__ffs(stops); stop = true; }     // an eviction follows that iteration
+                                watch = __ballot_sync(0xFFFFFFFFu, room && need_next <= fb_k);
+                            }
+                        }
+                        __syncwarp();
+                        sl.tbuf[lane] = lane < cnt ? t_k : 0.0;          // + 0.0 changes no sum
+                        __syncwarp();
+                        if (cnt == 32) {
+                            ctx_k = ctx_k + 32.0 * nd;
+                            const double t_next = decode_time<TIME_SUM>(ctx_k, c_f9, dc_tha, c_kvx, c_f10, c_b10, icA, imA, dc_fix, dc_comm,
+                                                                        dc_head, Nd, rt.tovh, lf);
+                            double sum = acc;
                             #pragma unroll
-                            for (int d = 1; d < 32; d <<= 1) {
-                                const u32 up = __shfl_up_sync(0xFFFFFFFFu, incl, d);
-                                if (lane >= (u32)d) incl += up;
+                            for (u32 k = 0; k < 32; k += 2) {
+                                const double2 v = *(const double2 *)&sl.tbuf[k];
+                                sum = sum + v.x;
+                                sum = sum + v.y;
                             }
-                            fb_k = fb - (incl - need_k);                  // wraps only behind a lane that already stops
-                            stops = __ballot_sync(0xFFFFFFFFu, lane < nb && (it + lane + 1 == steps_max || need_k > fb_k));
-                            last = stops ? (u32)__ffs(stops) - 1 : 31u;   // a completion, the cap or an eviction follows it
-                            watch = __ballot_sync(0xFFFFFFFFu, room && need_next <= fb_k) & (0xFFFFFFFFu >> (31 - last));
+                            if (watch == 0 || !__any_sync(0xFFFFFFFFu, lane < 16 && arr_next <= sum)) {
+                                acc = sum; it += 32; t_k = t_next;
+                                if (stop) { if (counted) used = fb0 - fb + total - __shfl_sync(0xFFFFFFFFu, need_k, 31); break; }
+                                if (counted) { fb -= total; fb_it = it; }
+                                continue;
+                            }
                         }
-                        sl.tbuf[lane] = t_k;
-                        __syncwarp();
-                        // the clock, one iteration after the other: four per trip, the arrival tests of a trip taken together
-                        u32 k = 0;
+                        // the others, sixteen iterations at a time: lane k of a half adds up the times of the first
+                        // k + 1 only, in order, so that every clock of the sixteen is there at once
+                        u32 ran = 0;
                         bool arrived = false;
-                        const u32 cnt = last + 1;
-                        double2 va = *(const double2 *)&sl.tbuf[0], vb = *(const double2 *)&sl.tbuf[2];
-                        while (k + 4 <= cnt) {
-                            // the next trip's times are loaded ahead of this trip's additions (past the end: wraps, unused)
-                            const double2 na = *(const double2 *)&sl.tbuf[(k + 4) & 31], nb2 = *(const double2 *)&sl.tbuf[(k + 6) & 31];
-                            const double c1 = clock + va.x, c2 = c1 + va.y, c3 = c2 + vb.x, c4 = c3 + vb.y;
-                            const double d1 = dec_time + va.x, d2 = d1 + va.y, d3 = d2 + vb.x, d4 = d3 + vb.y;
-                            const u32 wbits = (watch >> k) & 15u;
-                            u32 hit = 0;
-                            if (wbits)
-                                hit = ((u32)(arr_next <= c1) | ((u32)(arr_next <= c2) << 1) | ((u32)(arr_next <= c3) << 2) |
-                                       ((u32)(arr_next <= c4) << 3)) & wbits;
-                            if (hit) {                                             // the queue head can come in after one of the four
-                                const u32 f = (u32)__ffs(hit) - 1;
-                                clock = f == 0 ? c1 : f == 1 ? c2 : f == 2 ? c3 : c4;
-                                dec_time = f == 0 ? d1 : f == 1 ? d2 : f == 2 ? d3 : d4;
-                                k += f;
-                                arrived = true;
-                                break;
+                        const u32 hl = lane & 15;
+                        #pragma unroll 1
+                        for (u32 q = 0; q < cnt && !arrived; q += 16) {
+                            const u32 m = min(16u, cnt - q);
+                            double sum = acc;
+                            #pragma unroll
+                            for (u32 k = 0; k < 16; k += 2) {
+                                if (k == 2 && m <= 2) break;
+                                if (k == 4 && m <= 4) break;
+                                if (k == 8 && m <= 8) break;
+                                const double2 v = *(const double2 *)&sl.tbuf[q + k];
+                                if (k <= hl) sum = sum + v.x;
+                                if (k + 1 <= hl) sum = sum + v.y;
                             }
-                            clock = c4; dec_time = d4;
-                            va = na; vb = nb2;
-                            k += 4;
+                            // the queue head can come in after the first iteration that ends past its arrival, if it may
+                            const u32 in = __ballot_sync(0xFFFFFFFFu, lane < m && ((watch >> (q + hl)) & 1u) && arr_next <= sum);
+                            arrived = in != 0;
+                            const u32 last = arrived ? (u32)__ffs(in) - 1 : m - 1;
+                            acc = __shfl_sync(0xFFFFFFFFu, sum, (lane & 16) + last);
+                            ran = q + last + 1;
                         }
-                        if (!arrived) {
-                            for (; k < cnt; k++) {
-                                const double v = sl.tbuf[k];
-                                clock = clock + v;
-                                dec_time = dec_time + v;
-                                if (((watch >> k) & 1u) && arr_next <= clock) { arrived = true; break; }
-                            }
-                            if (!arrived) k = last;
-                        }
-                        it += k + 1;
-                        __syncwarp();
-                        if (stops || arrived) {
-                            fb = plenty ? fb - __reduce_add_sync(0xFFFFFFFFu, lane < k ? need_k : 0u) : __shfl_sync(0xFFFFFFFFu, fb_k, k);
+                        it += ran;
+                        if (arrived || stop) {
+                            if (counted && it > 1) used = fb0 - fb + __reduce_add_sync(0xFFFFFFFFu, lane < ran - 1 ? need_k : 0u);
                             break;
                         }
-                        fb = plenty ? fb - total : __shfl_sync(0xFFFFFFFFu, fb_k - need_k, 31);
-                        hidx = hidx >= m32 ? hidx - m32 : hidx + blk - m32;
+                        if (counted) { fb -= total; fb_it = it; }
+                        // a full batch in which the head had arrived but found no blocks: on to the next one
+                        t_k = decode_time<TIME_SUM>(ctx_k, c_f9, dc_tha, c_kvx, c_f10, c_b10, icA, imA, dc_fix, dc_comm, dc_head, Nd, rt.tovh, lf);
                     }
+                    clock = __shfl_sync(0xFFFFFFFFu, acc, 0); dec_time = acc;
                     const double cd = cd0 + nd * (double)it;
                     const u64 tok = (u64)it * nrun;
+                    // what is asked for after the last iteration is taken by the next pass
+                    if (it > 1) free_blocks -= used != 0xFFFFFFFFu ? used : taken(it - 1);
                     D += it;
                     Dmod += it < blk ? it : modb(it);           // short runs are the rule
                     if (Dmod >= blk) Dmod -= blk;
                     csum += tok; csum_d = cd;
                     dec_tok += tok; n_req_iters += tok; n_iters += it;
                     min_rem -= it;
-                    free_blocks -= fb0 - fb;
                     any_done = min_rem == 0;
                 } else {
                     const u64 ctx = csum + nrun;                       // cached tokens + the new one, summed
@@ -679,44 +755,47 @@ k_trace_sim(DSpace s, DTrace tr, Range r, int tp_model, u64 max_iters_opt, guide
             // ---- 5. retire finished sequences, keep the rest in order ----
             if (any_done) {
                 __syncwarp();
-                u32 kept = 0, local_min = NO_COMPLETION;
-                u64 freed = 0, gone = 0;
-                const u32 n_before = nrun;
-                for (u32 base = 0; base < n_before; base += 32) {
-                    const u32 k = base + lane;
-                    const bool valid = k < n_before;
-                    u32 rq = 0, bs = 0, fn = 0, mt = 0;
-                    if (valid) { rq = sl.req[k]; bs = sl.base[k]; fn = sl.fin[k]; mt = sl.meta[k]; }
-                    const u32 rem = fn - D;
-                    const bool done = valid && rem == 0;
-                    if (done) {
-                        const u32 cv = bs + D;
-                        gen[rq] = GEN_DONE;
-                        tpot[rq] = clock;              // time of its last token; the results turn it into time per output token
-                        freed += blocks_of(cv);
-                        gone += cv;
-                        if (use_hist) atomicSub(&sl.hist[mt & M_PHASE], 1u);
-                    }
-                    const bool keep = valid && !done;
-                    if (keep) local_min = min(local_min, rem);
-                    const u32 ballot = __ballot_sync(0xFFFFFFFFu, keep);
-                    __syncwarp();
-                    if (keep) {
-                        const u32 d = kept + __popc(ballot & lt_mask);
-                        sl.req[d] = rq; sl.base[d] = bs; sl.fin[d] = fn; sl.meta[d] = (unsigned char)mt;
-                    }
-                    kept += __popc(ballot);
-                    __syncwarp();
+                // which slots are through (bit c of a lane: its slot of chunk c), and the next completion among the others
+                u32 done = 0, local_min = NO_COMPLETION;
+                #pragma unroll 4
+                for (u32 c = 0; c < SLOTS / 32; c++) {
+                    const u32 k = 32 * c + lane;
+                    if (32 * c >= nrun) break;
+                    const u32 rem = k < nrun ? sl.fin[k] - D : NO_COMPLETION;
+                    if (rem == 0) done |= 1u << c;
+                    else local_min = min(local_min, rem);
                 }
-                free_blocks += warp_sum(freed);
-                csum -= warp_sum(gone);
+                // Usually one.  Highest slot first: the last slot, which fills the hole, is then never one of them.
+                u32 chunks = __reduce_or_sync(0xFFFFFFFFu, done);
+                while (chunks) {
+                    const u32 c = 31 - __clz(chunks);
+                    chunks ^= 1u << c;
+                    u32 in_chunk = __ballot_sync(0xFFFFFFFFu, (done >> c) & 1u);
+                    while (in_chunk) {
+                        const u32 l = 31 - __clz(in_chunk), k = 32 * c + l, tail = nrun - 1;
+                        in_chunk ^= 1u << l;
+                        const u32 rq = sl.req[k], cv = sl.base[k] + D, mt = sl.meta[k];
+                        const u32 t_rq = sl.req[tail], t_bs = sl.base[tail], t_fn = sl.fin[tail], t_mt = sl.meta[tail];
+                        __syncwarp();
+                        if (lane == 0) {
+                            gen[rq] = GEN_DONE;
+                            tpot[rq] = clock;          // time of its last token; the results turn it into time per output token
+                            if (use_hist) sl.hist[mt & M_PHASE] -= 1;
+                            sl.req[k] = t_rq; sl.base[k] = t_bs; sl.fin[k] = t_fn; sl.meta[k] = (unsigned char)t_mt;
+                        }
+                        free_blocks += blocks_of(cv);
+                        csum -= cv;
+                        nrun = tail;
+                        __syncwarp();
+                    }
+                }
                 min_rem = warp_min(local_min);
-                nrun = kept;
                 csum_d = (double)(long long)csum;
             }
         }
 
         // ---- results ----
+        dec_time = __shfl_sync(0xFFFFFFFFu, dec_time, 16);
         write_trace_results(o, j, n, st, fit, clock, dec_time, dec_tok, n_iters, n_req_iters, rt.price * (double)t, tr, Lout,
                                   first, tpot, lane);
         __syncwarp();
