@@ -61,6 +61,33 @@ static u128 weight_bytes(const guide_model &m) {
     return ((u128)m.n_layers * (2 * H * H + 2 * H * Dkv + (2 + (u128)m.gated) * H * I) + 2 * V * H) * m.w_bytes;
 }
 
+// Can the closed form of the whole space be evaluated from products of doubles (stage_parts in
+// model.cuh)?  1: every byte sum of every config stays below 2^52 (and so do the token counts and the
+// factors); 2: every
+// FLOP and byte count, single products all, stays below 2^53, which the binary32 variant needs.  Asked of the largest
+// batch and the longest lengths, which bounds all configs.
+static uint32_t closed_form_exact(const guide_space &s) {
+    // below 2^52 (sums) and 2^53 (single products) by more than the rounding of the products here
+    const double lim = 4.5e15, lim_count = 9.0e15;
+    uint32_t level = 2;
+    for (const guide_model &m : s.models) {
+        const double H = m.hidden, I = m.ffn, V = m.vocab, nh = m.n_heads, ab = m.a_bytes, wb = m.w_bytes, kvb = m.kv_bytes,
+                   Dkv = (double)m.n_kv_heads * (m.hidden / m.n_heads), g = m.gated, t = s.max_tp;
+        const double b = s.max_batch, lin = s.max_lin, n = s.max_lout;
+        const double R = n, T = b * std::max(lin, n), C = b * (n * lin + n * (n + 1) / 2 + lin), A = C + b * lin * lin;
+        const double sums[] = {T, A, R * H * H * wb + T * H * ab, R * H * Dkv * wb + T * Dkv * kvb, R * H * I * wb + T * I * ab,
+                             R * H * V * wb + T * V * ab, T * H * ab + C * Dkv * kvb + nh * A * ab, 4 * H * H, 4 * H * Dkv, 4 * H * I,
+                             2 * H * V, (2 + g) * I * ab, 6 * H * ab, 2 * t * H * ab, 2 * t * R};
+        const double counts[] = {8 * T * H, 2 * T * H * H, 4 * T * H * Dkv, 4 * T * H * I, 4 * T * I, 6 * T * H * ab, (2 + g) * T * I * ab,
+                               2 * T * H * V, 2 * H * A, 5 * nh * A, 2 * nh * A * ab, 2 * t * T * H * ab};
+        for (double v : sums)
+            if (v >= lim) return 0;
+        for (double v : counts)
+            if (v >= lim_count) level = 1;
+    }
+    return level;
+}
+
 static int check_closed_form_overflow(const guide_space &s) {
     for (size_t mi = 0; mi < s.models.size(); mi++) {
         const guide_model &m = s.models[mi];
@@ -382,6 +409,7 @@ int space_on_device(guide_space *s, DSpace *out, unsigned **ticket, cudaStream_t
     d.view.dp = (const u32 *)(blob + o_d);
     d.view.chunked = s->chunked ? 1u : 0u;
     d.view.clamp_seq = 0;
+    d.view.exact = s->exact;
     d.view.pairs = (const uint2 *)(blob + o_p);
     d.view.cost_hr = (const double *)(blob + o_ch);
     d.view.cost_sec = (const double *)(blob + o_cs);
@@ -587,6 +615,7 @@ int guide_space_create(const guide_space_desc *d, guide_space **out) {
                 rc = fail(GUIDE_ERR_OVERFLOW, "KV bytes of one request overflow");
     }
     if (!rc) rc = check_closed_form_overflow(*s);
+    if (!rc) s->exact = closed_form_exact(*s);
     if (rc) { delete s; return rc; }
     *out = s;
     return GUIDE_OK;

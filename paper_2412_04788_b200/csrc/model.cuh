@@ -67,6 +67,7 @@ struct DSpace {
     u32 n_m, n_h, n_f, n_b, n_t, n_l;
     u32 chunked;                 // per-framework prompt splitting or cache eviction, or a per-call option below: only the
                                  // one-thread-per-config evaluation handles those (no tables shared between frameworks)
+    u32 exact;                   // closed form of the whole space: 1 = the byte sums stay below 2^52, 2 = every count is exact in a double (see stage_parts)
     u32 clamp_seq;               // cut sequences that do not fit to S_max (Sec. 3.3.2); set per call
 };
 
@@ -85,6 +86,16 @@ struct Cfg { u32 m, h, f, b, t, l; };
 
 __device__ __forceinline__ Cfg decode_index(const DSpace &s, u64 idx) {
     Cfg c;
+    if ((idx >> 32) == 0) {                // 64-bit divisions take several times the instructions
+        u32 i = (u32)idx;
+        c.l = i % s.n_l; i /= s.n_l;
+        c.t = i % s.n_t; i /= s.n_t;
+        c.b = i % s.n_b; i /= s.n_b;
+        c.f = i % s.n_f; i /= s.n_f;
+        c.h = i % s.n_h; i /= s.n_h;
+        c.m = i;
+        return c;
+    }
     c.l = (u32)(idx % s.n_l); idx /= s.n_l;
     c.t = (u32)(idx % s.n_t); idx /= s.n_t;
     c.b = (u32)(idx % s.n_b); idx /= s.n_b;
@@ -462,6 +473,103 @@ __device__ __forceinline__ void closed_form_metrics(double t_pre, double t_dec, 
     o.n_req_iters = (u64)b * (n_seg + (u64)n);
 }
 
+// ---- a stage of one config from the factors of its (model, TP degree) --------------------------------
+//
+// The integer table above costs a few hundred instructions a stage: 64-bit products and conversions.
+// From the StageConst factors an entry is one product of doubles.  That gives the same bits: a product
+// of two exact factors is rounded once, as the conversion of the integer product is, and the scalings
+// by 1/t and by the multiplicities are by powers of two; a sum of products must be exact before its one
+// rounding, so the byte sums have to stay below 2^52.  In binary32 the value is rounded to binary32
+// afterwards, so there every count has to be exact (below 2^53).  The host checks both on the
+// largest batch and lengths of the space (DSpace::exact); other spaces take the integer table.
+template <class F> __device__ __forceinline__ F rounded(double x);
+template <> __device__ __forceinline__ double rounded<double>(double x) { return x; }
+template <> __device__ __forceinline__ float rounded<float>(double x) { return __double2float_rn(x); }
+
+template <class F> struct Rates { F icL, icA, icE, imL, imA, imE, inv_comm, clat, tovh; bool flash; };
+
+template <int TIME_SUM, class F>
+__device__ __forceinline__ F time_of(F work, F bytes, F ic, F im) {
+    const F tc = work * ic, tm = bytes * im;
+    return TIME_SUM ? tc + tm : (tc > tm ? tc : tm);
+}
+
+// what a stage of T new tokens and R repeats has besides attention and LM head: as stage_fixed
+template <int TIME_SUM, class F>
+__device__ __forceinline__ void stage_parts(const StageConst &c, const Rates<F> &r, double Td, double Rd, F &fix, F &comm) {
+    const double tha = Td * c.ha;
+    const F rep = rounded<F>(tha);                          // the replicated activations
+    const F t2 = time_of<TIME_SUM, F>(rounded<F>(Td * c.f2), rounded<F>((Rd * c.w2 + tha) * c.inv_t) + rep, r.icL, r.imL);
+    F s = time_of<TIME_SUM, F>(rounded<F>(Td * c.f1), rounded<F>(Td * c.b1), r.icE, r.imE);
+    s = s + t2;
+    s = s + time_of<TIME_SUM, F>(rounded<F>(Td * c.f3), (F)2 * (rounded<F>((Rd * c.w3 + Td * c.dk) * c.inv_t) + rep), r.icL, r.imL);
+    s = s + t2;
+    s = s + time_of<TIME_SUM, F>(rounded<F>(Td * c.f5), rounded<F>(Td * c.b5), r.icE, r.imE);
+    const F up = rounded<F>((Rd * c.w6 + Td * c.ia) * c.inv_t) + rep;
+    s = s + time_of<TIME_SUM, F>(rounded<F>(Td * c.f6), rounded<F>(c.mult6) * up, r.icL, r.imL);
+    s = s + time_of<TIME_SUM, F>(rounded<F>(Td * c.f7), rounded<F>(Td * c.b7), r.icE, r.imE);
+    s = s + time_of<TIME_SUM, F>(rounded<F>(Td * c.f8), up, r.icL, r.imL);
+    fix = s;
+    comm = (F)2 * (rounded<F>(Rd * c.hops) * r.clat + rounded<F>(Td * c.cb) * r.inv_comm);
+}
+template <int TIME_SUM, class F>
+__device__ __forceinline__ F stage_attention(const StageConst &c, const Rates<F> &r, double Td, double Ad, double Cd) {
+    double by = Td * c.ha + Cd * c.kv;
+    if (!r.flash) by = by + Ad * c.xb;
+    const F t9 = time_of<TIME_SUM, F>(rounded<F>(Ad * c.f9), rounded<F>(by * c.inv_t), r.icA, r.imA);
+    const F t10 = time_of<TIME_SUM, F>(rounded<F>(Ad * c.f10), r.flash ? (F)0 : rounded<F>((2.0 * (Ad * c.xb)) * c.inv_t), r.icA, r.imA);
+    return (t9 + t10) + t9;
+}
+template <int TIME_SUM, class F>
+__device__ __forceinline__ F stage_head(const StageConst &c, const Rates<F> &r, double Ed, double Rd) {
+    return time_of<TIME_SUM, F>(rounded<F>(Ed * c.f13), rounded<F>((Rd * c.w13 + Ed * c.va) * c.inv_t) + rounded<F>(Ed * c.ha), r.icL, r.imL);
+}
+template <class F>
+__device__ __forceinline__ F stage_sum(F fix, F att, F comm, F head, F Rd, F Nd, F tovh, F lf) {
+    const F layer = (fix + att) + comm;
+    F tp = Rd * tovh + (Nd * layer + head);
+    if (lf != (F)1) tp = tp * lf;
+    return tp;
+}
+
+// Prompt of one sub-batch of sb requests, in passes of seg tokens (see segmented_prefill); passes of equal
+// length share everything but attention and head.
+template <int TIME_SUM, class F>
+__device__ __forceinline__ F prefill_passes(const StageConst &c, const Rates<F> &r, u32 sb, u32 lin, u32 seg, F Nd, F lf) {
+    F sum = (F)0, fix = (F)0, comm = (F)0;
+    u32 have = 0;
+    double Td = 0.0;
+#pragma unroll 1
+    for (u32 done = 0; done < lin;) {
+        const u32 q = min(seg, lin - done);
+        if (q != have) {
+            Td = (double)sb * (double)q;
+            stage_parts<TIME_SUM, F>(c, r, Td, 1.0, fix, comm);
+            have = q;
+        }
+        done += q;
+        const double seen = (double)done;
+        const F att = stage_attention<TIME_SUM, F>(c, r, Td, Td * seen, (double)sb * seen);
+        const F head = done == lin ? stage_head<TIME_SUM, F>(c, r, (double)sb, 1.0) : (F)0;
+        sum = sum + stage_sum<F>(fix, att, comm, head, (F)1, Nd, r.tovh, lf);
+    }
+    return sum;
+}
+// All prompts of a replica's share of b requests: sub-batches of split, the remainder as one more.
+template <int TIME_SUM, class F>
+__device__ __forceinline__ F prefill_time(const StageConst &c, const Rates<F> &r, u32 split, u32 n_full, u32 rest, u32 lin, u32 seg, F Nd, F lf) {
+    F t = (F)n_full * prefill_passes<TIME_SUM, F>(c, r, split, lin, seg, Nd, lf);
+    if (rest) t = t + prefill_passes<TIME_SUM, F>(c, r, rest, lin, seg, Nd, lf);
+    return t;
+}
+// n decode steps of T = b n tokens over a summed context ctx
+template <int TIME_SUM, class F>
+__device__ __forceinline__ F decode_stage_time(const StageConst &c, const Rates<F> &r, double Td, double ctx, double n, F Nd, F lf) {
+    F fix, comm;
+    stage_parts<TIME_SUM, F>(c, r, Td, n, fix, comm);
+    return stage_sum<F>(fix, stage_attention<TIME_SUM, F>(c, r, Td, ctx, ctx), comm, stage_head<TIME_SUM, F>(c, r, Td, n), rounded<F>(n), Nd, r.tovh, lf);
+}
+
 // Prompt processing of one sub-batch of sb requests in segments of seg tokens (Sec. 3.3.2): one pass
 // per segment, its tokens attending the prompt up to the end of the segment; the LM head runs with
 // the last segment only.  Passes are summed in order from 0.0.
@@ -483,12 +591,31 @@ __device__ __noinline__ double segmented_prefill(const DModel &m, const DRate &r
     return sum;
 }
 
+// The two stage times of one config from the integer table (spaces whose counts the doubles above do not hold).
+template <int TIME_SUM>
+__device__ __noinline__ double2 integer_stage_times(const DModel &m, const DRate &r, u32 tt, u32 b, u32 split, u32 n_full, u32 rest, u32 lin,
+                                                    u32 seg, u32 n, u64 ctx, double Nd, double lf) {
+    double2 o;
+    o.x = (double)n_full * segmented_prefill<TIME_SUM>(m, r, tt, split, lin, seg, Nd, lf);
+    if (rest) o.x = o.x + segmented_prefill<TIME_SUM>(m, r, tt, rest, lin, seg, Nd, lf);
+    o.y = 0.0;
+    if (n > 0) {
+        TaskTab k;
+        const u64 Td = (u64)b * n;
+        build_fixed_tasks(m, tt, Td, Td, n, k);
+        build_attn_tasks(m, tt, Td, ctx, ctx, k);
+        o.y = eval_phase<TIME_SUM>(k, r, Nd, lf);
+    }
+    return o;
+}
+
 // Whole closed-form evaluation of one config, nothing cached (used where configs arrive in
 // arbitrary order; the tiled kernels hoist the table building out of the hardware x framework loop).
 template <int TIME_SUM>
 __device__ __forceinline__ void closed_form_eval(const DSpace &s, const Cfg &c, int tp_model, Metrics &o) {
-    const DModel m = s.models[c.m];
-    const DRate &r = s.rates[c.h * s.n_f + c.f];
+    const DModel &m = s.models[c.m];
+    const u32 hf = c.h * s.n_f + c.f;
+    const DRate &r = s.rates[hf];
     const u32 t = s.tp[c.t], b_all = s.batch[c.b];
     const u32 b = replica_batch(b_all, s.dp[c.t]);   // each of the dp replicas serves its share of the batch
     const uint2 pr = s.pairs[c.l];
@@ -507,38 +634,33 @@ __device__ __forceinline__ void closed_form_eval(const DSpace &s, const Cfg &c, 
     o.status = closed_form_feasibility(m, r, mi, t, b, lin, lout, o.bmax);
     o.seq_used = o.status ? 0u : lin + lout;
     if (o.status) { set_infeasible(o); return; }
-    const u32 tt = tp_model ? 1u : t;
     const double lf = log2_rule_factor(t, tp_model);
     const double Nd = (double)m.N;
-    TaskTab k;
-    double t_pre;
+    // Sec. 3.3.1: sub-batches of split requests, the remainder as one more; equal ones take equal time
+    const u32 split = (r.split == 0 || r.split > b) ? b : r.split;
+    const u32 seg = (r.seg == 0 || r.seg > lin) ? lin : r.seg;
+    u32 n_full = 1, rest = 0;
     u64 n_pass = 1, n_seg = 1;
     if (r.split | r.seg) {
-        // Sec. 3.3.1: sub-batches of split requests, the remainder as one more; equal ones take equal time
-        const u32 split = (r.split == 0 || r.split > b) ? b : r.split;
-        const u32 seg = (r.seg == 0 || r.seg > lin) ? lin : r.seg;
-        const u32 n_full = b / split, rest = b % split;
-        t_pre = (double)n_full * segmented_prefill<TIME_SUM>(m, r, tt, split, lin, seg, Nd, lf);
-        if (rest) t_pre = t_pre + segmented_prefill<TIME_SUM>(m, r, tt, rest, lin, seg, Nd, lf);
+        n_full = b / split; rest = b % split;
         n_seg = (lin + seg - 1) / seg;
         n_pass = (u64)(n_full + (rest != 0)) * n_seg;
-    } else {
-        const u64 Tp = (u64)b * lin;
-        build_fixed_tasks(m, tt, Tp, b, 1, k);
-        build_attn_tasks(m, tt, Tp, Tp * lin, Tp, k);
-        t_pre = eval_phase<TIME_SUM>(k, r, Nd, lf);
     }
     const u32 n = lout - 1;
-    double t_dec = 0.0;
-    if (n > 0) {
-        const u64 Td = (u64)b * n;
-        // step j attends lin + j tokens, of which the cache still holds the kept share
-        const u64 ctx = kept_tokens((u64)b * ((u64)n * lin + ((u64)n * (n + 1)) / 2), r.keep);
-        build_fixed_tasks(m, tt, Td, Td, n, k);
-        build_attn_tasks(m, tt, Td, ctx, ctx, k);
-        t_dec = eval_phase<TIME_SUM>(k, r, Nd, lf);
+    // step j attends lin + j tokens, of which the cache still holds the kept share
+    const u64 ctx = kept_tokens((u64)b * ((u64)n * lin + ((u64)n * (n + 1)) / 2), r.keep);
+    double t_pre, t_dec = 0.0;
+    if (s.exact) {
+        const StageConst &sc = s.stage_consts[(size_t)(tp_model ? s.n_t : c.t) * s.n_m + c.m];
+        const double *q = s.rate10 + (size_t)hf * 10;
+        const Rates<double> rr = {q[0], q[1], q[2], q[3], q[4], q[5], q[6], q[7], q[8], q[9] != 0.0};
+        t_pre = prefill_time<TIME_SUM, double>(sc, rr, split, n_full, rest, lin, seg, Nd, lf);
+        if (n > 0) t_dec = decode_stage_time<TIME_SUM, double>(sc, rr, (double)b * (double)n, (double)(long long)ctx, (double)n, Nd, lf);
+    } else {
+        const double2 tt = integer_stage_times<TIME_SUM>(m, r, tp_model ? 1u : t, b, split, n_full, rest, lin, seg, n, ctx, Nd, lf);
+        t_pre = tt.x; t_dec = tt.y;
     }
-    const u32 ci = (c.h * s.n_f + c.f) * s.n_t + c.t;
+    const u32 ci = hf * s.n_t + c.t;
     closed_form_metrics(t_pre, t_dec, b_all, n, s.cost_hr[ci], s.cost_sec[ci], o, n_pass, n_seg);
 }
 

@@ -89,7 +89,7 @@ __device__ __forceinline__ float segmented_prefill_f(const DModel &m, const Rate
 // closed_form_eval).
 template <int TIME_SUM>
 __device__ __forceinline__ void closed_form_eval_f32(const DSpace &s, const RateF *rates, const Cfg &c, int tp_model, Metrics &o) {
-    const DModel m = s.models[c.m];
+    const DModel &m = s.models[c.m];
     const DRate &r = s.rates[c.h * s.n_f + c.f];
     const RateF rf = rates[c.h * s.n_f + c.f];
     const u32 t = s.tp[c.t], b_all = s.batch[c.b], dp = s.dp[c.t];
@@ -110,15 +110,27 @@ __device__ __forceinline__ void closed_form_eval_f32(const DSpace &s, const Rate
     const u32 split = (r.split == 0 || r.split > b) ? b : r.split;
     const u32 seg = (r.seg == 0 || r.seg > lin) ? lin : r.seg;
     const u32 n_full = b / split, rest = b % split;
-    float t_pre = (float)n_full * segmented_prefill_f<TIME_SUM>(m, rf, t, split, lin, seg, tp_model);
-    if (rest) t_pre = t_pre + segmented_prefill_f<TIME_SUM>(m, rf, t, rest, lin, seg, tp_model);
     const u64 n_seg = (lin + seg - 1) / seg;
     const u32 n = lout - 1;
-    float t_dec = 0.0f;
-    if (n > 0) {
-        const u64 Td = (u64)b * n;
-        const u64 ctx = kept_tokens((u64)b * ((u64)n * lin + ((u64)n * (n + 1)) / 2), r.keep);
-        t_dec = stage_time_f<TIME_SUM>(m, rf, t, Td, Td, ctx, ctx, n, tp_model);
+    const u64 ctx = kept_tokens((u64)b * ((u64)n * lin + ((u64)n * (n + 1)) / 2), r.keep);
+    float t_pre, t_dec = 0.0f;
+    if (s.exact == 2) {
+        // the counts as exact doubles, each rounded to binary32 once (stage_parts)
+        const StageConst &sc = s.stage_consts[(size_t)(tp_model ? s.n_t : c.t) * s.n_m + c.m];
+        const Rates<float> rr = {rf.inv_c[CLS_LINEAR], rf.inv_c[CLS_ATTN], rf.inv_c[CLS_ELEM], rf.inv_m[CLS_LINEAR], rf.inv_m[CLS_ATTN],
+                                 rf.inv_m[CLS_ELEM], rf.inv_comm, rf.clat, rf.tovh, rf.flash != 0};
+        float lf = 1.0f;
+        if (tp_model) lf = (float)(1 + (31 - __clz(t))) / (float)t;
+        const float Nd = (float)m.N;
+        t_pre = prefill_time<TIME_SUM, float>(sc, rr, split, n_full, rest, lin, seg, Nd, lf);
+        if (n > 0) t_dec = decode_stage_time<TIME_SUM, float>(sc, rr, (double)b * (double)n, (double)(long long)ctx, (double)n, Nd, lf);
+    } else {
+        t_pre = (float)n_full * segmented_prefill_f<TIME_SUM>(m, rf, t, split, lin, seg, tp_model);
+        if (rest) t_pre = t_pre + segmented_prefill_f<TIME_SUM>(m, rf, t, rest, lin, seg, tp_model);
+        if (n > 0) {
+            const u64 Td = (u64)b * n;
+            t_dec = stage_time_f<TIME_SUM>(m, rf, t, Td, Td, ctx, ctx, n, tp_model);
+        }
     }
     const float inf = __int_as_float(0x7F800000);
     const float lat = t_pre + t_dec;
