@@ -72,10 +72,8 @@ int space_on_device(guide_space *s, DSpace *out, unsigned **ticket, cudaStream_t
 int trace_on_device(guide_trace *t, DTrace *out, cudaStream_t st);
 
 // closed_form.cu
-struct LineSelect;           // select_sink.cuh: both selections of a combined simulate-and-select call
-bool closed_form_by_lines(const DSpace &s, Range r, const guide_outputs &o);
 int launch_closed_form(const DSpace &s, Range r, int time_model, int tp_model, const guide_outputs &o,
-                       unsigned *ticket, cudaStream_t st, const LineSelect *sel = nullptr);
+                       unsigned *ticket, cudaStream_t st);
 int launch_closed_form_f32(const DSpace &s, Range r, int time_model, int tp_model, const guide_outputs &o, cudaStream_t st);
 // trace_sim.cu
 // What the host knows about the configs the one-lane-per-config kernel would take: per class of max

@@ -67,7 +67,7 @@ __device__ __forceinline__ void line_walk(const DSpace &s, int tp_model, u32 n_c
             if (!__any_sync(0xFFFFFFFFu, any)) continue;
         }
         __syncwarp();                                 // the previous item's reads of the tables are over
-        build_stage_table(mp, tp_model ? 1u : t, b, pr16.x, pr16.y - 1, lane >> 4, (lane >> 4) ? &tb_dec : &tb_pre, lane & 15);
+        build_stage_table(s.exact ? s.stage_consts + (size_t)(tp_model ? s.n_t : tpos) * s.n_m + mpos : nullptr, mp, tp_model ? 1u : t, b, pr16.x, pr16.y - 1, lane >> 4, (lane >> 4) ? &tb_dec : &tb_pre, lane & 15);
         __syncwarp();
         // the four points this lane evaluates: 4q + u
         u64 S4[4];

@@ -29,11 +29,12 @@ __device__ __forceinline__ void put_stage(Tab &tb, u32 u, const TaskTab &k) {
 }
 
 // One stage table of one point, written to shared memory: stage 0 is the prompt pass, stage 1 the
-// aggregated decode steps.  Eight lanes of a warp call it together (four points x two stages): the
-// instruction stream is the same for both stages, only the token counts differ.  Kept out of line:
-// it runs once per work item and needs far more registers than the walk around it.
+// aggregated decode steps.  Lanes of a warp call it together (points x stages): the instruction stream is
+// the same for both stages, only the token counts differ.  From the factors of the (model, TP degree)
+// when the space allows it (stage_parts in model.cuh: the same bits for a fifth of the instructions),
+// else (sc null) from the integer table, out of line.
 template <class Tab>
-static __device__ __noinline__ void build_stage_table(const DModel *mp, u32 tt, u32 b, u32 lin, u32 n, u32 stage, Tab *tb, u32 u) {
+static __device__ __noinline__ void build_stage_table_int(const DModel *mp, u32 tt, u32 b, u32 lin, u32 n, u32 stage, Tab *tb, u32 u) {
     const DModel m = *mp;
     TaskTab k;
     const u32 nn = n > 0 ? n : 1;          // a decode table is built either way; unused when n == 0
@@ -43,6 +44,30 @@ static __device__ __noinline__ void build_stage_table(const DModel *mp, u32 tt, 
     build_fixed_tasks(m, tt, T, stage ? Td : (u64)b, stage ? (u64)nn : 1ull, k);
     build_attn_tasks(m, tt, T, stage ? ctx : Tp * lin, stage ? ctx : Tp, k);
     put_stage(*tb, u, k);
+}
+template <class Tab>
+static __device__ __forceinline__ void build_stage_table(const StageConst *sc, const DModel *mp, u32 tt, u32 b, u32 lin, u32 n, u32 stage,
+                                                         Tab *tb, u32 u) {
+    if (!sc) { build_stage_table_int(mp, tt, b, lin, n, stage, tb, u); return; }
+    const StageConst &c = *sc;
+    const double bd = (double)b, lind = (double)lin, nd = (double)(n > 0 ? n : 1);
+    const double T = bd * (stage ? nd : lind), E = stage ? T : bd, R = stage ? nd : 1.0;
+    const double C = stage ? bd * (nd * lind + (nd * (nd + 1.0)) * 0.5) : T, A = stage ? C : T * lind;
+    const double tha = T * c.ha;
+    Tab &t = *tb;
+    t[E_F1][u] = T * c.f1; t[E_B1][u] = T * c.b1;
+    t[E_F2][u] = T * c.f2; t[E_B2][u] = (R * c.w2 + tha) * c.inv_t + tha;
+    t[E_F3][u] = T * c.f3; t[E_B3][u] = 2.0 * ((R * c.w3 + T * c.dk) * c.inv_t + tha);
+    t[E_F5][u] = T * c.f5; t[E_B5][u] = T * c.b5;
+    const double up = (R * c.w6 + T * c.ia) * c.inv_t + tha;
+    t[E_F6][u] = T * c.f6; t[E_B6][u] = c.mult6 * up;
+    t[E_F7][u] = T * c.f7; t[E_B7][u] = T * c.b7;
+    t[E_F8][u] = T * c.f8; t[E_B8][u] = up;
+    const double by = tha + C * c.kv, X = A * c.xb;
+    t[E_F9][u] = A * c.f9; t[E_B9][u] = by * c.inv_t; t[E_B9X][u] = (by + X) * c.inv_t;
+    t[E_F10][u] = A * c.f10; t[E_B10X][u] = (2.0 * X) * c.inv_t;
+    t[E_F13][u] = E * c.f13; t[E_B13][u] = (R * c.w13 + E * c.va) * c.inv_t + E * c.ha;
+    t[E_HOPS][u] = R * c.hops; t[E_CBYTES][u] = T * c.cb; t[E_RD][u] = R;
 }
 
 // rates of one pair in registers (a row of rate10)
@@ -106,6 +131,7 @@ __device__ __forceinline__ void model_walk(const DSpace &s, int tp_model, u32 n_
         const u32 tpos = tl / s.n_l, lpos = tl % s.n_l;
         const DModel *mp = s.models + mpos;
         const u32 t = s.tp[tpos], b_all = s.batch[bpos];
+        const StageConst *sc = s.exact ? s.stage_consts + (size_t)(tp_model ? s.n_t : tpos) * s.n_m + mpos : nullptr;
         const u32 b = replica_batch(b_all, s.dp[tpos]);
         const u32 nh = mp->nh, nkv = mp->nkv;
         if ((nh & (t - 1)) != 0 || (nkv & (t - 1)) != 0) continue;          // the foursome shares its TP degree: nothing fits
@@ -128,7 +154,7 @@ __device__ __forceinline__ void model_walk(const DSpace &s, int tp_model, u32 n_
         }
         if (!__any_sync(0xFFFFFFFFu, any)) continue;
         __syncwarp();                                 // the previous item's reads of the tables are over
-        if (h < 2) build_stage_table(mp, tp_model ? 1u : t, b, lin, n, h, h ? &tb_dec : &tb_pre, u);   // lanes 0-3: prompt stage of point u; 4-7: decode stage
+        if (h < 2) build_stage_table(sc, mp, tp_model ? 1u : t, b, lin, n, h, h ? &tb_dec : &tb_pre, u);   // lanes 0-3: prompt stage of point u; 4-7: decode stage
         __syncwarp();
         const u64 j0 = (u64)mpos * n_hf * stride_hf + (u64)bpos * n_tl + tl;
         const double lf = log2_rule_factor(t, tp_model);

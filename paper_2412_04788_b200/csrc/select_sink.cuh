@@ -1,8 +1,6 @@
-// What a kernel that has just evaluated a config needs in order to decide whether a selection can
-// still want it: the sampled bound of a top-k call, the dominating points ("killers") of a Pareto
-// call, and the lists the survivors go to.  Shared by the streaming selection kernels
-// (select_stream.cu) and by the closed-form line kernel when it runs as the filter pass of a
-// combined simulate-and-select call (closed_form.cu).
+// What a kernel needs in order to decide whether a selection can still want a config: the sampled bound
+// of a top-k call, the dominating points ("killers") of a Pareto call, and the lists the survivors go
+// to.  Shared by the one-launch selection (select_coop.cu) and the fused one (select_stream.cu).
 #pragma once
 #include "select.cuh"
 
@@ -62,12 +60,5 @@ struct KillerSet {
 __device__ __forceinline__ bool meets(const Cons &c, double latency, double ttft, double thr, double cost_hr) {
     return ttft <= c.max_ttft && latency <= c.max_latency && cost_hr <= c.max_cost_hr && thr >= c.min_thr;
 }
-
-// Both selections of a combined call, as the line kernel sees them: constraints and metric choice,
-// the workspace headers (bound pair, killer count, survivor counters) and the lists.
-struct LineSelect {
-    Cons ct; int key; u32 *header_t; KI *cand;
-    Cons cp; int xm, ym; u32 *header_p; const P2 *killers; P3 *surv;
-};
 
 }  // namespace guide

@@ -720,10 +720,10 @@ static bool cooperative_ok() {
 // the length pair.
 template <int TIME_SUM>
 __global__ void __launch_bounds__(SEL_THREADS) k_fused_sample(DSpace s, int tp_model, Sample sm, Cons c, int m0, int m1,
-                                                              u64 *row_base, uint8_t *pass, double *a0, double *a1, int beside) {
+                                                              u64 *row_base, uint8_t *pass, double *a0, double *a1) {
     grid_dep_launch();
     const u64 slot = (u64)blockIdx.x * (SEL_THREADS / ROW) + threadIdx.x / ROW;
-    if (slot >= sm.n_slots) { if (beside) grid_dep_wait(); return; }
+    if (slot >= sm.n_slots) return;
     const u32 l = threadIdx.x % ROW;
     const u64 first = sm.row(slot) * ROW;
     Metrics m;
@@ -735,9 +735,6 @@ __global__ void __launch_bounds__(SEL_THREADS) k_fused_sample(DSpace s, int tp_m
     a0[q] = a;
     if (m1 >= 0) a1[q] = b;
     if (l == 0) row_base[slot] = first;
-    // Launched beside its predecessor in the stream (another sample), the grid must not be complete
-    // before that one is: whatever follows in the stream waits for this grid only.
-    if (beside) grid_dep_wait();
 }
 
 // Filter pass of the fused top-k: the model walk, with the configs that fit, meet the constraints
@@ -814,22 +811,13 @@ static FusedScratch fused_scratch(unsigned char *base) {
 // sample rows of the space -> compact scratch; returns the walk over the scratch (row c of it is slot c)
 template <int TIME_SUM>
 static int fused_sample(const DSpace &s, int tp_model, const Cons &c, int m0, int m1, u32 want_rows, u32 max_r, const FusedScratch &f,
-                        Sample *compact, cudaStream_t st, int phase) {
-    const bool beside = phase == FUSED_SAMPLE_BESIDE;
+                        Sample *compact, cudaStream_t st) {
     const u64 total = (u64)s.n_m * s.n_h * s.n_f * s.n_b * s.n_t * s.n_l;
     Sample sm = make_sample(total / ROW, want_rows, max_r);
     sm.n_slots = std::min<u64>(sm.n_groups, FUSED_ROWS);
     const u32 grid = (u32)((sm.n_slots + SEL_THREADS / ROW - 1) / (SEL_THREADS / ROW));
-    if (phase == FUSED_BOUND_ONLY) {
-        // the rows were evaluated by an earlier call with the same arguments
-    } else if (beside) {
-        // the stream's previous kernel is the other selection's sample, which lets its dependents start at once
-        GUIDE_CUDA(launch_dependent(k_fused_sample<TIME_SUM>, grid, SEL_THREADS, 0, st, s, tp_model, sm, c, m0, m1, f.row_base, f.pass,
-                                    f.a0, f.a1, 1));
-    } else {
-        k_fused_sample<TIME_SUM><<<grid, SEL_THREADS, 0, st>>>(s, tp_model, sm, c, m0, m1, f.row_base, f.pass, f.a0, f.a1, 0);
-        GUIDE_CUDA(cudaGetLastError());
-    }
+    k_fused_sample<TIME_SUM><<<grid, SEL_THREADS, 0, st>>>(s, tp_model, sm, c, m0, m1, f.row_base, f.pass, f.a0, f.a1);
+    GUIDE_CUDA(cudaGetLastError());
     compact->n_groups = sm.n_slots; compact->n_slots = sm.n_slots; compact->mul = 1; compact->r = 1;
     return GUIDE_OK;
 }
@@ -846,28 +834,20 @@ static cudaError_t launch_model_dependent_cfg(cudaLaunchConfig_t *cfg, cudaLaunc
 
 template <int TIME_SUM>
 static int topk_fused_t(const DSpace &s, int tp_model, const guide_constraints &gc, int key, u32 k, u32 *header,
-                        unsigned char *region, unsigned *ticket, u64 *idx_out, double *key_out, u32 *count_out, cudaStream_t st,
-                        int phase) {
+                        unsigned char *region, unsigned *ticket, u64 *idx_out, double *key_out, u32 *count_out, cudaStream_t st) {
     const Cons c = make_cons(gc);
     const FusedScratch f = fused_scratch(region + TK_OFF_FUSED);
     ulonglong2 *minima = reinterpret_cast<ulonglong2 *>(region);
     ulonglong2 *spairs = reinterpret_cast<ulonglong2 *>(region + TK_OFF_SKEYS);
     KI *cand = reinterpret_cast<KI *>(region + TK_OFF_CAND);
     const size_t smem = (size_t)TK_CAND_SMEM * sizeof(KI);
-    if (phase == FUSED_RANK) {
-        GUIDE_CUDA(cudaFuncSetAttribute(k_topk_rank, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        GUIDE_CUDA(launch_dependent(k_topk_rank, num_sms(), SEL_THREADS, smem, st, header, (const KI *)cand, k,
-                                    key == GUIDE_THROUGHPUT ? 1 : 0, idx_out, key_out, count_out));
-        return GUIDE_OK;
-    }
-    if (phase == FUSED_ALL) GUIDE_CUDA(cudaMemsetAsync(ticket, 0, 4, st));           // the model walk's work counter
+    GUIDE_CUDA(cudaMemsetAsync(ticket, 0, 4, st));           // the model walk's work counter
     Sample sm;
     // Half the rows of the materialised path's sample: here a row costs an evaluation of 64 configs, not a
     // read, and the filter pass behind it tolerates the wider bound (workload 5: 3,542 survivors instead
     // of 2,465, the call 10 us shorter).
-    int rc = fused_sample<TIME_SUM>(s, tp_model, c, key, -1, TK_SAMPLE_ROWS / 2, TK_SAMPLE_MAX_R * 2, f, &sm, st, phase);
+    int rc = fused_sample<TIME_SUM>(s, tp_model, c, key, -1, TK_SAMPLE_ROWS / 2, TK_SAMPLE_MAX_R * 2, f, &sm, st);
     if (rc) return rc;
-    if (phase == FUSED_SAMPLE || phase == FUSED_SAMPLE_BESIDE) return GUIDE_OK;
     Src<1> src;
     src.a[0] = Arr{f.a0, 0.0, 0, 0};                         // pick_metric has negated the throughput already
     src.status = f.pass;
@@ -886,7 +866,6 @@ static int topk_fused_t(const DSpace &s, int tp_model, const guide_constraints &
         GUIDE_CUDA(cudaGetLastError());
         GUIDE_CUDA(launch_dependent(k_topk_refine<1>, TK_SAMPLE_BLOCKS, SEL_THREADS, 0, st, src, sm, (u64)0, k, header, spairs));
     }
-    if (phase == FUSED_BOUND || phase == FUSED_BOUND_ONLY) return GUIDE_OK;
     const u32 n_chunks = (s.n_h * s.n_f + MODEL_CHUNK - 1) / MODEL_CHUNK;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at[1];
@@ -899,23 +878,14 @@ static int topk_fused_t(const DSpace &s, int tp_model, const guide_constraints &
 }
 
 int launch_topk_fused(const DSpace &s, int time_model, int tp_model, const guide_constraints &c, int key, u32 k, u32 *header,
-                      unsigned char *region, unsigned *ticket, u64 *idx_out, double *key_out, u32 *count_out, cudaStream_t st,
-                      int phase) {
-    return time_model ? topk_fused_t<1>(s, tp_model, c, key, k, header, region, ticket, idx_out, key_out, count_out, st, phase)
-                      : topk_fused_t<0>(s, tp_model, c, key, k, header, region, ticket, idx_out, key_out, count_out, st, phase);
-}
-
-// Where the filter pass of a combined call finds the lists of the two selections' workspaces.
-void fused_lists(unsigned char *topk_region, unsigned char *pareto_region, LineSelect *sel) {
-    sel->cand = reinterpret_cast<KI *>(topk_region + TK_OFF_CAND);
-    sel->killers = reinterpret_cast<const P2 *>(pareto_region + PA_OFF_KILLERS);
-    sel->surv = reinterpret_cast<P3 *>(pareto_region + PA_OFF_SURV);
+                      unsigned char *region, unsigned *ticket, u64 *idx_out, double *key_out, u32 *count_out, cudaStream_t st) {
+    return time_model ? topk_fused_t<1>(s, tp_model, c, key, k, header, region, ticket, idx_out, key_out, count_out, st)
+                      : topk_fused_t<0>(s, tp_model, c, key, k, header, region, ticket, idx_out, key_out, count_out, st);
 }
 
 template <int TIME_SUM>
 static int pareto_fused_t(const DSpace &s, int tp_model, const guide_constraints &gc, int xm, int ym, u32 *header,
-                          unsigned char *region, unsigned *ticket, u64 *idx_out, u32 cap, u32 *count_out, cudaStream_t st,
-                          int phase) {
+                          unsigned char *region, unsigned *ticket, u64 *idx_out, u32 cap, u32 *count_out, cudaStream_t st) {
     const Cons c = make_cons(gc);
     const FusedScratch f = fused_scratch(region + PA_OFF_FUSED);
     P2 *local = reinterpret_cast<P2 *>(region);
@@ -924,17 +894,10 @@ static int pareto_fused_t(const DSpace &s, int tp_model, const guide_constraints
     P3 *surv = reinterpret_cast<P3 *>(region + PA_OFF_SURV);
     KI *front = reinterpret_cast<KI *>(region + PA_OFF_FRONT);
     const size_t smem = (size_t)PA_SURV_CAP * 16;
-    if (phase == FUSED_RANK) {
-        GUIDE_CUDA(cudaFuncSetAttribute(k_pareto_rank, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        GUIDE_CUDA(launch_dependent(k_pareto_rank, num_sms(), SEL_THREADS, smem, st, header, (const P3 *)surv, front, idx_out, cap,
-                                    count_out));
-        return GUIDE_OK;
-    }
-    if (phase == FUSED_ALL) GUIDE_CUDA(cudaMemsetAsync(ticket, 0, 4, st));
+    GUIDE_CUDA(cudaMemsetAsync(ticket, 0, 4, st));
     Sample sm;
-    int rc = fused_sample<TIME_SUM>(s, tp_model, c, xm, ym, PA_SAMPLE_ROWS, 1u << 20, f, &sm, st, phase);
+    int rc = fused_sample<TIME_SUM>(s, tp_model, c, xm, ym, PA_SAMPLE_ROWS, 1u << 20, f, &sm, st);
     if (rc) return rc;
-    if (phase == FUSED_SAMPLE || phase == FUSED_SAMPLE_BESIDE) return GUIDE_OK;
     Src<2> src;
     src.a[0] = Arr{f.a0, 0.0, 0, 0};
     src.a[1] = Arr{f.a1, 0.0, 0, 0};
@@ -942,7 +905,6 @@ static int pareto_fused_t(const DSpace &s, int tp_model, const guide_constraints
     src.row_base = f.row_base;
     k_pareto_sample<2><<<PA_SAMPLE_BLOCKS, SEL_THREADS, 0, st>>>(src, sm, header, local, local_n, killers);
     GUIDE_CUDA(cudaGetLastError());
-    if (phase == FUSED_BOUND || phase == FUSED_BOUND_ONLY) return GUIDE_OK;
     const u32 n_chunks = (s.n_h * s.n_f + MODEL_CHUNK - 1) / MODEL_CHUNK;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at[1];
@@ -956,10 +918,9 @@ static int pareto_fused_t(const DSpace &s, int tp_model, const guide_constraints
 }
 
 int launch_pareto_fused(const DSpace &s, int time_model, int tp_model, const guide_constraints &c, int xm, int ym, u32 *header,
-                        unsigned char *region, unsigned *ticket, u64 *idx_out, u32 cap, u32 *count_out, cudaStream_t st,
-                        int phase) {
-    return time_model ? pareto_fused_t<1>(s, tp_model, c, xm, ym, header, region, ticket, idx_out, cap, count_out, st, phase)
-                      : pareto_fused_t<0>(s, tp_model, c, xm, ym, header, region, ticket, idx_out, cap, count_out, st, phase);
+                        unsigned char *region, unsigned *ticket, u64 *idx_out, u32 cap, u32 *count_out, cudaStream_t st) {
+    return time_model ? pareto_fused_t<1>(s, tp_model, c, xm, ym, header, region, ticket, idx_out, cap, count_out, st)
+                      : pareto_fused_t<0>(s, tp_model, c, xm, ym, header, region, ticket, idx_out, cap, count_out, st);
 }
 
 }  // namespace guide
