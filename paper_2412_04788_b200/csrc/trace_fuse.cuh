@@ -71,6 +71,14 @@ __device__ __forceinline__ u64 fuse_warp_scan(u64 v, u32 lane) {
 // around this call keeps its own copies in registers.
 struct FuseTrace { const double *arrival; const u32 *in_len, *out_len; };
 
+// attention time of nrun residents' next decode token from the integer table (configs whose counts the doubles do not hold)
+template <int TIME_SUM>
+__device__ __noinline__ double fuse_attn_int(const DModel *m, const DRate *rt, u32 tt, u32 nrun, u64 ctx) {
+    TaskTab ka;
+    build_attn_tasks(*m, tt, nrun, ctx, ctx, ka);
+    return eval_attn<TIME_SUM>(ka, *rt);
+}
+
 template <int TIME_SUM>
 __device__ __noinline__ u32 fuse_schedule(const DModel *mp, const DRate *rp, const double *arrival, const u32 *in_len,
                                           const u32 *out_len, u32 n, u32 tt, u32 b, u32 Lin, u32 Lout, u64 blocks_total,
@@ -114,7 +122,7 @@ __device__ __noinline__ u32 fuse_schedule(const DModel *mp, const DRate *rp, con
         const double t10 = task_time<TIME_SUM>(Ad * sc.f10, rt.flash ? 0.0 : (2.0 * (Ad * sc.xb)) * sc.inv_t, icA, imA);
         return (t9 + t10) + t9;
     };
-    double clock = 0.0, dec_time = 0.0;
+    double clock = 0.0, dec_time = 0.0;              // dec_time: in the upper half of the lanes
     u64 dec_tok = 0, n_iters = 0, n_req_iters = 0, free_blocks = blocks_total;
     u32 next = 0, high_water = 0, nrun = 0, st = 0;
     u32 n_pre = 0;                                   // residents still in their prompt
@@ -245,7 +253,6 @@ __device__ __noinline__ u32 fuse_schedule(const DModel *mp, const DRate *rp, con
             const u64 cap_left = max_iters - n_iters;
             const bool room = nrun < b;
             const u32 steps_max = (u32)min((u64)min_rem, cap_left);
-            const u32 lmod = modb(lane);
             // The terms of a decode iteration that depend on the resident count only are kept for a window
             // of 32 neighbouring counts (worked out one per lane): the count moves by one or two per event.
             if (nrun - dw0 >= 32u) {
@@ -260,87 +267,108 @@ __device__ __noinline__ u32 fuse_schedule(const DModel *mp, const DRate *rp, con
                 __syncwarp();
             }
             const double d_fix = sl.dterm[nrun - dw0][0], d_comm = sl.dterm[nrun - dw0][1], d_head = sl.dterm[nrun - dw0][2];
-            u32 it = 0, off = 0;                                   // off = it mod block size
             // The iterations of the run depend on one another through the clock only: the lanes work out
-            // the times of 32 consecutive ones at once (summed context ctx_i + k * nrun), a prefix sum
-            // over the histogram bins tells which of them finds its blocks, and the clock then advances
-            // one iteration after the other, in order, watching for the arrival of the queue head.
-            for (;;) {
-                const u32 nb = min(32u, steps_max - it);
-                const u64 ctx_k = ctx_i + (u64)lane * nrun;
+            // the times of 32 consecutive ones at once (summed context ctx_i + k * nrun), and the clock then
+            // advances one iteration after the other, in order, half of the lanes carrying it and half the
+            // decode time; a full batch is one straight block with the next one's times in its shadow (as
+            // in k_trace_sim).
+            auto time_of_lane = [&](u32 first_it) {
+                const u64 ctx_k = ctx_i + (u64)(first_it + lane) * nrun;
                 double s_att;
                 if (sc_ok) {
                     const double cd = (double)(long long)ctx_k;
                     s_att = attn_d((double)nrun, cd, cd);
                 } else {
-                    TaskTab ka;
-                    build_attn_tasks(m, tt, nrun, ctx_k, ctx_k, ka);
-                    s_att = eval_attn<TIME_SUM>(ka, rt);
+                    s_att = fuse_attn_int<TIME_SUM>(mp, rp, tt, nrun, ctx_k);
                 }
-                const double t_k = combine_phase(d_fix, s_att, d_comm, d_head, 1.0, Nd, rt.tovh, lf);
-                u32 need_k = 0;                                    // residents whose last block is full before lane's iteration
-                if (lane < nb) {
-                    const u32 o = off + lmod >= blk ? off + lmod - blk : off + lmod;
-                    need_k = sl.hist[o == 0 ? 0 : blk - o];
+                return combine_phase(d_fix, s_att, d_comm, d_head, 1.0, Nd, rt.tovh, lf);
+            };
+            // residents whose last block is full before iteration j of the run, and blocks taken by the first j
+            auto bin = [&](u32 j) { const u32 o = modb(j); return o == 0 ? 0u : blk - o; };
+            auto taken = [&](u32 j) -> u64 {
+                const u32 q = divb(j), rest = j - q * blk;
+                u32 v = 0;
+                if (lane < rest) v = sl.hist[bin(lane)];
+                if (lane + 32 < rest) v += sl.hist[bin(lane + 32)];
+                return (u64)q * nrun + fuse_warp_sum32(v);
+            };
+            const u64 free0 = free_blocks;
+            double acc = lane < 16 ? clock : dec_time;
+            double t_k = 0.0;
+            bool have = false;                                     // t_k was worked out with the batch before
+            u32 it = 0;
+            for (;;) {
+                if (!have) t_k = time_of_lane(it);
+                have = false;
+                const u32 nb = min(32u, steps_max - it);
+                u32 can = nb, watch = room ? 0xFFFFFFFFu : 0u, short_at = 0;
+                // blocks cover the batch and the queue head's need whatever their spread over the residents, as a
+                // rule (each resident takes one every blk iterations); else a prefix sum over the histogram bins tells
+                if ((u64)nrun * divb(it + nb + blk - 1) + (room ? need_next : 0u) > free0) {
+                    const u64 free_it = it ? free0 - taken(it) : free0;
+                    const u32 need_k = lane < nb ? sl.hist[bin(it + lane)] : 0;
+                    u32 incl = need_k;
+                    #pragma unroll
+                    for (int d = 1; d < 32; d <<= 1) {
+                        const u32 up = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+                        if (lane >= (u32)d) incl += up;
+                    }
+                    // free blocks before lane's iteration takes its own (meaningful up to the first shortage)
+                    const u64 free_k = free_it - (incl - need_k);
+                    short_at = __ballot_sync(0xFFFFFFFFu, lane < nb && need_k > free_k);   // eviction: the general path below
+                    if (short_at) can = (u32)__ffs(short_at) - 1;             // iterations that find their blocks
+                    if (can == 0) break;
+                    watch = __ballot_sync(0xFFFFFFFFu, room && need_next <= free_k - need_k);
                 }
-                u32 incl = need_k;
-                #pragma unroll
-                for (int d = 1; d < 32; d <<= 1) {
-                    const u32 up = __shfl_up_sync(0xFFFFFFFFu, incl, d);
-                    if (lane >= (u32)d) incl += up;
-                }
-                // free blocks before lane's iteration takes its own (meaningful up to the first shortage)
-                const u64 free_k = free_blocks - (incl - need_k);
-                const u32 short_at = __ballot_sync(0xFFFFFFFFu, lane < nb && need_k > free_k);   // eviction: the general path below
-                const u32 can = short_at ? (u32)__ffs(short_at) - 1 : nb;     // iterations that find their blocks
-                if (can == 0) break;
-                const u32 last = can - 1;
                 const bool counted_out = it + can == steps_max;    // a completion or the cap follows the last one
-                const u32 watch = __ballot_sync(0xFFFFFFFFu, room && need_next <= free_k - need_k) & (0xFFFFFFFFu >> (31 - last));
-                sl.tbuf[lane] = t_k;
                 __syncwarp();
-                // the clock, one iteration after the other: four per trip, the arrival tests of a trip taken together
-                u32 k = 0;
+                sl.tbuf[lane] = lane < can ? t_k : 0.0;            // + 0.0 changes no sum
+                __syncwarp();
+                if (can == 32) {
+                    const double t_next = time_of_lane(it + 32);
+                    double sum = acc;
+                    #pragma unroll
+                    for (u32 k = 0; k < 32; k += 2) {
+                        const double2 v = *(const double2 *)&sl.tbuf[k];
+                        sum = sum + v.x;
+                        sum = sum + v.y;
+                    }
+                    if (watch == 0 || !__any_sync(0xFFFFFFFFu, lane < 16 && arr_next <= sum)) {
+                        acc = sum; it += 32; t_k = t_next; have = true;
+                        if (counted_out || short_at) break;
+                        continue;
+                    }
+                }
+                // the others, sixteen iterations at a time: lane k of a half adds up the times of the first k + 1
+                // only, in order, so that every clock of the sixteen is there at once
+                u32 ran = 0;
                 bool arrived = false;
-                const u32 cnt = last + 1;
-                double2 va = *(const double2 *)&sl.tbuf[0], vb = *(const double2 *)&sl.tbuf[2];
-                while (k + 4 <= cnt) {
-                    const double2 na = *(const double2 *)&sl.tbuf[(k + 4) & 31], nb2 = *(const double2 *)&sl.tbuf[(k + 6) & 31];
-                    const double c1 = clock + va.x, c2 = c1 + va.y, c3 = c2 + vb.x, c4 = c3 + vb.y;
-                    const double d1 = dec_time + va.x, d2 = d1 + va.y, d3 = d2 + vb.x, d4 = d3 + vb.y;
-                    const u32 wbits = (watch >> k) & 15u;
-                    u32 hit = 0;
-                    if (wbits)
-                        hit = ((u32)(arr_next <= c1) | ((u32)(arr_next <= c2) << 1) | ((u32)(arr_next <= c3) << 2) |
-                               ((u32)(arr_next <= c4) << 3)) & wbits;
-                    if (hit) {                                             // the queue head can come in after one of the four
-                        const u32 f = (u32)__ffs(hit) - 1;
-                        clock = f == 0 ? c1 : f == 1 ? c2 : f == 2 ? c3 : c4;
-                        dec_time = f == 0 ? d1 : f == 1 ? d2 : f == 2 ? d3 : d4;
-                        k += f;
-                        arrived = true;
-                        break;
+                const u32 hl = lane & 15;
+                #pragma unroll 1
+                for (u32 q = 0; q < can && !arrived; q += 16) {
+                    const u32 mq = min(16u, can - q);
+                    double sum = acc;
+                    #pragma unroll
+                    for (u32 k = 0; k < 16; k += 2) {
+                        if (k == 2 && mq <= 2) break;
+                        if (k == 4 && mq <= 4) break;
+                        if (k == 8 && mq <= 8) break;
+                        const double2 v = *(const double2 *)&sl.tbuf[q + k];
+                        if (k <= hl) sum = sum + v.x;
+                        if (k + 1 <= hl) sum = sum + v.y;
                     }
-                    clock = c4; dec_time = d4;
-                    va = na; vb = nb2;
-                    k += 4;
+                    // the queue head can come in after the first iteration that ends past its arrival, if it may
+                    const u32 in = __ballot_sync(0xFFFFFFFFu, lane < mq && ((watch >> (q + hl)) & 1u) && arr_next <= sum);
+                    arrived = in != 0;
+                    const u32 last = arrived ? (u32)__ffs(in) - 1 : mq - 1;
+                    acc = __shfl_sync(0xFFFFFFFFu, sum, (lane & 16) + last);
+                    ran = q + last + 1;
                 }
-                if (!arrived) {
-                    for (; k < cnt; k++) {
-                        const double v = sl.tbuf[k];
-                        clock = clock + v;
-                        dec_time = dec_time + v;
-                        if (((watch >> k) & 1u) && arr_next <= clock) { arrived = true; break; }
-                    }
-                    if (!arrived) k = last;
-                }
-                free_blocks -= __shfl_sync(0xFFFFFFFFu, incl, k);
-                it += k + 1;
-                ctx_i += (u64)(k + 1) * nrun;
-                { const u32 adv = modb(k + 1); off = off + adv >= blk ? off + adv - blk : off + adv; }
-                __syncwarp();
+                it += ran;
                 if (arrived || counted_out || short_at) break;
             }
+            clock = __shfl_sync(0xFFFFFFFFu, acc, 0); dec_time = acc;
+            if (it > 0) free_blocks = free0 - taken(it);
             if (it > 0) {
                 for (u32 base = 0; base < nrun; base += 32) {
                     const u32 k = base + lane;
@@ -498,6 +526,7 @@ __device__ __noinline__ u32 fuse_schedule(const DModel *mp, const DRate *rp, con
         if (any_done) retire();
     }
     __syncwarp();
+    dec_time = __shfl_sync(0xFFFFFFFFu, dec_time, 16);
     if (lane == 0) {
         sl.res.clock = clock; sl.res.dec_time = dec_time; sl.res.dec_tok = dec_tok; sl.res.n_iters = n_iters;
         sl.res.n_req_iters = n_req_iters;

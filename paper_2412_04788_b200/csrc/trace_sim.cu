@@ -618,49 +618,34 @@ k_trace_sim(DSpace s, DTrace tr, Range r, int tp_model, u64 max_iters_opt, guide
                     const u32 steps_max = (u32)min((u64)min_rem, cap_left);
                     const u32 fb0 = (u32)min(free_blocks, (u64)0xFFFFFFFFu);
                     const u32 hidx0 = Dmod + 1 == blk ? 0 : blk - (Dmod + 1);     // histogram bin of those who need a block before the second iteration
-                    // the bin of those who need one before iteration j + 2, and the blocks taken before the first j of those
-                    auto bin = [&](u32 j) { const u32 o = modb(j); return hidx0 >= o ? hidx0 - o : hidx0 + blk - o; };
-                    auto taken = [&](u32 j) {
-                        if (blk == 1) return j * nrun;
-                        const u32 q = divb(j), rest = j - q * blk;
-                        u32 v = 0;
-                        if (lane < rest) v = sl.hist[bin(lane)];
-                        if (lane + 32 < rest) v += sl.hist[bin(lane + 32)];
-                        return q * nrun + __reduce_add_sync(0xFFFFFFFFu, v);
-                    };
+                    auto bin = [&](u32 j) { const u32 o = modb(j); return hidx0 >= o ? hidx0 - o : hidx0 + blk - o; };   // ... iteration j + 2
                     const bool room = nrun < b;
                     const double nd = dc_nd, cd0 = csum_d;
                     double ctx_k = cd0 + nd * (double)(lane + 1);
                     double t_k = decode_time<TIME_SUM>(ctx_k, c_f9, dc_tha, c_kvx, c_f10, c_b10, icA, imA, dc_fix, dc_comm, dc_head, Nd, rt.tovh, lf);
                     double acc = lane < 16 ? clock : dec_time;        // half of the lanes carry the clock, half the decode time: one addition for both
                     u32 it = 0;
-                    u32 fb = fb0, fb_it = 0;                          // blocks free after the first fb_it iterations (and what they ask for)
-                    u32 used = 0xFFFFFFFFu;                           // blocks taken by the whole run, once known
+                    u32 fb = fb0;                                     // blocks free at the start of the batch
+                    u32 used = 0;                                     // blocks taken by the whole run
                     for (;;) {
                         const u32 nb = min(32u, steps_max - it);
-                        u32 need_k = 0, total = 0;                    // blocks asked for after lane's iteration of the batch, and after all of them
-                        bool counted = false;
                         u32 cnt = nb, watch = room ? 0xFFFFFFFFu : 0u;
                         bool stop = it + nb == steps_max;             // a completion or the cap follows the batch
-                        // Blocks usually cover the batch and the queue head's need whatever their spread over the
-                        // residents (each takes one every blk iterations); then no count is needed.
-                        if ((u64)nrun * divb(it + nb + blk - 1) + (room ? need_next : 0u) > fb0) {
-                            if (fb_it != it) fb = fb0 - taken(it);
-                            counted = true;
-                            if (lane < nb) need_k = blk == 1 ? nrun : sl.hist[bin(it + lane)];
-                            total = __reduce_add_sync(0xFFFFFFFFu, need_k);
-                            if ((u64)total + (room ? need_next : 0u) > fb) {      // short somewhere, or the queue head may have to wait
-                                u32 incl = need_k;
-                                #pragma unroll
-                                for (int d = 1; d < 32; d <<= 1) {
-                                    const u32 up = __shfl_up_sync(0xFFFFFFFFu, incl, d);
-                                    if (lane >= (u32)d) incl += up;
-                                }
-                                const u32 fb_k = fb - (incl - need_k);            // wraps only behind a lane that already stops
-                                const u32 stops = __ballot_sync(0xFFFFFFFFu, lane < nb && need_k > fb_k);
-                                if (stops) { cnt = (u32)__ffs(stops); stop = true; }     // an eviction follows that iteration
-                                watch = __ballot_sync(0xFFFFFFFFu, room && need_next <= fb_k);
+                        // blocks asked for after lane's iteration of the batch, and after all of them
+                        u32 need_k = 0;
+                        if (lane < nb) need_k = blk == 1 ? nrun : sl.hist[bin(it + lane)];
+                        const u32 total = __reduce_add_sync(0xFFFFFFFFu, need_k);
+                        if ((u64)total + (room ? need_next : 0u) > fb) {          // short somewhere, or the queue head may have to wait
+                            u32 incl = need_k;
+                            #pragma unroll
+                            for (int d = 1; d < 32; d <<= 1) {
+                                const u32 up = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+                                if (lane >= (u32)d) incl += up;
                             }
+                            const u32 fb_k = fb - (incl - need_k);            // wraps only behind a lane that already stops
+                            const u32 stops = __ballot_sync(0xFFFFFFFFu, lane < nb && need_k > fb_k);
+                            if (stops) { cnt = (u32)__ffs(stops); stop = true; }     // an eviction follows that iteration
+                            watch = __ballot_sync(0xFFFFFFFFu, room && need_next <= fb_k);
                         }
                         __syncwarp();
                         sl.tbuf[lane] = lane < cnt ? t_k : 0.0;          // + 0.0 changes no sum
@@ -678,8 +663,8 @@ k_trace_sim(DSpace s, DTrace tr, Range r, int tp_model, u64 max_iters_opt, guide
                             }
                             if (watch == 0 || !__any_sync(0xFFFFFFFFu, lane < 16 && arr_next <= sum)) {
                                 acc = sum; it += 32; t_k = t_next;
-                                if (stop) { if (counted) used = fb0 - fb + total - __shfl_sync(0xFFFFFFFFu, need_k, 31); break; }
-                                if (counted) { fb -= total; fb_it = it; }
+                                if (stop) { used = fb0 - fb + total - __shfl_sync(0xFFFFFFFFu, need_k, 31); break; }
+                                fb -= total;
                                 continue;
                             }
                         }
@@ -710,18 +695,17 @@ k_trace_sim(DSpace s, DTrace tr, Range r, int tp_model, u64 max_iters_opt, guide
                         }
                         it += ran;
                         if (arrived || stop) {
-                            if (counted && it > 1) used = fb0 - fb + __reduce_add_sync(0xFFFFFFFFu, lane < ran - 1 ? need_k : 0u);
+                            if (it > 1) used = fb0 - fb + __reduce_add_sync(0xFFFFFFFFu, lane < ran - 1 ? need_k : 0u);
                             break;
                         }
-                        if (counted) { fb -= total; fb_it = it; }
+                        fb -= total;
                         // a full batch in which the head had arrived but found no blocks: on to the next one
                         t_k = decode_time<TIME_SUM>(ctx_k, c_f9, dc_tha, c_kvx, c_f10, c_b10, icA, imA, dc_fix, dc_comm, dc_head, Nd, rt.tovh, lf);
                     }
                     clock = __shfl_sync(0xFFFFFFFFu, acc, 0); dec_time = acc;
                     const double cd = cd0 + nd * (double)it;
                     const u64 tok = (u64)it * nrun;
-                    // what is asked for after the last iteration is taken by the next pass
-                    if (it > 1) free_blocks -= used != 0xFFFFFFFFu ? used : taken(it - 1);
+                    free_blocks -= used;                        // what is asked for after the last iteration is taken by the next pass
                     D += it;
                     Dmod += it < blk ? it : modb(it);           // short runs are the rule
                     if (Dmod >= blk) Dmod -= blk;
