@@ -337,7 +337,7 @@ def extra_workloads(guide, torch, inputs, which, flush, hbm_peak, peak_kind, fra
                             "roofline": {"guide_simulate": hbm_roofline(BYTES_SIM * n, t_sim, hbm_peak, peak_kind, "53 B written per config"),
                                          "guide_select_topk (fused)": alu_roofline(ops / t_kf * 1e3, what),
                                          "guide_pareto (fused)": alu_roofline(ops / t_pf * 1e3, what)},
-                            "kernel_launches": 2 + 6 + 5 + 5 + 4}
+                            "kernel_launches": 2 + 6 + 5 + 1 + 2}
             if oracle is not None:
                 stride_all, stride_one = (1, 16) if k == 2 else (8, 128)
                 res[f"C{k}"]["cpu_baseline"] = cpu_baseline_of(oracle, w["space"], None, n, stride_all, stride_one, False)
@@ -509,9 +509,7 @@ def run_ours(args):
     torch.cuda.synchronize()
     one_call = {"ms": sum(e[0].elapsed_time(e[3]) for e in ev1) / n_turn,
                 "sweep_ms": sum(e[1].elapsed_time(e[2]) for e in ev1) / n_turn,
-                "what": "guide_simulate_select: the selections ride along with the sweep and nothing is read back; the sample "
-                        "evaluation before it and the rank kernels behind it cost more than the two filter passes they replace, "
-                        "which overlap on two streams, so the timed step keeps the three calls"}
+                "what": "guide_simulate_select: the sweep, then both selections, on one stream"}
     if world > 1:
         tt = torch.tensor([total_ms], dtype=torch.float64, device="cuda")
         dist.all_reduce(tt, op=dist.ReduceOp.MAX)
@@ -635,7 +633,7 @@ def run_ours(args):
     # simulate: memory + model kernel; top-k: bound, filter, rank and the two gated fallback kernels
     # (scan, merge: they return at once); Pareto: sample, filter, rank and the gated general kernel;
     # with several ranks the merge of the gathered lists (scan + merge, too short for the streaming path)
-    launches_per_step = 2 + 5 + 4 + (2 if world > 1 else 0)
+    launches_per_step = 2 + 1 + 2 + (2 if world > 1 else 0)
     line = {"metric": "configs/sec", "value": value, "unit": "configs/s", "n_gpus": world, "steps": args.steps,
             "warmup": max(args.warmup, 3), "ms_per_step": total_ms / args.steps, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
