@@ -188,26 +188,11 @@ __global__ void k_build_tables(const guide_model *gm, u32 n_m, const guide_hw *g
 
 static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-// ---- device memory of handles --------------------------------------------------------------------
-//
-// A handle's tables take tens of KB, and a program that asks one question per set of tables makes and
-// destroys a handle per question: cudaMalloc and cudaFree (which maps, unmaps and waits for the device)
-// were most of such a question's time (504 configs, answer read on the host: 830 us, 167 with the memory
-// kept and the tables uploaded in one copy instead of ten).  Blocks of destroyed handles are kept for the next ones: at most
-// TABLE_POOL_BLOCKS per device and TABLE_POOL_BYTES each (larger ones, and any beyond that number, are
-// freed), all of a device's when an allocation fails, the rest when the library is unloaded.  A block is
-// put back only after the device has been waited for, as cudaFree does, so whoever gets it next may
-// write it on any stream.  Blocks remember their context: those of a context that has been reset since
-// are forgotten.
-static constexpr size_t TABLE_POOL_BLOCKS = 4, TABLE_POOL_BYTES = 1u << 20;
+// ---- device memory of handles (table_pool.h) ----------------------------------------------------------
 
-struct TablePool {
-    struct Block { int device; unsigned long long context; void *p; size_t bytes; };
-    std::mutex mu;
-    std::vector<Block> blocks;
-
-    // a number that identifies the current context for the life of the process (0: not to be had, nothing is kept)
-    static unsigned long long context_id() {
+struct CudaDevice {
+    // an id of the current context that is not used again in the life of the process
+    static unsigned long long context(bool make) {
         typedef int (*GetCurrent)(void **);
         typedef int (*GetId)(void *, unsigned long long *);
         static void *get_current = nullptr, *get_id = nullptr;
@@ -217,55 +202,27 @@ struct TablePool {
             if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &get_current, 12000, cudaEnableDefault, &q) != cudaSuccess) get_current = nullptr;
             if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &get_id, 12000, cudaEnableDefault, &q) != cudaSuccess) get_id = nullptr;
         });
+        if (!get_current || !get_id) return 0;
         void *ctx = nullptr;
         unsigned long long id = 0;
-        if (!get_current || !get_id || ((GetCurrent)get_current)(&ctx) != 0 || !ctx || ((GetId)get_id)(ctx, &id) != 0) return 0;
-        return id;
-    }
-    cudaError_t take(int device, size_t need, void **p, size_t *bytes) {
-        const unsigned long long ctx = context_id();
-        {
-            std::lock_guard<std::mutex> lock(mu);
-            size_t best;
-            blocks.erase(std::remove_if(blocks.begin(), blocks.end(), [&](const Block &b) { return b.device == device && b.context != ctx; }),
-                         blocks.end());
-            best = blocks.size();
-            for (size_t i = 0; i < blocks.size(); i++)
-                if (blocks[i].device == device && blocks[i].bytes >= need && (best == blocks.size() || blocks[i].bytes < blocks[best].bytes)) best = i;
-            if (best < blocks.size()) {
-                *p = blocks[best].p; *bytes = blocks[best].bytes;
-                blocks.erase(blocks.begin() + best);
-                return cudaSuccess;
-            }
+        if (((GetCurrent)get_current)(&ctx) != 0) return 0;
+        if (!ctx) {                                        // a thread whose first CUDA call this is
+            if (!make) return 0;
+            if (cudaFree(nullptr) != cudaSuccess) { (void)cudaGetLastError(); return 0; }
+            if (((GetCurrent)get_current)(&ctx) != 0 || !ctx) return 0;
         }
-        *bytes = align_up(need, 64 * 1024);                 // so that a block suits the next handle of about that size
-        cudaError_t e = cudaMalloc(p, *bytes);
-        if (e == cudaErrorMemoryAllocation) {
-            (void)cudaGetLastError();
-            drop(device);
-            e = cudaMalloc(p, *bytes);
-        }
-        return e;
+        return ((GetId)get_id)(ctx, &id) == 0 ? id : 0;
     }
-    // the caller has made `device` current
-    void give(int device, void *p, size_t bytes) {
-        const unsigned long long ctx = context_id();
-        if (ctx != 0 && bytes <= TABLE_POOL_BYTES && cudaDeviceSynchronize() == cudaSuccess) {
-            std::lock_guard<std::mutex> lock(mu);
-            size_t n = 0;
-            for (const Block &b : blocks) n += b.device == device;
-            if (n < TABLE_POOL_BLOCKS) { blocks.push_back({device, ctx, p, bytes}); return; }
-        }
-        cudaFree(p);
+    static int alloc(void **p, size_t bytes) {
+        const cudaError_t e = cudaMalloc(p, bytes);
+        if (e == cudaErrorMemoryAllocation) (void)cudaGetLastError();
+        return (int)e;
     }
-    void drop(int device) {                                 // device < 0: every device's
-        std::lock_guard<std::mutex> lock(mu);
-        for (size_t i = blocks.size(); i-- > 0;)
-            if (device < 0 || blocks[i].device == device) { cudaFree(blocks[i].p); blocks.erase(blocks.begin() + i); }
-    }
-    ~TablePool() { drop(-1); }                              // an error once the runtime has gone, and then there is nothing to free
+    static bool out_of_memory(int e) { return e == (int)cudaErrorMemoryAllocation; }
+    static void release(void *p) { cudaFree(p); }
+    static bool wait() { return cudaDeviceSynchronize() == cudaSuccess; }
 };
-static TablePool g_tables;
+static TablePool<CudaDevice> g_tables;
 
 // Work orders for the closed-form model kernel.  They decide which thread evaluates what, never a
 // value: any permutation gives the same outputs.
@@ -379,9 +336,9 @@ int space_on_device(guide_space *s, DSpace *out, unsigned **ticket, cudaStream_t
     put(o_hs, hf_sorted.data(), hf_sorted.size() * sizeof(HfSorted));
     put(o_po, plane_order.data(), plane_order.size() * 4);
     put(o_lo, line_order.data(), line_order.size() * 4);
-    char *blob = nullptr;
-    size_t blob_bytes = 0;
-    GUIDE_CUDA(g_tables.take(dev, off, (void **)&blob, &blob_bytes));
+    TableBlock block;
+    GUIDE_CUDA((cudaError_t)g_tables.take(off, &block));
+    char *const blob = (char *)block.p;
     cudaError_t e = cudaMemcpyAsync(blob, image.data(), from_host, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) {
         const u32 n = (u32)std::max(n_m, n_h * n_f);
@@ -397,11 +354,10 @@ int space_on_device(guide_space *s, DSpace *out, unsigned **ticket, cudaStream_t
         // the image must outlive the copy, and another stream may use the tables next
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     }
-    if (e != cudaSuccess) { g_tables.give(dev, blob, blob_bytes); return cuda_fail(e, "uploading the space tables"); }
+    if (e != cudaSuccess) { CudaDevice::release(blob); return cuda_fail(e, "uploading the space tables"); }
     DeviceTables d;
     d.device = dev;
-    d.blob = blob;
-    d.blob_bytes = blob_bytes;
+    d.block = block;
     d.view.models = (const DModel *)(blob + o_dm);
     d.view.rates = (const DRate *)(blob + o_dr);
     d.view.batch = (const u32 *)(blob + o_b);
@@ -436,18 +392,17 @@ int trace_on_device(guide_trace *t, DTrace *out, cudaStream_t st) {
         if (d.device == dev) { *out = d.view; return GUIDE_OK; }
     const size_t n = t->arrival.size();
     const size_t o_a = 0, o_i = align_up(n * 8, 256), o_o = o_i + align_up(n * 4, 256), total = o_o + align_up(n * 4, 256);
-    char *blob = nullptr;
-    size_t blob_bytes = 0;
-    GUIDE_CUDA(g_tables.take(dev, total, (void **)&blob, &blob_bytes));
+    TableBlock block;
+    GUIDE_CUDA((cudaError_t)g_tables.take(total, &block));
+    char *const blob = (char *)block.p;
     cudaError_t e = cudaMemcpyAsync(blob + o_a, t->arrival.data(), n * 8, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(blob + o_i, t->in_len.data(), n * 4, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(blob + o_o, t->out_len.data(), n * 4, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);      // the copies are done before another stream can use the trace
-    if (e != cudaSuccess) { g_tables.give(dev, blob, blob_bytes); return cuda_fail(e, "uploading the trace"); }
+    if (e != cudaSuccess) { CudaDevice::release(blob); return cuda_fail(e, "uploading the trace"); }
     DeviceTrace d;
     d.device = dev;
-    d.blob = blob;
-    d.blob_bytes = blob_bytes;
+    d.block = block;
     d.view.arrival = (const double *)(blob + o_a);
     d.view.in_len = (const u32 *)(blob + o_i);
     d.view.out_len = (const u32 *)(blob + o_o);
@@ -626,7 +581,7 @@ void guide_space_destroy(guide_space *s) {
     int cur = 0;
     const bool have = cudaGetDevice(&cur) == cudaSuccess;
     for (DeviceTables &d : s->dev) {
-        if (have && cudaSetDevice(d.device) == cudaSuccess) g_tables.give(d.device, d.blob, d.blob_bytes);
+        if (have && cudaSetDevice(d.device) == cudaSuccess) g_tables.give(d.block);
     }
     if (have && !s->dev.empty()) cudaSetDevice(cur);
     delete s;
@@ -686,7 +641,7 @@ void guide_trace_destroy(guide_trace *t) {
     int cur = 0;
     const bool have = cudaGetDevice(&cur) == cudaSuccess;
     for (DeviceTrace &d : t->dev)
-        if (have && cudaSetDevice(d.device) == cudaSuccess) g_tables.give(d.device, d.blob, d.blob_bytes);
+        if (have && cudaSetDevice(d.device) == cudaSuccess) g_tables.give(d.block);
     if (have && !t->dev.empty()) cudaSetDevice(cur);
     delete t;
 }

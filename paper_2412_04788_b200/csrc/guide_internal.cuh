@@ -9,6 +9,7 @@
 #include "../../include/guide.h"
 #include "model.cuh"
 #include "model_f32.cuh"
+#include "table_pool.h"
 #include "tiled.cuh"
 
 namespace guide {
@@ -28,8 +29,7 @@ static constexpr unsigned TICKET_SLOTS = 64;
 
 struct DeviceTables {
     int device = -1;
-    void *blob = nullptr;
-    size_t blob_bytes = 0;
+    TableBlock block;
     DSpace view{};
     unsigned *tickets = nullptr;     // TICKET_SLOTS slots, 32 words apart
     std::vector<void *> ticket_streams;   // slot i belongs to the calls on ticket_streams[i]
@@ -37,8 +37,7 @@ struct DeviceTables {
 
 struct DeviceTrace {
     int device = -1;
-    void *blob = nullptr;
-    size_t blob_bytes = 0;
+    TableBlock block;
     DTrace view{};
 };
 

@@ -58,3 +58,39 @@ def test_handles_on_several_threads_and_streams():
     for t in threads:
         t.join()
     assert not errors, errors
+
+
+def test_fresh_threads_lose_no_memory():
+    """Threads whose first CUDA call is one of this library's, each with a handle of its own: what one leaves
+    behind serves the next, and nothing is lost on the way."""
+    import torch
+    w = I.workload(4)["space"]                           # tables of about half a megabyte
+    count = 4096
+    sp = guide.Space(w)
+    out = guide.alloc_outputs(count)
+    stream = torch.cuda.current_stream()
+    guide.guide_simulate(sp, None, out, count=count)
+    torch.cuda.synchronize()
+    want = {k: v.clone() for k, v in out.items()}
+    errors = []
+
+    def question():
+        try:
+            mine = guide.Space(w)
+            guide.guide_simulate(mine, None, out, count=count, stream=stream)
+            mine.close()
+        except Exception as e:                           # noqa: BLE001 - reported by the main thread
+            errors.append(repr(e))
+
+    def run(n):
+        for _ in range(n):
+            t = threading.Thread(target=question)
+            t.start()
+            t.join()
+        torch.cuda.synchronize()
+        return torch.cuda.mem_get_info()[0]
+    before = run(8)                                      # the pool has its blocks
+    after = run(64)
+    assert not errors, errors
+    assert all(torch.equal(want[k], out[k]) for k in want)
+    assert before - after < 8 << 20, f"{(before - after) >> 20} MB lost"
