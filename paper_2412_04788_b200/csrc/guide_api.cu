@@ -220,7 +220,15 @@ struct CudaDevice {
     }
     static bool out_of_memory(int e) { return e == (int)cudaErrorMemoryAllocation; }
     static void release(void *p) { cudaFree(p); }
-    static bool wait() { return cudaDeviceSynchronize() == cudaSuccess; }
+    // an id of the stream that no later one gets; 0 while it is being captured
+    static unsigned long long stream_id(cudaStream_t st) {
+        cudaStreamCaptureStatus cap;
+        unsigned long long id = 0;
+        if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) { (void)cudaGetLastError(); return 0; }
+        if (cap != cudaStreamCaptureStatusNone) return 0;      // asking for the id would end the capture
+        if (cudaStreamGetId(st, &id) != cudaSuccess) { (void)cudaGetLastError(); return 0; }
+        return id + 1;
+    }
 };
 static TablePool<CudaDevice> g_tables;
 
@@ -306,6 +314,7 @@ int space_on_device(guide_space *s, DSpace *out, unsigned **ticket, cudaStream_t
     for (DeviceTables &d : s->dev)
         if (d.device == dev) {
             *out = d.view;
+            if (ticket) d.block.used_on(CudaDevice::stream_id(st));      // a selection on given metrics reads no tables
             return ticket ? ticket_for(d, st, ticket) : GUIDE_OK;
         }
 
@@ -337,7 +346,7 @@ int space_on_device(guide_space *s, DSpace *out, unsigned **ticket, cudaStream_t
     put(o_po, plane_order.data(), plane_order.size() * 4);
     put(o_lo, line_order.data(), line_order.size() * 4);
     TableBlock block;
-    GUIDE_CUDA((cudaError_t)g_tables.take(off, &block));
+    GUIDE_CUDA((cudaError_t)g_tables.take(off, CudaDevice::stream_id(st), &block));
     char *const blob = (char *)block.p;
     cudaError_t e = cudaMemcpyAsync(blob, image.data(), from_host, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) {
@@ -379,6 +388,7 @@ int space_on_device(guide_space *s, DSpace *out, unsigned **ticket, cudaStream_t
     d.view.n_m = (u32)n_m; d.view.n_h = (u32)n_h; d.view.n_f = (u32)n_f;
     d.view.n_b = (u32)s->batch.size(); d.view.n_t = (u32)s->tp.size(); d.view.n_l = (u32)s->pairs.size();
     d.tickets = (unsigned *)(blob + o_tk);
+    if (ticket) d.block.used_on(CudaDevice::stream_id(st));
     s->dev.push_back(d);
     *out = d.view;
     return ticket ? ticket_for(s->dev.back(), st, ticket) : GUIDE_OK;
@@ -388,12 +398,12 @@ int trace_on_device(guide_trace *t, DTrace *out, cudaStream_t st) {
     int dev = 0;
     GUIDE_CUDA(cudaGetDevice(&dev));
     std::lock_guard<std::mutex> lock(t->mu);
-    for (const DeviceTrace &d : t->dev)
-        if (d.device == dev) { *out = d.view; return GUIDE_OK; }
+    for (DeviceTrace &d : t->dev)
+        if (d.device == dev) { *out = d.view; d.block.used_on(CudaDevice::stream_id(st)); return GUIDE_OK; }
     const size_t n = t->arrival.size();
     const size_t o_a = 0, o_i = align_up(n * 8, 256), o_o = o_i + align_up(n * 4, 256), total = o_o + align_up(n * 4, 256);
     TableBlock block;
-    GUIDE_CUDA((cudaError_t)g_tables.take(total, &block));
+    GUIDE_CUDA((cudaError_t)g_tables.take(total, CudaDevice::stream_id(st), &block));
     char *const blob = (char *)block.p;
     cudaError_t e = cudaMemcpyAsync(blob + o_a, t->arrival.data(), n * 8, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(blob + o_i, t->in_len.data(), n * 4, cudaMemcpyHostToDevice, st);
@@ -412,6 +422,7 @@ int trace_on_device(guide_trace *t, DTrace *out, cudaStream_t st) {
     d.view.sum_out = t->sum_out;
     d.view.sum_in = t->sum_in;
     d.view.n_zero = t->n_zero;
+    d.block.used_on(CudaDevice::stream_id(st));
     t->dev.push_back(d);
     *out = d.view;
     return GUIDE_OK;

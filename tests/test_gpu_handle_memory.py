@@ -94,3 +94,60 @@ def test_fresh_threads_lose_no_memory():
     assert not errors, errors
     assert all(torch.equal(want[k], out[k]) for k in want)
     assert before - after < 8 << 20, f"{(before - after) >> 20} MB lost"
+
+
+@pytest.mark.parametrize("mode,thread", [("relaxed", False), ("relaxed", True), ("thread_local", True)])
+def test_destroyed_during_a_capture(mode, thread):
+    """A handle that is destroyed while a stream is being captured (by the collector, on another thread) does not
+    end the capture."""
+    import torch
+    w = spaces()[0]
+    sp = guide.Space(w)
+    out = guide.alloc_outputs(sp.size)
+    guide.guide_simulate(sp, None, out)
+    torch.cuda.synchronize()
+    x = torch.zeros(1, device="cuda")
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, capture_error_mode=mode):
+        x.add_(1.0)
+        if thread:
+            t = threading.Thread(target=sp.close)
+            t.start()
+            t.join()
+        else:
+            sp.close()
+        x.add_(1.0)
+    x.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    assert x.item() == 2.0
+
+
+def test_captured_use_and_the_next_handle():
+    """A graph that holds a handle's kernels may run on any stream, until the handle is destroyed: its memory is
+    not handed to a handle that is used meanwhile."""
+    import torch
+    w = spaces()
+    want = [oracle.simulate(x) for x in w[:2]]
+    a = guide.Space(w[0])
+    out_a = guide.alloc_outputs(a.size)
+    side, other = torch.cuda.Stream(), torch.cuda.Stream()
+    guide.guide_simulate(a, None, out_a, stream=side)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=side):
+        guide.guide_simulate(a, None, out_a)
+    for v in out_a.values():
+        v.zero_()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(other):
+        for _ in range(50):
+            g.replay()
+    a.close()
+    b = guide.Space(w[1])
+    out_b = guide.alloc_outputs(b.size)
+    guide.guide_simulate(b, None, out_b, stream=side)
+    torch.cuda.synchronize()
+    for out, ref in ((out_a, want[0]), (out_b, want[1])):
+        assert not any(bit_mismatches({k: v.cpu().numpy() for k, v in out.items()}, ref).values())
+    b.close()
