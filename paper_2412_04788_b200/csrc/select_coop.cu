@@ -28,9 +28,15 @@
 // Ranges of up to 2048 configs are one block: its barriers are block barriers and nothing goes
 // through the workspace.
 //
-// Top-k + front after a sweep on a B200, against chains of kernels (sample, refined bound, filter, rank,
-// gated fallback): 983,040 configs 14 + 21 us instead of 38 + 39; 504 configs 7 + 8 us instead of 14 + 19;
-// 16.8 M configs (one row of 14 sampled) 60 + 65 us instead of 65 + 78.
+// Blocks per SM: ranges whose rows all fit the warps' registers (1.2 M configs) take two, and their kernels have no
+// pass over the arrays in them (WHOLE: half the code, 983,040 configs 25 -> 19 us top-k, 25 -> 23 front).  Longer
+// ranges take one.  A cooperative launch starts only when all of its blocks have room, so with two per SM two
+// selections on two streams run one after the other: 16.8 M configs, sweep and both selections, 334 us against 289
+// with one, 2.2 M 124 against 100.  On one stream one block per SM costs nothing that a pass with more in flight does
+// not give back (16.8 M: 63 + 79 us with two, 67 + 78 with one; 2.2 M: 33 + 39 and 33 + 33).
+//
+// Top-k + front on a B200 against chains of kernels (sample, refined bound, filter, rank, gated fallback): 983,040
+// configs 19 + 23 us instead of 35 + 34; 30,720 configs 17 + 17 instead of 68 + 42; 16.8 M 67 + 78 instead of 65 + 83.
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
@@ -42,7 +48,7 @@
 namespace guide {
 
 static constexpr u32 CO_THREADS = 512, CO_WARPS = CO_THREADS / 32;
-static constexpr u32 CO_BLOCKS_PER_SM = 2;      // 64 registers: 32 warps per SM, and few enough blocks for a quick grid barrier
+static constexpr u32 CO_BLOCKS_PER_SM = 2;      // 64 registers: 32 warps per SM, of one call or of two side by side
 static constexpr u32 CO_ROWS = 4;               // sample rows a warp keeps in registers
 static constexpr u32 CO_ONE_BLOCK_ROWS = 32;    // ranges up to this many rows are one block; its survivors stay in shared memory
 static constexpr u32 CO_BOUND_LIST = 1024;      // most pairs a bound is worked out from: group minima, sample pairs within the coarse bound
@@ -59,7 +65,7 @@ template <int NA>
 struct CoopSrc {
     Arr a[NA];        // entry 0 is the key (top-k) or x (Pareto), entry 1 is y (Pareto only)
     const uint8_t *status;
-    int vec;          // every array is 16-byte aligned (status: 2-byte)
+    int vec;          // every array is 16-byte aligned, status 4-byte (2: 16-byte too); 0: no wide loads
 };
 
 // The sample: groups of r consecutive rows, one row of each, at a hashed offset so that it does not
@@ -74,14 +80,19 @@ struct Walk {
     }
 };
 
-// status and values of this lane's two configs of a row; outside the range: status 0xFF
-template <int NA>
+// status and values of this lane's two configs of a row; outside the range: status 0xFF.  LAST: not read again
+// (marked for early eviction: with the lines kept, the sweep that overwrites the arrays next takes 8 of 68 us longer).
+template <bool LAST, int NA>
 __device__ __forceinline__ void load_row(const CoopSrc<NA> &s, u64 count, u64 row, bool live, u32 lane, u32 &st, double2 (&v)[NA]) {
     const u64 j = row * ROW + 2 * lane;
     if (live && s.vec && (row + 1) * ROW <= count) {
-        st = __ldcg(reinterpret_cast<const unsigned short *>(s.status + j));
+        const unsigned short *sp = reinterpret_cast<const unsigned short *>(s.status + j);
+        st = LAST ? __ldcs(sp) : __ldcg(sp);
 #pragma unroll
-        for (int a = 0; a < NA; a++) v[a] = __ldcg(reinterpret_cast<const double2 *>(s.a[a].p + j));
+        for (int a = 0; a < NA; a++) {
+            const double2 *vp = reinterpret_cast<const double2 *>(s.a[a].p + j);
+            v[a] = LAST ? __ldcs(vp) : __ldcg(vp);
+        }
     } else {
         const bool in0 = live && j < count, in1 = live && j + 1 < count;
         st = (in0 ? (u32)s.status[j] : 0xFFu) | ((in1 ? (u32)s.status[j + 1] : 0xFFu) << 8);
@@ -104,60 +115,88 @@ __device__ __forceinline__ void row_ok(const CoopSrc<NA> &s, u32 st, const doubl
     }
 }
 
-// A pass over everything, in chunks of CO_ROWS rows taken in turn by all warps, from the end of the range
-// backwards (when the metrics were written just before this call the end of the arrays is what the L2
-// still holds).  Neighbouring chunks go to different blocks, and a warp takes a different place in every
-// round: rows that fit come in runs, and a fixed place would share its position modulo the batch and TP
-// axes, whose lengths are powers of two as the number of warps nearly is.
-struct FilterWalk {
-    u64 n_rows, stride, base;
-    u32 pos;
-    __device__ __forceinline__ FilterWalk(u64 rows, u64 warps, u32 first) : n_rows(rows), stride(warps), base(0), pos(first) {}
-    // row u of the current chunk; past the end of the walk: a huge number
-    __device__ __forceinline__ u64 row(u32 u) const { return n_rows - 1 - ((base + pos) * CO_ROWS + u); }
-    __device__ __forceinline__ bool more() const { return base * CO_ROWS < n_rows; }
-    __device__ __forceinline__ void next() { base += stride; pos = (pos + 37u) % (u32)stride; }
+// ---- a pass over everything ---------------------------------------------------------------------------
+//
+// Chunks of CO_CHUNK rows, from the end of the range backwards (when the metrics were written just before this call the
+// end of the arrays is what the L2 still holds).  Every warp starts with three of its own; the others are taken
+// through a counter in the workspace as warps get to them: rows that fit come in runs, and a chunk of live rows
+// costs many times one without.
+//
+// A chunk's status bytes are one 16-byte load per lane, asked for two chunks ahead; values are loaded for rows with a
+// config that passed its memory check only, which most rows of a large sweep have not, several such rows at a time,
+// and looked at together.  That keeps enough in flight for one block of 16 warps per SM, so that two selections on
+// two streams run side by side.
+static constexpr u32 CO_CHUNK = 8;
+template <int NA> __host__ __device__ constexpr int group_rows() { return NA <= 2 ? 4 : 2; }   // rows whose values are in flight at a time
+
+struct ChunkWalk {
+    u64 n_rows, chunk;                                 // chunk: number from the end, or past the last one
+    // row u of the chunk; past the end of the walk: a huge number
+    __device__ __forceinline__ u64 row(u32 u) const { return n_rows - 1 - (chunk * CO_CHUNK + u); }
+    __device__ __forceinline__ bool more() const { return chunk * CO_CHUNK < n_rows; }
 };
 
-// The status bytes of a chunk come first (asked for a round ahead); a row's values are loaded only if
-// some config of it passed its memory check, which most rows of a large sweep do not.
+// status of 16 consecutive configs of a row (lane L: part L % 4 of row L / 4 of the chunk); outside the range: 0xFF
 template <int NA>
-__device__ __forceinline__ void load_chunk_status(const CoopSrc<NA> &s, u64 count, const FilterWalk &fw, u32 lane, u32 (&st)[CO_ROWS]) {
-#pragma unroll
-    for (u32 u = 0; u < CO_ROWS; u++) {
-        const u64 row = fw.row(u), j = row * ROW + 2 * lane;
-        st[u] = 0xFFFFu;
-        if (row < fw.n_rows) {
-            if (s.vec && (row + 1) * ROW <= count) st[u] = __ldcs(reinterpret_cast<const unsigned short *>(s.status + j));
-            else st[u] = (j < count ? (u32)s.status[j] : 0xFFu) | ((j + 1 < count ? (u32)s.status[j + 1] : 0xFFu) << 8);
-        }
+__device__ __forceinline__ uint4 chunk_status(const CoopSrc<NA> &s, u64 count, const ChunkWalk &w, u32 lane) {
+    uint4 st = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
+    const u64 row = w.row(lane >> 2);
+    if (row >= w.n_rows) return st;
+    const u64 j = row * ROW + 16 * (lane & 3);
+    if (s.vec && j + 16 <= count) {
+        if (s.vec == 2) return __ldcs(reinterpret_cast<const uint4 *>(s.status + j));
+        const u32 *q = reinterpret_cast<const u32 *>(s.status + j);
+        return make_uint4(__ldcs(q), __ldcs(q + 1), __ldcs(q + 2), __ldcs(q + 3));
     }
+    u32 wd[4];
+#pragma unroll
+    for (u32 i = 0; i < 4; i++) {
+        wd[i] = 0;
+#pragma unroll
+        for (u32 k = 0; k < 4; k++) wd[i] |= (j + 4 * i + k < count ? (u32)s.status[j + 4 * i + k] : 0xFFu) << (8 * k);
+    }
+    return make_uint4(wd[0], wd[1], wd[2], wd[3]);
 }
-// returns false when no row of the chunk has a config to look at
-template <int NA>
-__device__ __forceinline__ bool load_chunk_values(const CoopSrc<NA> &s, u64 count, const FilterWalk &fw, u32 lane,
-                                                  const u32 (&st)[CO_ROWS], double2 (&v)[CO_ROWS][NA]) {
-    u32 any = 0;
+__device__ __forceinline__ bool has_zero_byte(u32 w) { return __vcmpeq4(w, 0u) != 0; }
+
+// each(j, v, ok) for groups of rows that have a config to look at, by whole warps: the lane's two configs of row g are
+// entries j[g] and j[g] + 1 of the arrays, v[g] their values; bits 2 g and 2 g + 1 of ok: they pass the constraints.
+// counter: a word of the workspace, 0 on entry.
+template <int NA, class Each>
+__device__ __forceinline__ void for_live_rows(const CoopSrc<NA> &s, u64 count, u64 n_rows, u32 lane, u32 warp, u32 *counter, Each each) {
+    constexpr int GROUP = group_rows<NA>();
+    const u32 warps = gridDim.x * CO_WARPS;
+    ChunkWalk w{n_rows, (u64)warp * gridDim.x + blockIdx.x}, w1{n_rows, w.chunk + warps}, w2{n_rows, w.chunk + 2 * (u64)warps};
+    uint4 st = chunk_status(s, count, w, lane), st1 = chunk_status(s, count, w1, lane), st2 = chunk_status(s, count, w2, lane);
+    while (w.more()) {
+        u32 ticket = 0;
+        if (lane == 0 && w2.more()) ticket = atomicAdd(counter, 1u);
+        u32 live = __ballot_sync(0xFFFFFFFFu, has_zero_byte(st.x) | has_zero_byte(st.y) | has_zero_byte(st.z) | has_zero_byte(st.w));
+        live |= live >> 1;
+        live = (live | live >> 2) & 0x11111111u;       // bit 4 u: row u
+        while (live) {
+            double2 v[GROUP][NA];
+            u64 j[GROUP];
+            u32 st_v[GROUP], ok = 0;
 #pragma unroll
-    for (u32 u = 0; u < CO_ROWS; u++)
-        if (__any_sync(0xFFFFFFFFu, (st[u] & 0xFFu) == 0 || (st[u] >> 8) == 0)) any |= 1u << u;
-    if (any == 0) return false;
-#pragma unroll
-    for (u32 u = 0; u < CO_ROWS; u++) {
-        const u64 row = fw.row(u), j = row * ROW + 2 * lane;
-#pragma unroll
-        for (int a = 0; a < NA; a++) {
-            v[u][a] = make_double2(0.0, 0.0);
-            if ((any >> u) & 1u) {
-                if (s.vec && (row + 1) * ROW <= count) v[u][a] = __ldcs(reinterpret_cast<const double2 *>(s.a[a].p + j));
-                else {
-                    if (j < count) v[u][a].x = s.a[a].p[j];
-                    if (j + 1 < count) v[u][a].y = s.a[a].p[j + 1];
-                }
+            for (int g = 0; g < GROUP; g++) {
+                const u64 row = w.row(((u32)__ffs(live) - 1) >> 2);
+                j[g] = row * ROW + 2 * lane;
+                load_row<true>(s, count, row, live != 0, lane, st_v[g], v[g]);
+                live &= live - 1;
             }
+#pragma unroll
+            for (int g = 0; g < GROUP; g++) {
+                bool ok0, ok1;
+                row_ok(s, st_v[g], v[g], ok0, ok1);
+                ok |= (ok0 ? 1u : 0u) << (2 * g) | (ok1 ? 1u : 0u) << (2 * g + 1);
+            }
+            each(j, v, ok);
         }
+        w = w1; w1 = w2; st = st1; st1 = st2;
+        w2.chunk = w1.more() ? 3 * (u64)warps + __shfl_sync(0xFFFFFFFFu, ticket, 0) : w1.chunk;     // past the end: stays there
+        st2 = chunk_status(s, count, w2, lane);
     }
-    return true;
 }
 
 __device__ __forceinline__ void grid_barrier() {
@@ -352,9 +391,10 @@ __device__ __noinline__ void topk_finish(const KI *cand, u32 n, u32 k, FinishScr
         }
         __syncthreads();
     }
-    // down to CO_RANKED pairs: those within a bound of what shared memory holds.  A list that does not fit
-    // it is gone through again with that bound, which leaves out most of what was looked at.
-    while (c > CO_RANKED) {
+    // down to CO_RANKED pairs, and once towards the k that are wanted (ranking 232 pairs takes 10 us, 70 take 3): those
+    // within a bound of what shared memory holds.  A list that does not fit it is gone through again with that bound,
+    // which leaves out most of what was looked at.
+    for (bool cut = false; c > CO_RANKED || (!cut && c > found + CO_RANKED / 4); cut = true) {
         if (c > CO_LIST) {
             __syncthreads();
             if (threadIdx.x == 0) f.n = 0;
@@ -407,7 +447,8 @@ __device__ __noinline__ void topk_finish(const KI *cand, u32 n, u32 k, FinishScr
     }
 }
 
-template <int NA>
+// WHOLE: the sample is everything (w.r == 1), and the one pass over the arrays is the sample's.
+template <int NA, bool WHOLE>
 __global__ void __launch_bounds__(CO_THREADS, CO_BLOCKS_PER_SM)
 k_topk_coop(CoopSrc<NA> s, Range r, Walk w, u32 k, u32 group_log2, u32 *header, KI *minima, KI *spairs, KI *cand, int negate,
             u64 *idx_out, double *key_out, u32 *count_out) {
@@ -429,7 +470,7 @@ k_topk_coop(CoopSrc<NA> s, Range r, Walk w, u32 k, u32 group_log2, u32 *header, 
 #pragma unroll
         for (u32 u = 0; u < CO_ROWS; u++) {
             const u64 slot = (u64)((u << group_log2) + member) * n_groups + group;
-            load_row(s, r.count, w.row(slot), slot < w.n_slots, lane, st[u], v[u]);
+            load_row<false>(s, r.count, w.row(slot), slot < w.n_slots, lane, st[u], v[u]);
         }
 #pragma unroll
         for (u32 u = 0; u < CO_ROWS; u++) {
@@ -445,7 +486,7 @@ k_topk_coop(CoopSrc<NA> s, Range r, Walk w, u32 k, u32 group_log2, u32 *header, 
         return r.first + w.row(slot) * ROW + 2 * lane + (i & 1);
     };
     // ---- one block: what passes is ranked where it is ----
-    if (gridDim.x == 1) {
+    if (WHOLE && gridDim.x == 1) {
         if (threadIdx.x == 0) fin.n = 0;
         __syncthreads();
 #pragma unroll
@@ -481,24 +522,24 @@ k_topk_coop(CoopSrc<NA> s, Range r, Walk w, u32 k, u32 group_log2, u32 *header, 
     u64 bkey, bidx;
     list_bound<CO_BOUND_LIST / CO_THREADS>(minima, n_groups, k, fin.bins, sc, bkey, bidx);
     // ---- the sample values within it: the survivors themselves, or (r > 1) the pairs of a closer bound ----
-    const bool whole = w.r == 1;
     u32 *count = header + TK_COUNT;
 #pragma unroll
     for (u32 i = 0; i < 2 * CO_ROWS; i++) {
         KI e; e.key = key[i]; e.idx = index_of(i);
         const bool take = ((ok >> i) & 1u) && pair_le(e.key, e.idx, bkey, bidx);
-        if (whole) warp_append(take, e, count, cand, TK_CAND_CAP);
+        if (WHOLE) warp_append(take, e, count, cand, TK_CAND_CAP);
         else warp_append(take, e, header + TK_SAMPLED, spairs, CO_BOUND_LIST);
     }
     grid_barrier();
-    if (!whole) {
+    if (!WHOLE) {
         // of more pairs than the list holds the stored ones still give a valid bound; fewer than k only
         // when the coarse bound is all-ones, which then stays
         const u32 ns = min(__ldcg(header + TK_SAMPLED), CO_BOUND_LIST);
         if (ns >= k) list_bound<CO_BOUND_LIST / CO_THREADS>(spairs, ns, k, fin.bins, sc, bkey, bidx);
     }
     // ---- filter passes over everything: none when the sample was everything and its survivors fit ----
-    for (bool first_pass = !whole;; first_pass = false) {
+    u32 *ticket = header + TK_TICKET;
+    for (bool first_pass = !WHOLE;; first_pass = false) {
         if (!first_pass) {
             const u32 n = __ldcg(count);
             if (n <= TK_CAND_CAP) {
@@ -507,36 +548,26 @@ k_topk_coop(CoopSrc<NA> s, Range r, Walk w, u32 k, u32 group_log2, u32 *header, 
             }
             // the list overflowed: k pairs of what it holds are within a bound that excludes more
             list_bound<CO_BOUND_LIST / CO_THREADS>(cand, TK_CAND_CAP, k, fin.bins, sc, bkey, bidx);
-            u32 *next = count == header + TK_COUNT ? header + TK_TICKET : header + TK_COUNT;   // last read two barriers ago
-            if (blockIdx.x == 0 && threadIdx.x == 0) *next = 0;
-            count = next;
+            // the other pair of counters: last read two barriers ago
+            count = count == header + TK_COUNT ? header + TK_COUNT2 : header + TK_COUNT;
+            ticket = ticket == header + TK_TICKET ? header + TK_TICKET2 : header + TK_TICKET;
+            if (blockIdx.x == 0 && threadIdx.x == 0) *count = *ticket = 0;
             grid_barrier();
         }
-        const u64 stride = (u64)gridDim.x * CO_WARPS;
-        FilterWalk fw(w.n_rows, stride, warp * gridDim.x + blockIdx.x), ahead = fw;
-        u32 st[CO_ROWS], st_ahead[CO_ROWS];
-        load_chunk_status(s, r.count, ahead, lane, st_ahead);
-        for (; fw.more(); fw = ahead) {
+        for_live_rows<NA>(s, r.count, w.n_rows, lane, warp, ticket, [&](const u64 *j, const double2 (*v)[NA], u32 pass) {
 #pragma unroll
-            for (u32 u = 0; u < CO_ROWS; u++) st[u] = st_ahead[u];
-            ahead.next();
-            load_chunk_status(s, r.count, ahead, lane, st_ahead);
-            double2 v[CO_ROWS][NA];
-            if (!load_chunk_values(s, r.count, fw, lane, st, v)) continue;
-#pragma unroll
-            for (u32 u = 0; u < CO_ROWS; u++) {
-                bool ok0, ok1;
-                row_ok(s, st[u], v[u], ok0, ok1);
-                const u64 k0 = metric_key(s.a[0], v[u][0].x), k1 = metric_key(s.a[0], v[u][0].y);
-                ok0 = ok0 && k0 <= bkey; ok1 = ok1 && k1 <= bkey;
-                if (!__any_sync(0xFFFFFFFFu, ok0 | ok1)) continue;     // the usual case
-                KI e0, e1;
-                e0.key = k0; e0.idx = r.first + fw.row(u) * ROW + 2 * lane;
-                e1.key = k1; e1.idx = e0.idx + 1;
-                warp_append(ok0 && pair_le(e0.key, e0.idx, bkey, bidx), e0, count, cand, TK_CAND_CAP);
-                warp_append(ok1 && pair_le(e1.key, e1.idx, bkey, bidx), e1, count, cand, TK_CAND_CAP);
+            for (int g = 0; g < group_rows<NA>(); g++) {
+                if (metric_key(s.a[0], v[g][0].x) > bkey) pass &= ~(1u << (2 * g));
+                if (metric_key(s.a[0], v[g][0].y) > bkey) pass &= ~(2u << (2 * g));
             }
-        }
+            if (!__any_sync(0xFFFFFFFFu, pass)) return;                // the usual case
+#pragma unroll
+            for (int i = 0; i < 2 * group_rows<NA>(); i++) {
+                KI e;
+                e.key = metric_key(s.a[0], (i & 1) ? v[i >> 1][0].y : v[i >> 1][0].x); e.idx = r.first + j[i >> 1] + (i & 1);
+                warp_append(((pass >> i) & 1u) && pair_le(e.key, e.idx, bkey, bidx), e, count, cand, TK_CAND_CAP);
+            }
+        });
         grid_barrier();
     }
 }
@@ -560,13 +591,22 @@ __device__ __forceinline__ bool warp_best(u32 score) {
 
 struct Killers8 {
     const P2 *k;
-    // strictly dominated by one of them?  The high halves decide nearly always.
-    __device__ __forceinline__ bool kills(u64 x, u64 y) const {
-        const u32 X = (u32)(x >> 32), Y = (u32)(y >> 32);
-        bool dead = false;
+    const uint2 *hi;                                   // their high halves, which decide nearly always
+    // of n points, those whose high halves no killer's rule out (all bits of alive: the ones to ask about)
+    template <int N>
+    __device__ __forceinline__ u32 left(const u32 (&X)[N], const u32 (&Y)[N], u32 alive) const {
 #pragma unroll
-        for (u32 q = 0; q < CO_DIRS; q++) dead |= (u32)(k[q].x >> 32) < X && (u32)(k[q].y >> 32) < Y;
-        if (dead) return true;
+        for (u32 q = 0; q < CO_DIRS; q++) {
+            const uint2 h = hi[q];
+#pragma unroll
+            for (int i = 0; i < N; i++)
+                if (h.x < X[i] && h.y < Y[i]) alive &= ~(1u << i);
+        }
+        return alive;
+    }
+    // strictly dominated by one of them?
+    __device__ __forceinline__ bool kills(u64 x, u64 y) const {
+        bool dead = false;
 #pragma unroll 1
         for (u32 q = 0; q < CO_DIRS; q++) dead |= dominates(k[q].x, k[q].y, x, y);
         return dead;
@@ -602,13 +642,14 @@ __device__ __noinline__ void pareto_small(const P3 *sv, u32 n, unsigned char *fl
     if (threadIdx.x == 0) *count_out = total > GUIDE_PARETO_MAX ? 0xFFFFFFFFu : total;
 }
 
-template <int NA>
+template <int NA, bool WHOLE>
 __global__ void __launch_bounds__(CO_THREADS, CO_BLOCKS_PER_SM)
 k_pareto_coop(CoopSrc<NA> s, Range r, Walk w, u32 *header, P2 *local, P3 *surv, KI *front_list, u64 *idx_out, u32 out_cap, u32 *count_out) {
     __shared__ P3 sv[CO_P_CHUNK];
     __shared__ unsigned char flags[CO_P_CHUNK];
     __shared__ P2 best[CO_DIRS][CO_WARPS];
     __shared__ P2 ks[CO_DIRS];
+    __shared__ uint2 kh[CO_DIRS];
     __shared__ u32 s_n;
     grid_dep_wait();
     const u32 lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -624,7 +665,7 @@ k_pareto_coop(CoopSrc<NA> s, Range r, Walk w, u32 *header, P2 *local, P3 *surv, 
 #pragma unroll
         for (u32 u = 0; u < CO_ROWS; u++) {
             const u64 slot = (u64)u * total_warps + gwarp;
-            load_row(s, r.count, w.row(slot), slot < w.n_slots, lane, st[u], v[u]);
+            load_row<false>(s, r.count, w.row(slot), slot < w.n_slots, lane, st[u], v[u]);
         }
 #pragma unroll
         for (u32 u = 0; u < CO_ROWS; u++) {
@@ -653,14 +694,14 @@ k_pareto_coop(CoopSrc<NA> s, Range r, Walk w, u32 *header, P2 *local, P3 *surv, 
         P2 p; p.x = KEY_MAX; p.y = KEY_MAX;
         if (lane < CO_WARPS) p = best[warp][lane];
         if (warp_best(direction_score(p.x, p.y, direction_weight(warp)))) {
-            if (gridDim.x == 1) ks[warp] = p;
+            if (WHOLE && gridDim.x == 1) ks[warp] = p;
             else {
                 ulonglong2 e; e.x = p.x; e.y = p.y;
                 *reinterpret_cast<ulonglong2 *>(local + (size_t)warp * CO_MAX_BLOCKS + blockIdx.x) = e;
             }
         }
     }
-    if (gridDim.x > 1) {
+    if (!WHOLE || gridDim.x > 1) {
         static_assert(CO_WARPS == 2 * CO_DIRS, "two warps per direction");
         constexpr u32 PER = CO_MAX_BLOCKS / 64;
         grid_barrier();
@@ -688,49 +729,53 @@ k_pareto_coop(CoopSrc<NA> s, Range r, Walk w, u32 *header, P2 *local, P3 *surv, 
         }
     }
     __syncthreads();
-    const Killers8 K = {ks};
+    if (threadIdx.x < CO_DIRS) kh[threadIdx.x] = make_uint2((u32)(ks[threadIdx.x].x >> 32), (u32)(ks[threadIdx.x].y >> 32));
+    __syncthreads();
+    const Killers8 K = {ks, kh};
     const u32 lim = min(out_cap, GUIDE_PARETO_MAX);
     // ---- filter: the sample itself when it was everything, else one pass over the arrays ----
-    if (w.r == 1) {
+    if (WHOLE) {
+        u32 X[N_PTS], Y[N_PTS], alive = 0;
 #pragma unroll
         for (u32 i = 0; i < N_PTS; i++) {
-            const bool real = !(px[i] == KEY_MAX && py[i] == KEY_MAX);
-            if (!__any_sync(0xFFFFFFFFu, real)) continue;
+            X[i] = (u32)(px[i] >> 32); Y[i] = (u32)(py[i] >> 32);
+            alive |= (px[i] == KEY_MAX && py[i] == KEY_MAX ? 0u : 1u) << i;
+        }
+        alive = K.left(X, Y, alive);
+#pragma unroll
+        for (u32 i = 0; i < N_PTS; i++) {
+            if (!__any_sync(0xFFFFFFFFu, (alive >> i) & 1u)) continue;
             P3 e; e.x = px[i]; e.y = py[i];
             e.idx = r.first + ((u64)(i >> 1) * total_warps + gwarp) * ROW + 2 * lane + (i & 1);
-            const bool take = real && !K.kills(px[i], py[i]);
+            const bool take = ((alive >> i) & 1u) && !K.kills(px[i], py[i]);
             if (gridDim.x == 1) warp_append(take, e, &s_n, sv, CO_P_CHUNK);
             else warp_append(take, e, header + PH_COUNT, surv, PA_SURV_CAP);
         }
     } else {
-        const u64 stride = (u64)gridDim.x * CO_WARPS;
-        FilterWalk fw(w.n_rows, stride, warp * gridDim.x + blockIdx.x), ahead = fw;
-        u32 st[CO_ROWS], st_ahead[CO_ROWS];
-        load_chunk_status(s, r.count, ahead, lane, st_ahead);
-        for (; fw.more(); fw = ahead) {
+        for_live_rows<NA>(s, r.count, w.n_rows, lane, warp, header + PH_TICKET, [&](const u64 *j, const double2 (*v)[NA], u32 pass) {
+            constexpr int N = 2 * group_rows<NA>();
+            u32 X[N], Y[N];
 #pragma unroll
-            for (u32 u = 0; u < CO_ROWS; u++) st[u] = st_ahead[u];
-            ahead.next();
-            load_chunk_status(s, r.count, ahead, lane, st_ahead);
-            double2 v[CO_ROWS][NA];
-            if (!load_chunk_values(s, r.count, fw, lane, st, v)) continue;
-#pragma unroll
-            for (u32 u = 0; u < CO_ROWS; u++) {
-                bool okh[2];
-                row_ok(s, st[u], v[u], okh[0], okh[1]);
-                if (!__any_sync(0xFFFFFFFFu, okh[0] | okh[1])) continue;
-                const u64 x[2] = {metric_key(s.a[0], v[u][0].x), metric_key(s.a[0], v[u][0].y)};
-                const u64 y[2] = {metric_key(s.a[1], v[u][1].x), metric_key(s.a[1], v[u][1].y)};
-#pragma unroll
-                for (u32 h = 0; h < 2; h++) {
-                    P3 e; e.x = x[h]; e.y = y[h]; e.idx = r.first + fw.row(u) * ROW + 2 * lane + h;
-                    warp_append(okh[h] && !K.kills(x[h], y[h]), e, header + PH_COUNT, surv, PA_SURV_CAP);
-                }
+            for (int i = 0; i < N; i++) {
+                const double2 *q = v[i >> 1];
+                X[i] = (u32)(metric_key(s.a[0], (i & 1) ? q[0].y : q[0].x) >> 32);
+                Y[i] = (u32)(metric_key(s.a[1], (i & 1) ? q[1].y : q[1].x) >> 32);
             }
-        }
+            pass = K.left(X, Y, pass);
+            if (!__any_sync(0xFFFFFFFFu, pass)) return;
+#pragma unroll
+            for (int i = 0; i < N; i++) {
+                if (!__any_sync(0xFFFFFFFFu, (pass >> i) & 1u)) continue;
+                const double2 *q = v[i >> 1];
+                P3 e;
+                e.x = metric_key(s.a[0], (i & 1) ? q[0].y : q[0].x); e.y = metric_key(s.a[1], (i & 1) ? q[1].y : q[1].x);
+                e.idx = r.first + j[i >> 1] + (i & 1);
+                warp_append(((pass >> i) & 1u) && !K.kills(e.x, e.y), e, header + PH_COUNT, surv, PA_SURV_CAP);
+            }
+        });
     }
     // ---- finish ----
-    if (gridDim.x == 1) {
+    if (WHOLE && gridDim.x == 1) {
         __syncthreads();
         if (s_n > CO_P_CHUNK) { if (threadIdx.x == 0) header[1] = 1; }      // the general kernel redoes the call
         else pareto_small(sv, s_n, flags, lim, idx_out, count_out);
@@ -818,18 +863,22 @@ bool coop_select_ok() {
     if (!cached[dev]) {
         int coop = 0, t = 0, p = 0;
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&t, k_topk_coop<MAX_ARR - 1>, CO_THREADS, 0);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, k_pareto_coop<MAX_ARR>, CO_THREADS, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&t, k_topk_coop<MAX_ARR - 1, false>, CO_THREADS, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, k_pareto_coop<MAX_ARR, false>, CO_THREADS, 0);
         if (getenv("GUIDE_NO_COOPERATIVE")) coop = 0;
         cached[dev] = (coop && t >= (int)CO_BLOCKS_PER_SM && p >= (int)CO_BLOCKS_PER_SM) ? 1 : 2;
     }
     return cached[dev] == 1;
 }
 
-// One row per warp while that fills the machine; a range one block can hold in its registers is one block.
+// A range one block can hold in its registers is one block; up to what CO_BLOCKS_PER_SM blocks per SM hold, a row per
+// warp while that fills the machine.  Beyond, one block per SM: its pass over everything has enough in flight, and two
+// selections on two streams fit side by side.
 static u32 coop_grid(u64 n_rows) {
     if (n_rows <= CO_ONE_BLOCK_ROWS) return 1;
-    return (u32)std::min<u64>((n_rows + CO_WARPS - 1) / CO_WARPS, std::min<u64>((u64)num_sms() * CO_BLOCKS_PER_SM, CO_MAX_BLOCKS));
+    const u64 full = std::min<u64>((u64)num_sms() * CO_BLOCKS_PER_SM, CO_MAX_BLOCKS);
+    if (n_rows > full * CO_WARPS * CO_ROWS) return (u32)std::min<u64>((u64)num_sms(), CO_MAX_BLOCKS);
+    return (u32)std::min<u64>((n_rows + CO_WARPS - 1) / CO_WARPS, full);
 }
 
 // All rows while the warps' registers hold them, else one out of every r, as many as they hold.
@@ -865,13 +914,14 @@ static int topk_coop_na(const Arr *arr, Range r, const guide_outputs &mat, u32 k
     CoopSrc<NA> s;
     for (int i = 0; i < NA; i++) s.a[i] = arr[i];
     s.status = mat.status;
-    s.vec = mat_vec_ok(mat);
+    s.vec = mat_vec_ok(mat) ? ((uintptr_t)mat.status % 16 == 0 ? 2 : 1) : 0;
     KI *minima = reinterpret_cast<KI *>(region), *spairs = minima + CO_BOUND_LIST, *cand = spairs + CO_BOUND_LIST;
     const u64 n_rows = (r.count + ROW - 1) / ROW;
     const u32 grid = coop_grid(n_rows);
     u32 group_log2 = 0;
     while (((grid * CO_WARPS) >> group_log2) > CO_BOUND_LIST) group_log2++;
-    GUIDE_CUDA(launch_coop(k_topk_coop<NA>, grid, st, s, r, make_walk(n_rows, grid), k, group_log2, header, minima, spairs, cand, negate,
+    const Walk w = make_walk(n_rows, grid);
+    GUIDE_CUDA(launch_coop(w.r == 1 ? k_topk_coop<NA, true> : k_topk_coop<NA, false>, grid, st, s, r, w, k, group_log2, header, minima, spairs, cand, negate,
                            idx_out, key_out, count_out));
     return GUIDE_OK;
 }
@@ -897,13 +947,14 @@ static int pareto_coop_na(const Arr *arr, Range r, const guide_outputs &mat, u32
     CoopSrc<NA> s;
     for (int i = 0; i < NA; i++) s.a[i] = arr[i];
     s.status = mat.status;
-    s.vec = mat_vec_ok(mat);
+    s.vec = mat_vec_ok(mat) ? ((uintptr_t)mat.status % 16 == 0 ? 2 : 1) : 0;
     P2 *local = reinterpret_cast<P2 *>(region);
     P3 *surv = reinterpret_cast<P3 *>(region + (size_t)CO_DIRS * CO_MAX_BLOCKS * sizeof(P2));
     KI *front = reinterpret_cast<KI *>(region + (size_t)CO_DIRS * CO_MAX_BLOCKS * sizeof(P2) + (size_t)PA_SURV_CAP * sizeof(P3));
     const u64 n_rows = (r.count + ROW - 1) / ROW;
     const u32 grid = coop_grid(n_rows);
-    GUIDE_CUDA(launch_coop(k_pareto_coop<NA>, grid, st, s, r, make_walk(n_rows, grid), header, local, surv, front, idx_out, cap, count_out));
+    const Walk w = make_walk(n_rows, grid);
+    GUIDE_CUDA(launch_coop(w.r == 1 ? k_pareto_coop<NA, true> : k_pareto_coop<NA, false>, grid, st, s, r, w, header, local, surv, front, idx_out, cap, count_out));
     return GUIDE_OK;
 }
 

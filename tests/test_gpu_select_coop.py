@@ -11,7 +11,8 @@ from test_gpu_select_stream import synth, to_dev
 
 pytestmark = pytest.mark.gpu
 
-REGISTERS = 148 * 2 * 16 * 4 * 64        # configs a full grid's registers hold: beyond it one row out of every r is sampled
+REGISTERS = 148 * 2 * 16 * 4 * 64        # configs a full grid's registers hold: beyond it one row out of every r is sampled,
+SAMPLED = 148 * 16 * 4                   # ... at most this many rows
 
 
 @pytest.fixture(scope="module")
@@ -62,13 +63,14 @@ def test_infinities_nan_and_negative_zero_order_as_in_the_accumulator_kernels(sp
 
 
 def test_candidate_list_overflow_runs_the_filter_again(sp):
-    """Passing configs only in the rows the sample leaves out (one row of every two is sampled at this
-    size, at a hashed place): no bound, the survivor list overflows, and the filter repeats with a closer
+    """Passing configs only in the rows the sample leaves out (one row out of every r, at a hashed place): no bound, the survivor list overflows, and the filter repeats with a closer
     bound of what it holds until the survivors fit.  Keys fall, rise and are all equal."""
     n = 2_000_001
-    assert REGISTERS < n < 2 * REGISTERS
-    slot = np.arange(n // 64 // 2, dtype=np.uint64)
-    sampled = slot * 2 + ((slot * 2654435761) % 2**32 >> 7) % 2
+    rows = (n + 63) // 64
+    assert n > REGISTERS
+    r = -(-rows // SAMPLED)
+    slot = np.arange(rows // r, dtype=np.uint64)
+    sampled = slot * r + ((slot * 2654435761) % 2**32 >> 7) % r
     unsampled = np.setdiff1d(np.arange(n // 64), sampled)
     host = synth(n, 9)
     host["status"][:] = 2
@@ -80,3 +82,68 @@ def test_candidate_list_overflow_runs_the_filter_again(sp):
             idx, val, cnt = run_topk(sp, dev, {}, "cost_per_token", k, count=n)
             w_idx, w_val, w_cnt = oracle.select_topk(host, {}, "cost_per_token", k)
             assert cnt == w_cnt and np.array_equal(idx, w_idx) and np.array_equal(val, w_val)
+
+
+@pytest.mark.parametrize("n", [REGISTERS + 1, REGISTERS + 64 * 8 * 3 + 63, 2_097_152, 2_000_003])
+@pytest.mark.parametrize("shift", [0, 2, 4, 8])
+def test_pass_over_a_long_range(sp, n, shift):
+    """One to six arrays; status at every alignment the loads tell apart (16, 4 and no wide loads); the last chunk
+    and the last row ragged; few, many and all rows with a config that passed its memory check."""
+    import torch
+    n -= shift                               # room inside the space's size for the shifted copy
+    for frac in (0.001, 0.02, 1.0):
+        host = synth(n, 200 + n % 89, pass_frac=frac)
+        dev = to_dev(host)
+        if shift:
+            dev["status"] = torch.cat([dev["status"][:shift], dev["status"]])[shift:]
+        for cons in ({}, {"max_latency": 4.0}, {"max_latency": 6.0, "min_throughput": 100.0, "max_cost_per_hr": 50.0, "max_ttft": 0.9,
+                                               "ttft_stat": "p50"}):
+            check(sp, host, dev, cons, "cost_per_token", 64, n)
+
+
+def test_two_selections_on_two_streams_run_side_by_side():
+    """A selection over a long range leaves room for another one: two on two streams take clearly less time than
+    one after the other, and give the same answers."""
+    import torch
+    w = I.workload(5)
+    big = guide.Space(w["space"])
+    out = guide.alloc_outputs(big.size, 0, ("latency", "thr_decode", "cost_per_hr", "cost_per_token", "status"))
+    guide.guide_simulate(big, None, out)
+    dev = dict(dtype=torch.int64, device="cuda")
+    res = [[torch.zeros(64, **dev), torch.zeros(64, dtype=torch.float64, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda"),
+            torch.zeros(guide.PARETO_MAX, **dev), torch.zeros(1, dtype=torch.int32, device="cuda")] for _ in range(2)]
+    wk = torch.empty(guide.guide_select_workspace_bytes(big, 64), dtype=torch.uint8, device="cuda")
+    wp = torch.empty(guide.guide_pareto_workspace_bytes(big), dtype=torch.uint8, device="cuda")
+    main, side = torch.cuda.current_stream(), torch.cuda.Stream()
+
+    def topk(r):
+        guide.guide_select_topk(big, None, out, w["constraints"], "cost_per_token", 64, r[0], r[1], r[2], wk)
+
+    def front(r):
+        guide.guide_pareto(big, None, out, w["constraints"], "latency", "cost_per_hr", r[3], r[4], wp)
+
+    def in_turn():
+        topk(res[0])
+        front(res[0])
+
+    def beside():
+        side.wait_stream(main)
+        with torch.cuda.stream(side):
+            topk(res[1])
+        front(res[1])
+        main.wait_stream(side)
+
+    def time_of(f):
+        times = []
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(20):
+                f()
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b))
+        return min(times[1:])
+    t_turn, t_beside = time_of(in_turn), time_of(beside)
+    assert all(torch.equal(a, b) for a, b in zip(res[0], res[1]))
+    assert t_beside < 0.88 * t_turn, (t_turn, t_beside)          # 0.71 measured; 0.98 when they cannot overlap
