@@ -21,7 +21,7 @@
 //            many of them.
 //
 // Bound and killers only exclude configs that cannot be part of the answer, whatever the sample
-// looked like.  If the top-k list overflows, the bound of what it holds excludes more, and the filter
+// looked like.  If the top-k list overflows, the k-th pair is closed in on by counting and the filter
 // runs again; a Pareto list that overflows raises the redo flag and the accumulator kernel queued
 // behind (select.cu) redoes the call.
 //
@@ -447,6 +447,98 @@ __device__ __noinline__ void topk_finish(const KI *cand, u32 n, u32 k, FinishScr
     }
 }
 
+// the passing pairs within a bound, appended to a list
+template <int NA>
+__device__ __forceinline__ void topk_filter(const CoopSrc<NA> &s, const Range &r, u64 n_rows, u32 *ticket, u64 bkey, u64 bidx, u32 *count, KI *cand) {
+    for_live_rows<NA>(s, r.count, n_rows, threadIdx.x & 31, threadIdx.x >> 5, ticket, [&](const u64 *j, const double2 (*v)[NA], u32 pass) {
+#pragma unroll
+        for (int g = 0; g < group_rows<NA>(); g++) {
+            if (metric_key(s.a[0], v[g][0].x) > bkey) pass &= ~(1u << (2 * g));
+            if (metric_key(s.a[0], v[g][0].y) > bkey) pass &= ~(2u << (2 * g));
+        }
+        if (!__any_sync(0xFFFFFFFFu, pass)) return;                    // the usual case
+#pragma unroll
+        for (int i = 0; i < 2 * group_rows<NA>(); i++) {
+            KI e;
+            e.key = metric_key(s.a[0], (i & 1) ? v[i >> 1][0].y : v[i >> 1][0].x); e.idx = r.first + j[i >> 1] + (i & 1);
+            warp_append(((pass >> i) & 1u) && pair_le(e.key, e.idx, bkey, bidx), e, count, cand, TK_CAND_CAP);
+        }
+    });
+}
+
+// The survivors did not fit their list (the sample had too few passing configs, or none of the better ones).  The k-th
+// pair is then closed in on by counting: every pass makes a histogram of the passing keys in [lo, hi] over the
+// whole grid, and [lo, hi] becomes the bin the k-th of them is in: ten bits a pass, seven passes at most, and four or five
+// on the index where one key alone is too many.  It ends as soon as the pairs up to that bin's end fit the
+// list; one more pass collects them.  (Tightening the bound by what the list holds takes as many passes as the
+// list goes into the passing configs when those are met worst first.)
+// Collective over the grid; khi: the bound's key.  gbins: two histograms in the workspace.  Returns the new count.
+template <int NA>
+__device__ __noinline__ u32 topk_overflow(const CoopSrc<NA> s, const Range r, u64 n_rows, u32 k, u32 *header, unsigned long long *gbins,
+                                          KI *cand, u32 *bins, CountScratch &sc, u64 khi) {
+    static_assert(CO_BINS == 1024 && 2 * CO_BINS * sizeof(u64) <= CO_BOUND_LIST * sizeof(KI), "ten bits; two histograms in the minima's place");
+    const u32 lane = threadIdx.x & 31, warp = threadIdx.x >> 5, FULL = 0xFFFFFFFFu;
+    u64 lo = 0, hi = khi, kkey = 0, before = 0;        // before: passing pairs below lo
+    bool by_idx = false;                               // [lo, hi] are indices of configs with key kkey
+    u32 *ticket;
+    for (u32 pass = 0;; pass++) {
+        unsigned long long *g = gbins + (pass & 1) * CO_BINS;           // last read two passes ago, as the ticket
+        ticket = header + ((pass & 1) ? TK_TICKET : TK_TICKET2);
+        for (u32 i = blockIdx.x * CO_THREADS + threadIdx.x; i < CO_BINS; i += gridDim.x * CO_THREADS) g[i] = 0;
+        if (blockIdx.x == 0 && threadIdx.x == 0) *ticket = 0;
+        for (u32 i = threadIdx.x; i < CO_BINS; i += CO_THREADS) bins[i] = 0;
+        grid_barrier();
+        const u32 width = 64 - __clzll((long long)((hi - lo) | 1ull)), shift = width > 10 ? width - 10 : 0;
+        for_live_rows<NA>(s, r.count, n_rows, lane, warp, ticket, [&](const u64 *j, const double2 (*v)[NA], u32 ok) {
+#pragma unroll
+            for (int i = 0; i < 2 * group_rows<NA>(); i++) {
+                const u64 key = metric_key(s.a[0], (i & 1) ? v[i >> 1][0].y : v[i >> 1][0].x), idx = r.first + j[i >> 1] + (i & 1);
+                const u64 at = by_idx ? idx : key;
+                if (((ok >> i) & 1u) && at >= lo && at <= hi && (!by_idx || key == kkey)) atomicAdd(&bins[(at - lo) >> shift], 1u);
+            }
+        });
+        __syncthreads();
+        for (u32 i = threadIdx.x; i < CO_BINS; i += CO_THREADS)
+            if (bins[i]) atomicAdd(g + i, (unsigned long long)bins[i]);
+        grid_barrier();
+        // the bin of the k-th pair: two bins per thread
+        const u64 b0 = __ldcg(g + 2 * threadIdx.x), b1 = __ldcg(g + 2 * threadIdx.x + 1);
+        u64 incl = b0 + b1;
+        for (u32 d = 1; d < 32; d <<= 1) {
+            const u64 o = __shfl_up_sync(FULL, incl, d);
+            if (lane >= d) incl += o;
+        }
+        if (lane == 31) sc.lo[warp] = incl;
+        __syncthreads();
+        u64 off = before;
+        for (u32 q = 0; q < warp; q++) off += sc.lo[q];
+        incl += off;
+        const u64 prev = incl - b0 - b1;
+        __syncthreads();
+        if (prev < k && incl >= k) {                   // one thread
+            const bool first = prev + b0 >= k;
+            sc.hi[0] = 2 * threadIdx.x + (first ? 0 : 1);              // the bin
+            sc.hi[1] = first ? prev : prev + b0;                       // pairs below it
+            sc.hi[2] = first ? prev + b0 : incl;                       // ... and up to its end
+        }
+        __syncthreads();
+        const u64 upto = sc.hi[2], span = (1ull << shift) - 1;
+        before = sc.hi[1];
+        lo += sc.hi[0] << shift;
+        hi = hi - lo <= span ? hi : lo + span;
+        __syncthreads();
+        if (upto <= TK_CAND_CAP) break;
+        if (!by_idx && lo == hi) { by_idx = true; kkey = lo; lo = r.first; hi = r.first + r.count - 1; }
+    }
+    u32 *count = header + TK_COUNT2;                   // untouched so far
+    ticket = ticket == header + TK_TICKET ? header + TK_TICKET2 : header + TK_TICKET;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *ticket = 0;
+    grid_barrier();
+    topk_filter(s, r, n_rows, ticket, by_idx ? kkey : hi, by_idx ? hi : KEY_MAX, count, cand);
+    grid_barrier();
+    return __ldcg(count);
+}
+
 // WHOLE: the sample is everything (w.r == 1), and the one pass over the arrays is the sample's.
 template <int NA, bool WHOLE>
 __global__ void __launch_bounds__(CO_THREADS, CO_BLOCKS_PER_SM)
@@ -522,12 +614,11 @@ k_topk_coop(CoopSrc<NA> s, Range r, Walk w, u32 k, u32 group_log2, u32 *header, 
     u64 bkey, bidx;
     list_bound<CO_BOUND_LIST / CO_THREADS>(minima, n_groups, k, fin.bins, sc, bkey, bidx);
     // ---- the sample values within it: the survivors themselves, or (r > 1) the pairs of a closer bound ----
-    u32 *count = header + TK_COUNT;
 #pragma unroll
     for (u32 i = 0; i < 2 * CO_ROWS; i++) {
         KI e; e.key = key[i]; e.idx = index_of(i);
         const bool take = ((ok >> i) & 1u) && pair_le(e.key, e.idx, bkey, bidx);
-        if (WHOLE) warp_append(take, e, count, cand, TK_CAND_CAP);
+        if (WHOLE) warp_append(take, e, header + TK_COUNT, cand, TK_CAND_CAP);
         else warp_append(take, e, header + TK_SAMPLED, spairs, CO_BOUND_LIST);
     }
     grid_barrier();
@@ -537,39 +628,15 @@ k_topk_coop(CoopSrc<NA> s, Range r, Walk w, u32 k, u32 group_log2, u32 *header, 
         const u32 ns = min(__ldcg(header + TK_SAMPLED), CO_BOUND_LIST);
         if (ns >= k) list_bound<CO_BOUND_LIST / CO_THREADS>(spairs, ns, k, fin.bins, sc, bkey, bidx);
     }
-    // ---- filter passes over everything: none when the sample was everything and its survivors fit ----
-    u32 *ticket = header + TK_TICKET;
-    for (bool first_pass = !WHOLE;; first_pass = false) {
-        if (!first_pass) {
-            const u32 n = __ldcg(count);
-            if (n <= TK_CAND_CAP) {
-                if (blockIdx.x == 0) topk_finish(cand, n, k, fin, sc, negate, idx_out, key_out, count_out);
-                return;
-            }
-            // the list overflowed: k pairs of what it holds are within a bound that excludes more
-            list_bound<CO_BOUND_LIST / CO_THREADS>(cand, TK_CAND_CAP, k, fin.bins, sc, bkey, bidx);
-            // the other pair of counters: last read two barriers ago
-            count = count == header + TK_COUNT ? header + TK_COUNT2 : header + TK_COUNT;
-            ticket = ticket == header + TK_TICKET ? header + TK_TICKET2 : header + TK_TICKET;
-            if (blockIdx.x == 0 && threadIdx.x == 0) *count = *ticket = 0;
-            grid_barrier();
-        }
-        for_live_rows<NA>(s, r.count, w.n_rows, lane, warp, ticket, [&](const u64 *j, const double2 (*v)[NA], u32 pass) {
-#pragma unroll
-            for (int g = 0; g < group_rows<NA>(); g++) {
-                if (metric_key(s.a[0], v[g][0].x) > bkey) pass &= ~(1u << (2 * g));
-                if (metric_key(s.a[0], v[g][0].y) > bkey) pass &= ~(2u << (2 * g));
-            }
-            if (!__any_sync(0xFFFFFFFFu, pass)) return;                // the usual case
-#pragma unroll
-            for (int i = 0; i < 2 * group_rows<NA>(); i++) {
-                KI e;
-                e.key = metric_key(s.a[0], (i & 1) ? v[i >> 1][0].y : v[i >> 1][0].x); e.idx = r.first + j[i >> 1] + (i & 1);
-                warp_append(((pass >> i) & 1u) && pair_le(e.key, e.idx, bkey, bidx), e, count, cand, TK_CAND_CAP);
-            }
-        });
+    // ---- filter: the sample's own survivors when it was everything, else one pass over the arrays ----
+    if (!WHOLE) {
+        topk_filter(s, r, w.n_rows, header + TK_TICKET, bkey, bidx, header + TK_COUNT, cand);
         grid_barrier();
     }
+    u32 n = __ldcg(header + TK_COUNT);
+    if (n > TK_CAND_CAP)
+        n = topk_overflow(s, r, w.n_rows, k, header, reinterpret_cast<unsigned long long *>(minima), cand, fin.bins, sc, bkey);
+    if (blockIdx.x == 0) topk_finish(cand, n, k, fin, sc, negate, idx_out, key_out, count_out);
 }
 
 // ---- Pareto ------------------------------------------------------------------------------------------

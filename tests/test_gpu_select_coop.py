@@ -62,10 +62,8 @@ def test_infinities_nan_and_negative_zero_order_as_in_the_accumulator_kernels(sp
         assert np.array_equal(a_val.view(np.uint64), b_val[:128].view(np.uint64))
 
 
-def test_candidate_list_overflow_runs_the_filter_again(sp):
-    """Passing configs only in the rows the sample leaves out (one row out of every r, at a hashed place): no bound, the survivor list overflows, and the filter repeats with a closer
-    bound of what it holds until the survivors fit.  Keys fall, rise and are all equal."""
-    n = 2_000_001
+def hidden_from_the_sample(n):
+    """Passing configs only in the rows the sample leaves out (one row out of every r, at a hashed place)."""
     rows = (n + 63) // 64
     assert n > REGISTERS
     r = -(-rows // SAMPLED)
@@ -75,13 +73,83 @@ def test_candidate_list_overflow_runs_the_filter_again(sp):
     host = synth(n, 9)
     host["status"][:] = 2
     host["status"][(unsampled[:, None] * 64 + np.arange(64)).ravel()] = 0
-    for keys in (np.arange(n, dtype=np.float64), -np.arange(n, dtype=np.float64), np.ones(n)):
+    return host
+
+
+def test_candidate_list_overflow_runs_the_filter_again(sp):
+    """No bound from the sample: the survivor list overflows, the k-th pair is closed in on by counting and the
+    filter repeats.  Keys fall, rise, are all equal, share their high bits, few and many of each."""
+    n = 2_000_001
+    host = hidden_from_the_sample(n)
+    rng = np.random.default_rng(3)
+    for keys in (np.arange(n, dtype=np.float64), -np.arange(n, dtype=np.float64), np.ones(n), 1.0 + np.arange(n)[::-1] * 2.0**-52,
+                 rng.permutation(n) * 2.0**-1074, np.floor(rng.random(n) * 4.0) - 2.0, rng.standard_normal(n) * 1e300,
+                 np.where(rng.random(n) < 0.02, 1.0, 2.0), np.where(np.arange(n) % 2_000 == 7, -np.inf, np.inf)):
         host["cost_per_token"] = keys
         dev = to_dev(host)
         for k in (1, 128):
             idx, val, cnt = run_topk(sp, dev, {}, "cost_per_token", k, count=n)
             w_idx, w_val, w_cnt = oracle.select_topk(host, {}, "cost_per_token", k)
             assert cnt == w_cnt and np.array_equal(idx, w_idx) and np.array_equal(val, w_val)
+    cons = {"max_latency": 6.0, "min_throughput": 100.0, "max_cost_per_hr": 50.0, "max_ttft": 0.9, "ttft_stat": "p50"}
+    host["cost_per_token"] = np.arange(n, dtype=np.float64)
+    idx, val, cnt = run_topk(sp, to_dev(host), cons, "cost_per_token", 64, count=n)
+    w_idx, w_val, w_cnt = oracle.select_topk(host, cons, "cost_per_token", 64)
+    assert cnt == w_cnt and np.array_equal(idx, w_idx) and np.array_equal(val, w_val)
+
+
+def test_overflow_inside_the_registers(sp):
+    """The sample is everything, but too few groups of it have a passing config for a bound."""
+    n = 1_000_003
+    host = synth(n, 31)
+    host["status"][:] = 2
+    live = np.arange(10, 310)                # 19,200 configs in neighbouring rows: more than the list holds
+    host["status"][(live[:, None] * 64 + np.arange(64)).ravel()] = 0
+    for keys in (np.arange(n, dtype=np.float64), -np.arange(n, dtype=np.float64), np.ones(n)):
+        host["cost_per_token"] = keys
+        dev = to_dev(host)
+        for k in (1, 64, 128):
+            idx, val, cnt = run_topk(sp, dev, {}, "cost_per_token", k, count=n)
+            w_idx, w_val, w_cnt = oracle.select_topk(host, {}, "cost_per_token", k)
+            assert cnt == w_cnt and np.array_equal(idx, w_idx) and np.array_equal(val, w_val)
+
+
+def test_overflow_takes_few_passes():
+    """Keys that rise with the index are met worst first by a pass that starts at the end of the range.  The number
+    of passes must not grow with the length of the range: 268 M configs, 2.4 GB."""
+    import torch
+    space = dict(I.workload(5)["space"])
+    for name in ("hw", "hw_mem"):
+        space[name] = np.concatenate([space[name]] * 16)
+    sp = guide.Space(space)
+    n = sp.size
+    assert n == 1 << 28
+    rows = n // 64
+    r = -(-rows // SAMPLED)
+    slot = torch.arange(rows // r, dtype=torch.int64, device="cuda")
+    sampled = slot * r + ((slot * 2654435761) % 2**32 >> 7) % r
+    status = torch.zeros(rows, 64, dtype=torch.uint8, device="cuda")
+    status[sampled] = 2
+    dev = {"status": status.reshape(-1), "cost_per_token": torch.arange(n, dtype=torch.float64, device="cuda")}
+    plain = dict(dev, status=torch.zeros_like(dev["status"]))
+    idx, val = torch.zeros(64, dtype=torch.int64, device="cuda"), torch.zeros(64, dtype=torch.float64, device="cuda")
+    cnt = torch.zeros(1, dtype=torch.int32, device="cuda")
+    ws = torch.empty(guide.guide_select_workspace_bytes(sp, 64), dtype=torch.uint8, device="cuda")
+
+    def time_of(d):
+        times = []
+        for _ in range(4):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            guide.guide_select_topk(sp, None, d, {}, "cost_per_token", 64, idx, val, cnt, ws)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b))
+        want = torch.nonzero(d["status"][:1 << 16] == 0)[:64, 0]
+        assert int(cnt.item()) == 64 and torch.equal(idx, want) and torch.equal(val, want.double())
+        return min(times[1:])
+    t_plain, t_hidden = time_of(plain), time_of(dev)
+    assert t_hidden < 30 * t_plain, (t_plain, t_hidden)
 
 
 @pytest.mark.parametrize("n", [REGISTERS + 1, REGISTERS + 64 * 8 * 3 + 63, 2_097_152, 2_000_003])
