@@ -133,7 +133,7 @@ inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 bl
 // Pareto: word 0 ticket of the per-warp kernel, word 1 redo flag, word 2 ticket of the general kernel;
 //         words 4..: the streaming path's tickets, survivor count, killer count and front count.
 enum { TK_TICKET = 2, TK_COUNT = 3, TK_REDO = 4, TK_SAMPLED = 5, TK_BOUND = 6, TK_TICKET2 = 10, TK_COUNT2 = 11 };
-enum { PH_TICKET = 4, PH_COUNT = 5, PH_KILLERS = 6, PH_FRONT = 7, PH_TICKET2 = 8 };
+enum { PH_TICKET = 4, PH_COUNT = 5, PH_KILLERS = 6, PH_FRONT = 7, PH_TICKET2 = 8, PH_COUNT2 = 9 };
 
 // ---- one-launch path over materialised metrics (select_coop.cu) ------------------------------------
 // A sample gives a bound (top-k) or a small set of dominating points (Pareto); one pass then keeps the

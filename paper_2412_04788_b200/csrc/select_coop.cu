@@ -13,7 +13,7 @@
 //            histogram of the encoded keys).  With r > 1 the sample pairs within it are gathered and
 //            give, in the same way, a bound close to the sample's own k-th pair.  Pareto: the extreme
 //            points of eight directions, over the lane, the warp, the block and, after a barrier, all
-//            blocks ("killers").
+//            blocks ("killers"); over long ranges, after another one, a staircase of the sample's points.
 //   filter : a config survives if it passes the constraints and its pair is within the bound, or no
 //            killer strictly dominates it.  With r = 1 the values are still in registers, otherwise
 //            one pass over the arrays.  Survivors go to a list in the workspace.
@@ -22,21 +22,24 @@
 //
 // Bound and killers only exclude configs that cannot be part of the answer, whatever the sample
 // looked like.  If the top-k list overflows, the k-th pair is closed in on by counting and the filter
-// runs again; a Pareto list that overflows raises the redo flag and the accumulator kernel queued
-// behind (select.cu) redoes the call.
+// runs again.  A Pareto list of many goes through a staircase of its own points, as do the arrays again when
+// it overflowed; only when it overflows a second time (fronts beyond the most a call reports, or thousands of equal
+// points) the redo flag is raised and the accumulator kernel queued behind (select.cu) redoes the call.
 //
 // Ranges of up to 2048 configs are one block: its barriers are block barriers and nothing goes
 // through the workspace.
 //
 // Blocks per SM: ranges whose rows all fit the warps' registers (1.2 M configs) take two, and their kernels have no
-// pass over the arrays in them (WHOLE: half the code, 983,040 configs 25 -> 19 us top-k, 25 -> 23 front).  Longer
+// pass over the arrays in them (WHOLE: half the code, 983,040 configs 25 -> 18 us top-k).  Longer
 // ranges take one.  A cooperative launch starts only when all of its blocks have room, so with two per SM two
-// selections on two streams run one after the other: 16.8 M configs, sweep and both selections, 334 us against 289
+// selections on two streams run one after the other: 16.8 M configs, sweep and both selections, 334 us against 285
 // with one, 2.2 M 124 against 100.  On one stream one block per SM costs nothing that a pass with more in flight does
-// not give back (16.8 M: 63 + 79 us with two, 67 + 78 with one; 2.2 M: 33 + 39 and 33 + 33).
+// not give back (16.8 M: 64 + 79 us with two, 66 + 80 with one; 2.2 M: 33 + 39 and 33 + 34).
 //
 // Top-k + front on a B200 against chains of kernels (sample, refined bound, filter, rank, gated fallback): 983,040
-// configs 19 + 23 us instead of 35 + 34; 30,720 configs 17 + 17 instead of 68 + 42; 16.8 M 67 + 78 instead of 65 + 83.
+// configs 18 + 25 us instead of 35 + 34; 30,720 configs 17 + 17 instead of 68 + 42; 16.8 M 66 + 80 instead of 65 + 83.
+// Fronts of two continuous metrics (14.7 M): TTFT against cost per token 88 instead of 123, TTFT against throughput 92
+// instead of 195; eight killers alone let more through than the list holds, and the call was done twice (588, 560).
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
@@ -57,6 +60,11 @@ static constexpr u32 CO_BINS = 2 * CO_THREADS;  // bins of a histogram
 static constexpr u32 CO_RANKED = 256;           // pairs the finishing block ranks by counting (at least two threads each)
 static constexpr u32 CO_DIRS = 8;               // killers of a Pareto call
 static constexpr u32 CO_P_DIRECT = 128;         // survivors one block compares all against all
+static constexpr u32 CO_P_REFINE = 1024;        // more survivors than these are filtered once more
+static constexpr u32 CO_STEPS = 2 * CO_THREADS; // steps of a staircase
+static constexpr u32 CO_STAIR_RATIO = 12;       // the sample makes a staircase from one row of so many on (7 M configs): it costs
+                                                // 3-6 us and saves the filter a second pass (14.7 M, TTFT against throughput: 89 us
+                                                // with, 240 without; 4.2 M, latency against cost: 44 with, 39 without)
 static constexpr u32 CO_P_CHUNK = 1024;         // survivors staged in shared memory at a time
 static constexpr u32 CO_MAX_BLOCKS = 512;       // workspace for the blocks' killer candidates
 static_assert(CO_ONE_BLOCK_ROWS * ROW <= CO_LIST && CO_LIST % CO_THREADS == 0, "one block's whole range fits its list");
@@ -66,7 +74,17 @@ struct CoopSrc {
     Arr a[NA];        // entry 0 is the key (top-k) or x (Pareto), entry 1 is y (Pareto only)
     const uint8_t *status;
     int vec;          // every array is 16-byte aligned, status 4-byte (2: 16-byte too); 0: no wide loads
+    // the bounds once more, as one comparison each: v, its sign flipped by flip, is at most bnd (unless free)
+    double bnd[NA];
+    u32 flip[NA], free[NA];
 };
+
+__device__ __forceinline__ double flipped(double v, u32 mask) { return __hiloint2double(__double2hiint(v) ^ (int)mask, __double2loint(v)); }
+// the high half of metric_key, or, for a zero of the other sign, a little less
+__device__ __forceinline__ u32 metric_key_high(const Arr &a, double v) {
+    const u32 h = (u32)__double2hiint(v) ^ (a.neg ? 0x80000000u : 0u);
+    return h ^ ((u32)((int)h >> 31) | 0x80000000u);
+}
 
 // The sample: groups of r consecutive rows, one row of each, at a hashed offset so that it does not
 // lock onto a period of the config index.
@@ -109,9 +127,9 @@ __device__ __forceinline__ void row_ok(const CoopSrc<NA> &s, u32 st, const doubl
     ok0 = (st & 0xFFu) == 0;
     ok1 = (st >> 8) == 0;
 #pragma unroll
-    for (int a = 0; a < NA; a++) {
-        ok0 &= within(s.a[a], v[a].x);
-        ok1 &= within(s.a[a], v[a].y);
+    for (int a = 0; a < NA; a++) {                     // a NaN fails an active bound
+        ok0 &= s.free[a] || flipped(v[a].x, s.flip[a]) <= s.bnd[a];
+        ok1 &= s.free[a] || flipped(v[a].y, s.flip[a]) <= s.bnd[a];
     }
 }
 
@@ -450,11 +468,14 @@ __device__ __noinline__ void topk_finish(const KI *cand, u32 n, u32 k, FinishScr
 // the passing pairs within a bound, appended to a list
 template <int NA>
 __device__ __forceinline__ void topk_filter(const CoopSrc<NA> &s, const Range &r, u64 n_rows, u32 *ticket, u64 bkey, u64 bidx, u32 *count, KI *cand) {
+    // first by the bound's value: what compares greater has a greater key (a NaN does not compare)
+    const double bval = dec(bkey);
+    const u32 neg = s.a[0].neg ? 0x80000000u : 0u;
     for_live_rows<NA>(s, r.count, n_rows, threadIdx.x & 31, threadIdx.x >> 5, ticket, [&](const u64 *j, const double2 (*v)[NA], u32 pass) {
 #pragma unroll
         for (int g = 0; g < group_rows<NA>(); g++) {
-            if (metric_key(s.a[0], v[g][0].x) > bkey) pass &= ~(1u << (2 * g));
-            if (metric_key(s.a[0], v[g][0].y) > bkey) pass &= ~(2u << (2 * g));
+            if (flipped(v[g][0].x, neg) > bval) pass &= ~(1u << (2 * g));
+            if (flipped(v[g][0].y, neg) > bval) pass &= ~(2u << (2 * g));
         }
         if (!__any_sync(0xFFFFFFFFu, pass)) return;                    // the usual case
 #pragma unroll
@@ -709,18 +730,135 @@ __device__ __noinline__ void pareto_small(const P3 *sv, u32 n, unsigned char *fl
     if (threadIdx.x == 0) *count_out = total > GUIDE_PARETO_MAX ? 0xFFFFFFFFu : total;
 }
 
+// Eight points guard the hull of a front only: of two continuous metrics thousands of points behind its concave stretches
+// survive them (TTFT against cost per token on 14.7 M configs 21,557, for a front of 42).  Behind them stands a
+// staircase: the range of x between the killers in equal parts of the encoded metric (what is left and right of it
+// apart), and on every step the smallest y of the points seen there.  A point with a y no smaller than one on a lower step
+// is out: that one is real, and its x is smaller.
+struct Staircase {
+    u64 xlo, xhi;
+    u32 shift;
+    const u64 *low;                                    // shared: per step, the smallest y of all lower ones; null: no staircase
+    __device__ __forceinline__ explicit Staircase(const Killers8 &K) : low(nullptr) {
+        xlo = KEY_MAX; xhi = 0;
+        for (u32 q = 0; q < CO_DIRS; q++) {
+            const P2 p = K.k[q];
+            if (p.x == KEY_MAX && p.y == KEY_MAX) continue;
+            xlo = p.x < xlo ? p.x : xlo; xhi = p.x > xhi ? p.x : xhi;
+        }
+        if (xlo > xhi) { xlo = 0; xhi = KEY_MAX; }     // no killer: the sample had no passing config
+        const u32 width = 64 - __clzll((long long)((xhi - xlo) | 1ull));
+        shift = width > 10 ? width - 10 : 0;
+    }
+    __device__ __forceinline__ u32 step(u64 x) const {
+        if (x <= xlo) return 0;
+        if (x >= xhi) return CO_STEPS - 1;
+        return 1 + ((u32)((x - xlo - 1) >> shift) * (CO_STEPS - 2) >> 10);
+    }
+    __device__ __forceinline__ void put(unsigned long long *g, u64 x, u64 y) const { atomicMin(g + step(x), y); }
+    // after a barrier: g's minima into shared memory, each step with those of all lower ones
+    __device__ __forceinline__ void read(const unsigned long long *g, u64 *steps, u64 *part) {
+        static_assert(CO_STEPS == 2 * CO_THREADS, "two steps per thread");
+        const u32 lane = threadIdx.x & 31, warp = threadIdx.x >> 5, FULL = 0xFFFFFFFFu;
+        const u64 e0 = __ldcg(g + 2 * threadIdx.x), e1 = __ldcg(g + 2 * threadIdx.x + 1);
+        u64 incl = e0 < e1 ? e0 : e1;
+        for (u32 d = 1; d < 32; d <<= 1) {
+            const u64 o = __shfl_up_sync(FULL, incl, d);
+            if (lane >= d && o < incl) incl = o;
+        }
+        if (lane == 31) part[warp] = incl;
+        u64 below = __shfl_up_sync(FULL, incl, 1);
+        if (lane == 0) below = KEY_MAX;
+        __syncthreads();
+        for (u32 q = 0; q < warp; q++) below = part[q] < below ? part[q] : below;
+        steps[2 * threadIdx.x] = below;
+        steps[2 * threadIdx.x + 1] = e0 < below ? e0 : below;
+        __syncthreads();
+        low = steps;
+    }
+    __device__ __forceinline__ bool behind(u64 x, u64 y) const {
+        if (!low) return false;
+        const u64 l = low[step(x)];
+        return l <= y && l != KEY_MAX;
+    }
+};
+
+// the passing points that no killer dominates and that are not behind the staircase, appended to a list
+template <int NA>
+__device__ __forceinline__ void pareto_filter(const CoopSrc<NA> &s, const Range &r, u64 n_rows, u32 *ticket, const Killers8 &K, const Staircase &S,
+                                              u32 *count, P3 *surv) {
+    for_live_rows<NA>(s, r.count, n_rows, threadIdx.x & 31, threadIdx.x >> 5, ticket, [&](const u64 *j, const double2 (*v)[NA], u32 pass) {
+        constexpr int N = 2 * group_rows<NA>();
+        u32 X[N], Y[N];
+#pragma unroll
+        for (int i = 0; i < N; i++) {
+            const double2 *q = v[i >> 1];
+            X[i] = metric_key_high(s.a[0], (i & 1) ? q[0].y : q[0].x);
+            Y[i] = metric_key_high(s.a[1], (i & 1) ? q[1].y : q[1].x);
+        }
+        pass = K.left(X, Y, pass);
+        if (!__any_sync(0xFFFFFFFFu, pass)) return;
+#pragma unroll
+        for (int i = 0; i < N; i++) {
+            if (!__any_sync(0xFFFFFFFFu, (pass >> i) & 1u)) continue;
+            const double2 *q = v[i >> 1];
+            P3 e;
+            e.x = metric_key(s.a[0], (i & 1) ? q[0].y : q[0].x); e.y = metric_key(s.a[1], (i & 1) ? q[1].y : q[1].x);
+            e.idx = r.first + j[i >> 1] + (i & 1);
+            warp_append(((pass >> i) & 1u) && !S.behind(e.x, e.y) && !K.kills(e.x, e.y), e, count, surv, PA_SURV_CAP);
+        }
+    });
+}
+
+// Still many survivors: they go into the staircase themselves, and it filters their list, or, when that overflowed, the
+// arrays again (the stored part of the list still is made of real points).  Collective over the grid; steps and part: shared.
+// Returns the new count.
+template <int NA, bool WHOLE>
+__device__ __noinline__ u32 pareto_refine(const CoopSrc<NA> s, const Range r, u64 n_rows, u32 n, u32 *header, const Killers8 K,
+                                          unsigned long long *gsteps, const P3 *surv, P3 *kept, u64 *steps, u64 *part) {
+    const u32 threads = gridDim.x * CO_THREADS, m = min(n, PA_SURV_CAP);
+    const u64 *words = reinterpret_cast<const u64 *>(surv);
+    Staircase S(K);
+    if (WHOLE) {                                       // made here: few ranges this short need it
+        if (blockIdx.x == 0) gsteps[threadIdx.x] = gsteps[threadIdx.x + CO_THREADS] = KEY_MAX;
+        grid_barrier();
+    }
+    for (u32 i = blockIdx.x * CO_THREADS + threadIdx.x; i < m; i += threads)
+        S.put(gsteps, __ldcg(words + 3 * (size_t)i), __ldcg(words + 3 * (size_t)i + 1));
+    grid_barrier();
+    S.read(gsteps, steps, part);
+    if (n <= PA_SURV_CAP) {
+        for (u32 i0 = blockIdx.x * CO_THREADS; i0 < m; i0 += threads) {
+            const u32 i = i0 + threadIdx.x;
+            P3 e; e.x = e.y = e.idx = 0;
+            if (i < m) { e.x = __ldcg(words + 3 * (size_t)i); e.y = __ldcg(words + 3 * (size_t)i + 1); e.idx = __ldcg(words + 3 * (size_t)i + 2); }
+            warp_append(i < m && !S.behind(e.x, e.y), e, header + PH_COUNT2, kept, PA_SURV_CAP);
+        }
+    } else {
+        pareto_filter(s, r, n_rows, header + PH_TICKET2, K, S, header + PH_COUNT2, kept);
+    }
+    grid_barrier();
+    return __ldcg(header + PH_COUNT2);
+}
+
 template <int NA, bool WHOLE>
 __global__ void __launch_bounds__(CO_THREADS, CO_BLOCKS_PER_SM)
-k_pareto_coop(CoopSrc<NA> s, Range r, Walk w, u32 *header, P2 *local, P3 *surv, KI *front_list, u64 *idx_out, u32 out_cap, u32 *count_out) {
+k_pareto_coop(CoopSrc<NA> s, Range r, Walk w, u32 *header, P2 *local, P3 *surv, P3 *kept, unsigned long long *gsteps, KI *front_list, u64 *idx_out,
+              u32 out_cap, u32 *count_out) {
     __shared__ P3 sv[CO_P_CHUNK];
     __shared__ unsigned char flags[CO_P_CHUNK];
     __shared__ P2 best[CO_DIRS][CO_WARPS];
     __shared__ P2 ks[CO_DIRS];
     __shared__ uint2 kh[CO_DIRS];
+    __shared__ u64 part[CO_WARPS];
+    static_assert(sizeof(sv) >= CO_STEPS * sizeof(u64), "the steps' place until the finish");
+    u64 *const steps = reinterpret_cast<u64 *>(sv);
     __shared__ u32 s_n;
     grid_dep_wait();
     const u32 lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // nothing reads these before the first barrier
     if (blockIdx.x == 0 && threadIdx.x < 64) header[threadIdx.x] = 0;
+    if (!WHOLE && blockIdx.x == gridDim.x - 1) gsteps[threadIdx.x] = gsteps[threadIdx.x + CO_THREADS] = KEY_MAX;
     if (threadIdx.x == 0) s_n = 0;
     // ---- sample ----
     const u32 total_warps = gridDim.x * CO_WARPS, gwarp = blockIdx.x * CO_WARPS + warp;
@@ -761,8 +899,10 @@ k_pareto_coop(CoopSrc<NA> s, Range r, Walk w, u32 *header, P2 *local, P3 *surv, 
         P2 p; p.x = KEY_MAX; p.y = KEY_MAX;
         if (lane < CO_WARPS) p = best[warp][lane];
         if (warp_best(direction_score(p.x, p.y, direction_weight(warp)))) {
-            if (WHOLE && gridDim.x == 1) ks[warp] = p;
-            else {
+            if (WHOLE && gridDim.x == 1) {
+                ks[warp] = p;
+                kh[warp] = make_uint2((u32)(p.x >> 32), (u32)(p.y >> 32));
+            } else {
                 ulonglong2 e; e.x = p.x; e.y = p.y;
                 *reinterpret_cast<ulonglong2 *>(local + (size_t)warp * CO_MAX_BLOCKS + blockIdx.x) = e;
             }
@@ -792,23 +932,26 @@ k_pareto_coop(CoopSrc<NA> s, Range r, Walk w, u32 *header, P2 *local, P3 *surv, 
         if (threadIdx.x < CO_DIRS) {
             const P2 a = best[threadIdx.x][0], b = best[threadIdx.x][1];
             const u32 wt = direction_weight(threadIdx.x);
-            ks[threadIdx.x] = direction_score(b.x, b.y, wt) < direction_score(a.x, a.y, wt) ? b : a;
+            const P2 p = direction_score(b.x, b.y, wt) < direction_score(a.x, a.y, wt) ? b : a;
+            ks[threadIdx.x] = p;
+            kh[threadIdx.x] = make_uint2((u32)(p.x >> 32), (u32)(p.y >> 32));
         }
     }
     __syncthreads();
-    if (threadIdx.x < CO_DIRS) kh[threadIdx.x] = make_uint2((u32)(ks[threadIdx.x].x >> 32), (u32)(ks[threadIdx.x].y >> 32));
-    __syncthreads();
     const Killers8 K = {ks, kh};
     const u32 lim = min(out_cap, GUIDE_PARETO_MAX);
-    // ---- filter: the sample itself when it was everything, else one pass over the arrays ----
-    if (WHOLE) {
+    // ---- filter: the sample itself when it was everything; else it makes the staircase, and one pass over the arrays ----
+    auto sample_left = [&]() {
         u32 X[N_PTS], Y[N_PTS], alive = 0;
 #pragma unroll
         for (u32 i = 0; i < N_PTS; i++) {
             X[i] = (u32)(px[i] >> 32); Y[i] = (u32)(py[i] >> 32);
             alive |= (px[i] == KEY_MAX && py[i] == KEY_MAX ? 0u : 1u) << i;
         }
-        alive = K.left(X, Y, alive);
+        return __any_sync(0xFFFFFFFFu, alive) ? K.left(X, Y, alive) : 0u;
+    };
+    if (WHOLE) {
+        const u32 alive = sample_left();
 #pragma unroll
         for (u32 i = 0; i < N_PTS; i++) {
             if (!__any_sync(0xFFFFFFFFu, (alive >> i) & 1u)) continue;
@@ -819,27 +962,16 @@ k_pareto_coop(CoopSrc<NA> s, Range r, Walk w, u32 *header, P2 *local, P3 *surv, 
             else warp_append(take, e, header + PH_COUNT, surv, PA_SURV_CAP);
         }
     } else {
-        for_live_rows<NA>(s, r.count, w.n_rows, lane, warp, header + PH_TICKET, [&](const u64 *j, const double2 (*v)[NA], u32 pass) {
-            constexpr int N = 2 * group_rows<NA>();
-            u32 X[N], Y[N];
+        Staircase S(K);
+        if (w.r >= CO_STAIR_RATIO) {
+            const u32 alive = sample_left();
 #pragma unroll
-            for (int i = 0; i < N; i++) {
-                const double2 *q = v[i >> 1];
-                X[i] = (u32)(metric_key(s.a[0], (i & 1) ? q[0].y : q[0].x) >> 32);
-                Y[i] = (u32)(metric_key(s.a[1], (i & 1) ? q[1].y : q[1].x) >> 32);
-            }
-            pass = K.left(X, Y, pass);
-            if (!__any_sync(0xFFFFFFFFu, pass)) return;
-#pragma unroll
-            for (int i = 0; i < N; i++) {
-                if (!__any_sync(0xFFFFFFFFu, (pass >> i) & 1u)) continue;
-                const double2 *q = v[i >> 1];
-                P3 e;
-                e.x = metric_key(s.a[0], (i & 1) ? q[0].y : q[0].x); e.y = metric_key(s.a[1], (i & 1) ? q[1].y : q[1].x);
-                e.idx = r.first + j[i >> 1] + (i & 1);
-                warp_append(((pass >> i) & 1u) && !K.kills(e.x, e.y), e, header + PH_COUNT, surv, PA_SURV_CAP);
-            }
-        });
+            for (u32 i = 0; i < N_PTS; i++)
+                if ((alive >> i) & 1u) S.put(gsteps, px[i], py[i]);
+            grid_barrier();
+            S.read(gsteps, steps, part);
+        }
+        pareto_filter(s, r, w.n_rows, header + PH_TICKET, K, S, header + PH_COUNT, surv);
     }
     // ---- finish ----
     if (WHOLE && gridDim.x == 1) {
@@ -849,7 +981,11 @@ k_pareto_coop(CoopSrc<NA> s, Range r, Walk w, u32 *header, P2 *local, P3 *surv, 
         return;
     }
     grid_barrier();
-    const u32 n = __ldcg(header + PH_COUNT);
+    u32 n = __ldcg(header + PH_COUNT);
+    if (n > CO_P_REFINE) {
+        n = pareto_refine<NA, WHOLE>(s, r, w.n_rows, n, header, K, gsteps, surv, kept, steps, part);
+        surv = kept;
+    }
     if (n > PA_SURV_CAP) {
         if (blockIdx.x == 0 && threadIdx.x == 0) header[1] = 1;
         return;
@@ -972,16 +1108,30 @@ static cudaError_t launch_coop(void (*kernel)(KArgs...), u32 grid, cudaStream_t 
 
 // workspace region of a top-k call: KI minima[CO_BOUND_LIST] | KI spairs[CO_BOUND_LIST] | KI cand[TK_CAND_CAP]
 size_t topk_coop_bytes() { return ((size_t)2 * CO_BOUND_LIST + TK_CAND_CAP) * sizeof(KI); }
-// ... and of a Pareto call: P2 local[CO_DIRS][CO_MAX_BLOCKS] | P3 surv[PA_SURV_CAP] | KI front[PA_SURV_CAP]
-size_t pareto_coop_bytes() { return (size_t)CO_DIRS * CO_MAX_BLOCKS * sizeof(P2) + (size_t)PA_SURV_CAP * (sizeof(P3) + sizeof(KI)); }
+// ... and of a Pareto call: P2 local[CO_DIRS][CO_MAX_BLOCKS] | P3 surv[PA_SURV_CAP] | P3 kept[PA_SURV_CAP] |
+// KI front[PA_SURV_CAP] | u64 steps[CO_STEPS]
+static constexpr size_t PC_SURV = (size_t)CO_DIRS * CO_MAX_BLOCKS * sizeof(P2), PC_KEPT = PC_SURV + (size_t)PA_SURV_CAP * sizeof(P3),
+                        PC_FRONT = PC_KEPT + (size_t)PA_SURV_CAP * sizeof(P3), PC_STEPS = PC_FRONT + (size_t)PA_SURV_CAP * sizeof(KI);
+size_t pareto_coop_bytes() { return PC_STEPS + CO_STEPS * sizeof(u64); }
+
+template <int NA>
+static CoopSrc<NA> coop_src(const Arr *arr, const guide_outputs &mat) {
+    CoopSrc<NA> s;
+    for (int i = 0; i < NA; i++) {
+        s.a[i] = arr[i];
+        s.free[i] = arr[i].cmp == 0;
+        s.flip[i] = arr[i].cmp == 2 ? 0x80000000u : 0u;
+        s.bnd[i] = arr[i].cmp == 2 ? -arr[i].bound : arr[i].bound;
+    }
+    s.status = mat.status;
+    s.vec = mat_vec_ok(mat) ? ((uintptr_t)mat.status % 16 == 0 ? 2 : 1) : 0;
+    return s;
+}
 
 template <int NA>
 static int topk_coop_na(const Arr *arr, Range r, const guide_outputs &mat, u32 k, int negate, u32 *header, unsigned char *region,
                         u64 *idx_out, double *key_out, u32 *count_out, cudaStream_t st) {
-    CoopSrc<NA> s;
-    for (int i = 0; i < NA; i++) s.a[i] = arr[i];
-    s.status = mat.status;
-    s.vec = mat_vec_ok(mat) ? ((uintptr_t)mat.status % 16 == 0 ? 2 : 1) : 0;
+    const CoopSrc<NA> s = coop_src<NA>(arr, mat);
     KI *minima = reinterpret_cast<KI *>(region), *spairs = minima + CO_BOUND_LIST, *cand = spairs + CO_BOUND_LIST;
     const u64 n_rows = (r.count + ROW - 1) / ROW;
     const u32 grid = coop_grid(n_rows);
@@ -1011,17 +1161,16 @@ int launch_topk_coop(Range r, const guide_outputs &mat, const guide_constraints 
 template <int NA>
 static int pareto_coop_na(const Arr *arr, Range r, const guide_outputs &mat, u32 *header, unsigned char *region, u64 *idx_out,
                           u32 cap, u32 *count_out, cudaStream_t st) {
-    CoopSrc<NA> s;
-    for (int i = 0; i < NA; i++) s.a[i] = arr[i];
-    s.status = mat.status;
-    s.vec = mat_vec_ok(mat) ? ((uintptr_t)mat.status % 16 == 0 ? 2 : 1) : 0;
+    const CoopSrc<NA> s = coop_src<NA>(arr, mat);
     P2 *local = reinterpret_cast<P2 *>(region);
-    P3 *surv = reinterpret_cast<P3 *>(region + (size_t)CO_DIRS * CO_MAX_BLOCKS * sizeof(P2));
-    KI *front = reinterpret_cast<KI *>(region + (size_t)CO_DIRS * CO_MAX_BLOCKS * sizeof(P2) + (size_t)PA_SURV_CAP * sizeof(P3));
+    P3 *surv = reinterpret_cast<P3 *>(region + PC_SURV), *kept = reinterpret_cast<P3 *>(region + PC_KEPT);
+    KI *front = reinterpret_cast<KI *>(region + PC_FRONT);
+    unsigned long long *steps = reinterpret_cast<unsigned long long *>(region + PC_STEPS);
     const u64 n_rows = (r.count + ROW - 1) / ROW;
     const u32 grid = coop_grid(n_rows);
     const Walk w = make_walk(n_rows, grid);
-    GUIDE_CUDA(launch_coop(w.r == 1 ? k_pareto_coop<NA, true> : k_pareto_coop<NA, false>, grid, st, s, r, w, header, local, surv, front, idx_out, cap, count_out));
+    GUIDE_CUDA(launch_coop(w.r == 1 ? k_pareto_coop<NA, true> : k_pareto_coop<NA, false>, grid, st, s, r, w, header, local, surv, kept, steps, front,
+                           idx_out, cap, count_out));
     return GUIDE_OK;
 }
 

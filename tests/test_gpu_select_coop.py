@@ -215,3 +215,62 @@ def test_two_selections_on_two_streams_run_side_by_side():
     t_turn, t_beside = time_of(in_turn), time_of(beside)
     assert all(torch.equal(a, b) for a, b in zip(res[0], res[1]))
     assert t_beside < 0.88 * t_turn, (t_turn, t_beside)          # 0.71 measured; 0.98 when they cannot overlap
+
+
+def continuous_space():
+    """14.7 M configs under a budget of eight GPUs: long stretches of these fronts are concave in the logarithms."""
+    seed = 1014
+    dp, tp = I.hybrid_axis(8)
+    hw, mem = I.seeded_hw(seed, 20, mem_choices=[24, 48, 80, 192])
+    fw_f, fw_i = I.seeded_fw(seed, 4)
+    return {"models": I.seeded_models(seed, 16), "hw": hw, "hw_mem": mem, "fw_f": fw_f, "fw_i": fw_i,
+            "batch": np.array([1, 2, 3, 5, 8, 16, 31, 64, 100, 256, 509, 1024], dtype=np.uint32), "tp": np.array(tp, dtype=np.uint32),
+            "dp": np.array(dp, dtype=np.uint32), "pairs": np.array(I.pairs_grid(I.LEN_GRID_8, I.LEN_GRID_8), dtype=np.uint32)}
+
+
+def test_fronts_of_continuous_metrics_are_not_done_twice():
+    """Pairs of metrics without few distinct values: the filter must leave so few that the list holds them (word 1
+    of the workspace tells the kernel behind to redo the call), over long ranges and ranges held in registers."""
+    import torch
+    sp = guide.Space(continuous_space())
+    assert sp.size == 14_745_600
+    fields = ("latency", "ttft", "tpot", "thr_decode", "cost_per_hr", "cost_per_token", "status")
+    out = guide.alloc_outputs(sp.size, 0, fields)
+    guide.guide_simulate(sp, None, out)
+    ws = torch.empty(guide.guide_pareto_workspace_bytes(sp), dtype=torch.uint8, device="cuda")
+    idx = torch.empty(guide.PARETO_MAX, dtype=torch.int64, device="cuda")
+    cnt = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for n in (sp.size, 8_000_000, 2_000_000, 1_200_000, 500_000):
+        part = {k: v[:n] for k, v in out.items()}
+        host = {k: v.cpu().numpy() for k, v in part.items()}
+        host["ttft_p50"] = host["ttft_p99"] = host["ttft"]
+        for x, y in (("ttft", "cost_per_token"), ("ttft", "throughput"), ("tpot", "cost_per_token"), ("latency", "cost_per_token"),
+                     ("cost_per_hr", "throughput"), ("throughput", "cost_per_token"), ("latency", "cost_per_hr")):
+            guide.guide_pareto(sp, None, part, {}, x, y, idx, cnt, ws, count=n)
+            torch.cuda.synchronize()
+            assert int(ws[:8].view(torch.int32)[1].item()) == 0, (n, x, y)
+            want, size = oracle.pareto(host, {}, x, y, cap=guide.PARETO_MAX)
+            assert int(cnt.item()) == size and np.array_equal(idx[:size].cpu().numpy().view(np.uint64), want), (n, x, y)
+
+
+@pytest.mark.parametrize("n", [40_000, REGISTERS, REGISTERS + 1, 2_000_001])
+def test_staircase_steps(sp, n):
+    """Fronts that put every point on a step of its own, many points on one step, duplicates of x and of y, a front that
+    fills the list and one that does not fit it: the refined filter against the oracle."""
+    rng = np.random.default_rng(n)
+    host = synth(n, 40 + n % 7, pass_frac=0.9)
+    t = rng.random(n)
+    for x, y in ((t, 1.0 - t + 0.3 * rng.random(n)),                       # a straight front: nothing is killed by its ends
+                 (1.0 + t, 1.0 / (1.0 + t) * (1.0 + rng.random(n))),             # hyperbola
+                 (np.floor(t * 3000.0), 1.0 - t + 0.1 * rng.random(n)),          # 3,000 values of x
+                 (t, np.floor((1.0 - t + 0.1 * rng.random(n)) * 500.0)),         # 500 values of y
+                 (np.where(t < 0.5, 1.0, 1e300 * t), np.where(t < 0.5, rng.random(n), 1e-300)),
+                 (-t, t * 4.0 + 0.01 * rng.random(n))):
+        host["latency"], host["cost_per_token"] = np.ascontiguousarray(x), np.ascontiguousarray(y)
+        dev = to_dev(host)
+        fidx, fcnt = run_pareto(sp, dev, {}, "latency", "cost_per_token", count=n)
+        want, size = oracle.pareto(host, {}, "latency", "cost_per_token", cap=guide.PARETO_MAX)
+        if size > guide.PARETO_MAX:
+            assert fcnt == 0xFFFFFFFF, (n, size)
+        else:
+            assert fcnt == size and np.array_equal(fidx, want), (n, size)
