@@ -1019,8 +1019,10 @@ int launch_topk(const DSpace &s, Range r, const guide_outputs *mat, int time_mod
     unsigned char *w = (unsigned char *)ws;
     if (mat) {
         MatSource src{*mat, make_cons(c), key, -1, mat_vec_ok(*mat)};
-        if (k <= STREAM_TOPK_MAX_K && coop_select_ok())
-            return launch_topk_coop(r, *mat, c, key, k, (u32 *)w, w + topk_stream_offset(k), idx_out, key_out, count_out, st);
+        if (k <= STREAM_TOPK_MAX_K && coop_select_ok()) {
+            const int rc = launch_topk_coop(r, *mat, c, key, k, (u32 *)w, w + topk_stream_offset(k), idx_out, key_out, count_out, st);
+            if (rc != COOP_REFUSED) return rc;
+        }
         return run_topk_scan(src, r, k, negate, SEL_MAX_BLOCKS, w, idx_out, key_out, count_out, st);
     }
     TileGeom g;
@@ -1121,10 +1123,10 @@ int launch_pareto(const DSpace &s, Range r, const guide_outputs *mat, int time_m
         MatSource src{*mat, make_cons(c), xm, ym, mat_vec_ok(*mat)};
         if (coop_select_ok()) {
             // one launch, then the general kernel gated on the redo flag (header word 1)
-            int rc = launch_pareto_coop(r, *mat, c, xm, ym, (u32 *)ws, (unsigned char *)ws + pareto_stream_offset(), idx_out, cap,
-                                        count_out, st);
-            if (rc) return rc;
-            return run_pareto_general(src, r, idx_out, cap, count_out, ws, st);
+            const int rc = launch_pareto_coop(r, *mat, c, xm, ym, (u32 *)ws, (unsigned char *)ws + pareto_stream_offset(), idx_out, cap,
+                                              count_out, st);
+            if (rc == GUIDE_OK) return run_pareto_general(src, r, idx_out, cap, count_out, ws, st);
+            if (rc != COOP_REFUSED) return rc;
         }
         return run_pareto_scan(src, r, idx_out, cap, count_out, ws, st);
     }

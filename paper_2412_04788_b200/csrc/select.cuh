@@ -1,6 +1,9 @@
 // Shared by the selection kernels (select.cu: accumulator-based scans and the fused kernels;
 // select_stream.cu: the sampled-bound streaming path over materialised metrics).
 #pragma once
+#include <cstdlib>
+#include <cstring>
+
 #include "guide_internal.cuh"
 
 namespace guide {
@@ -127,6 +130,34 @@ inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 bl
     return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
 
+// ---- cooperative launches ------------------------------------------------------------------------
+// All blocks of the grid are resident at once, or the launch is refused: where the process has fewer SMs to itself than
+// the device has (a partition, a limit on its share), a grid that suits the device does not fit.  Such a call takes the
+// kernels that need no cooperation.  Setting GUIDE_NO_COOPERATIVE in the environment takes every call there from the
+// start; set to "refuse", the launches ask for more blocks than any device holds and are refused by CUDA (the tests use both).
+static constexpr int COOP_REFUSED = 1;         // beside GUIDE_OK and the (negative) errors
+inline const char *coop_override() {
+    static const char *const v = getenv("GUIDE_NO_COOPERATIVE");
+    return v;
+}
+inline bool coop_disabled() { return coop_override() && strcmp(coop_override(), "refuse") != 0; }
+template <class... KArgs, class... Args>
+inline int launch_cooperative(void (*kernel)(KArgs...), u32 grid, u32 block, cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(coop_override() ? 1u << 20 : grid); cfg.blockDim = dim3(block); cfg.dynamicSmemBytes = 0; cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {
+        (void)cudaGetLastError();
+        return COOP_REFUSED;
+    }
+    GUIDE_CUDA(e);
+    return GUIDE_OK;
+}
+
 // ---- workspace headers (first 256 bytes of a selection workspace, zeroed at the start of a call) ----
 // top-k:  u64 at word 0: complement of the grid-wide key bound of the per-warp accumulators (0 = none);
 //         words 2..: the streaming path's tickets, candidate and sample counts, redo flag and (two u64 at word 6) its bound pair.
@@ -144,6 +175,7 @@ size_t topk_coop_bytes();
 size_t pareto_coop_bytes();
 int launch_topk_coop(Range r, const guide_outputs &mat, const guide_constraints &c, int key, u32 k, u32 *header,
                      unsigned char *region, u64 *idx_out, double *key_out, u32 *count_out, cudaStream_t st);
+// (both: or COOP_REFUSED, with nothing launched)
 // raises header word 1 when the survivors do not fit its list: the general kernel queued behind is gated on it
 int launch_pareto_coop(Range r, const guide_outputs &mat, const guide_constraints &c, int xm, int ym, u32 *header,
                        unsigned char *region, u64 *idx_out, u32 cap, u32 *count_out, cudaStream_t st);

@@ -41,8 +41,8 @@
 // Fronts of two continuous metrics (14.7 M): TTFT against cost per token 88 instead of 123, TTFT against throughput 92
 // instead of 195; eight killers alone let more through than the list holds, and the call was done twice (588, 560).
 #include <algorithm>
+#include <atomic>
 #include <cmath>
-#include <cstdlib>
 
 #include <cooperative_groups.h>
 
@@ -1056,11 +1056,9 @@ static int collect_arrays(const guide_outputs &o, const guide_constraints &c, in
     return n;
 }
 
-// Does the device launch cooperatively, with CO_BLOCKS_PER_SM blocks resident per SM?  Asked once per
-// device.  Setting GUIDE_NO_COOPERATIVE in the environment takes every call to the accumulator kernels
-// (the tests use it to cover both).
+// Does the device launch cooperatively, with CO_BLOCKS_PER_SM blocks resident per SM?  Asked once per device.
 bool coop_select_ok() {
-    static int cached[64] = {};                      // 0 unknown, 1 yes, 2 no
+    static std::atomic<int> cached[64] = {};         // 0 unknown, 1 yes, 2 no
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
     if (!cached[dev]) {
@@ -1068,8 +1066,7 @@ bool coop_select_ok() {
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&t, k_topk_coop<MAX_ARR - 1, false>, CO_THREADS, 0);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, k_pareto_coop<MAX_ARR, false>, CO_THREADS, 0);
-        if (getenv("GUIDE_NO_COOPERATIVE")) coop = 0;
-        cached[dev] = (coop && t >= (int)CO_BLOCKS_PER_SM && p >= (int)CO_BLOCKS_PER_SM) ? 1 : 2;
+        cached[dev] = (coop && !coop_disabled() && t >= (int)CO_BLOCKS_PER_SM && p >= (int)CO_BLOCKS_PER_SM) ? 1 : 2;
     }
     return cached[dev] == 1;
 }
@@ -1095,15 +1092,10 @@ static Walk make_walk(u64 n_rows, u32 grid) {
 }
 
 template <class... KArgs, class... Args>
-static cudaError_t launch_coop(void (*kernel)(KArgs...), u32 grid, cudaStream_t st, Args... args) {
-    if (grid == 1) return launch_dependent(kernel, 1, CO_THREADS, 0, st, args...);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(CO_THREADS); cfg.dynamicSmemBytes = 0; cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeCooperative;
-    at[0].val.cooperative = 1;
-    cfg.attrs = at; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+static int launch_coop(void (*kernel)(KArgs...), u32 grid, cudaStream_t st, Args... args) {
+    if (grid > 1) return launch_cooperative(kernel, grid, CO_THREADS, st, args...);
+    GUIDE_CUDA(launch_dependent(kernel, 1, CO_THREADS, 0, st, args...));
+    return GUIDE_OK;
 }
 
 // workspace region of a top-k call: KI minima[CO_BOUND_LIST] | KI spairs[CO_BOUND_LIST] | KI cand[TK_CAND_CAP]
@@ -1138,9 +1130,8 @@ static int topk_coop_na(const Arr *arr, Range r, const guide_outputs &mat, u32 k
     u32 group_log2 = 0;
     while (((grid * CO_WARPS) >> group_log2) > CO_BOUND_LIST) group_log2++;
     const Walk w = make_walk(n_rows, grid);
-    GUIDE_CUDA(launch_coop(w.r == 1 ? k_topk_coop<NA, true> : k_topk_coop<NA, false>, grid, st, s, r, w, k, group_log2, header, minima, spairs, cand, negate,
-                           idx_out, key_out, count_out));
-    return GUIDE_OK;
+    return launch_coop(w.r == 1 ? k_topk_coop<NA, true> : k_topk_coop<NA, false>, grid, st, s, r, w, k, group_log2, header, minima, spairs, cand, negate,
+                           idx_out, key_out, count_out);
 }
 
 int launch_topk_coop(Range r, const guide_outputs &mat, const guide_constraints &c, int key, u32 k, u32 *header,
@@ -1169,9 +1160,8 @@ static int pareto_coop_na(const Arr *arr, Range r, const guide_outputs &mat, u32
     const u64 n_rows = (r.count + ROW - 1) / ROW;
     const u32 grid = coop_grid(n_rows);
     const Walk w = make_walk(n_rows, grid);
-    GUIDE_CUDA(launch_coop(w.r == 1 ? k_pareto_coop<NA, true> : k_pareto_coop<NA, false>, grid, st, s, r, w, header, local, surv, kept, steps, front,
-                           idx_out, cap, count_out));
-    return GUIDE_OK;
+    return launch_coop(w.r == 1 ? k_pareto_coop<NA, true> : k_pareto_coop<NA, false>, grid, st, s, r, w, header, local, surv, kept, steps, front,
+                           idx_out, cap, count_out);
 }
 
 int launch_pareto_coop(Range r, const guide_outputs &mat, const guide_constraints &c, int xm, int ym, u32 *header,

@@ -27,8 +27,8 @@
 // Loads are laid out so that a warp reads 512 contiguous bytes of each array per instruction (a
 // thread takes two consecutive configs, 16 bytes).
 #include <algorithm>
+#include <atomic>
 #include <cmath>
-#include <cstdlib>
 
 #include <cooperative_groups.h>
 
@@ -695,19 +695,17 @@ static Sample make_sample(u64 n_rows, u32 want_rows, u32 max_r) {
 }
 
 // Can the bound kernel's grid (TK_SAMPLE_BLOCKS blocks of SEL_THREADS threads) be resident at once on
-// the current device, and does the device launch cooperatively?  Asked once per device.  Setting
-// GUIDE_NO_COOPERATIVE in the environment forces the two-kernel form (the tests use it to cover both).
+// the current device, and does the device launch cooperatively?  Asked once per device.
 template <int NA>
 static bool cooperative_ok() {
-    static int cached[64] = {};                      // 0 unknown, 1 yes, 2 no
+    static std::atomic<int> cached[64] = {};         // 0 unknown, 1 yes, 2 no
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
     if (!cached[dev]) {
         int coop = 0, per_sm = 0;
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_topk_bound<NA>, SEL_THREADS, 0);
-        if (getenv("GUIDE_NO_COOPERATIVE")) coop = 0;
-        cached[dev] = (coop && (u64)per_sm * num_sms() >= TK_SAMPLE_BLOCKS) ? 1 : 2;
+        cached[dev] = (coop && !coop_disabled() && (u64)per_sm * num_sms() >= TK_SAMPLE_BLOCKS) ? 1 : 2;
     }
     return cached[dev] == 1;
 }
@@ -852,19 +850,16 @@ static int topk_fused_t(const DSpace &s, int tp_model, const guide_constraints &
     src.a[0] = Arr{f.a0, 0.0, 0, 0};                         // pick_metric has negated the throughput already
     src.status = f.pass;
     src.row_base = f.row_base;
-    if (cooperative_ok<1>()) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(TK_SAMPLE_BLOCKS); cfg.blockDim = dim3(SEL_THREADS); cfg.dynamicSmemBytes = 0; cfg.stream = st;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeCooperative;
-        at[0].val.cooperative = 1;
-        cfg.attrs = at; cfg.numAttrs = 1;
-        GUIDE_CUDA(cudaLaunchKernelEx(&cfg, k_topk_bound<1>, src, sm, (u64)0, k, header, minima, spairs));
-    } else {
+    rc = COOP_REFUSED;
+    if (cooperative_ok<1>())
+        rc = launch_cooperative(k_topk_bound<1>, TK_SAMPLE_BLOCKS, SEL_THREADS, st, src, sm, (u64)0, k, header, minima, spairs);
+    if (rc == COOP_REFUSED) {
         GUIDE_CUDA(cudaMemsetAsync(header, 0, 256, st));
         k_topk_sample<1><<<TK_SAMPLE_BLOCKS, SEL_THREADS, 0, st>>>(src, sm, (u64)0, k, header, minima);
         GUIDE_CUDA(cudaGetLastError());
         GUIDE_CUDA(launch_dependent(k_topk_refine<1>, TK_SAMPLE_BLOCKS, SEL_THREADS, 0, st, src, sm, (u64)0, k, header, spairs));
+    } else if (rc) {
+        return rc;
     }
     const u32 n_chunks = (s.n_h * s.n_f + MODEL_CHUNK - 1) / MODEL_CHUNK;
     cudaLaunchConfig_t cfg;

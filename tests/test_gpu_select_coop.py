@@ -274,3 +274,47 @@ def test_staircase_steps(sp, n):
             assert fcnt == 0xFFFFFFFF, (n, size)
         else:
             assert fcnt == size and np.array_equal(fidx, want), (n, size)
+
+
+def without_cooperation(value):
+    """Selections of a process that cannot launch cooperatively (the library reads the variable once)."""
+    import os
+    import subprocess
+    import sys
+    code = (
+        "import sys; sys.path.insert(0, 'tests')\n"
+        "import numpy as np, oracle\n"
+        "import test_gpu_select_coop as t\n"
+        "from gpu_util import run_pareto, run_simulate_select, run_topk\n"
+        "from paper_2412_04788_b200 import guide, inputs as I\n"
+        "sp = guide.Space(I.workload(5, scale=0.125)['space'])\n"
+        "for n, seed in ((2049, 20), (70_001, 21), (1_310_785, 22)):\n"
+        "    host = t.synth(n, seed); dev = t.to_dev(host)\n"
+        "    for cons, key, k in (({'max_latency': 6.0}, 'cost_per_token', 64), ({}, 'cost_per_hr', 128), ({}, 'throughput', 1)):\n"
+        "        t.check(sp, host, dev, cons, key, k, n)\n"
+        "w = I.workload(2, scale=0.5)\n"
+        "sp2 = guide.Space(w['space'])\n"
+        "want = oracle.simulate(w['space'])\n"
+        "for cons in ({}, {'max_latency': 20.0}):\n"
+        "    for key, k in (('cost_per_token', 64), ('cost_per_hr', 128), ('latency', 1)):\n"
+        "        idx, val, cnt = run_topk(sp2, None, cons, key, k)\n"
+        "        w_idx, w_val, w_cnt = oracle.select_topk(want, cons, key, k)\n"
+        "        assert cnt == w_cnt and np.array_equal(idx, w_idx) and np.array_equal(val, w_val), (cons, key, k)\n"
+        "    f, n = run_pareto(sp2, None, cons, 'latency', 'cost_per_hr')\n"
+        "    w_f, w_n = oracle.pareto(want, cons, 'latency', 'cost_per_hr', cap=guide.PARETO_MAX)\n"
+        "    assert n == w_n and np.array_equal(f, w_f)\n"
+        "    _, (idx, val, cnt), (f, n), _, _ = run_simulate_select(w['space'], cons, 'cost_per_token', 64, cons, 'latency', 'cost_per_hr')\n"
+        "    w_idx, _, w_cnt = oracle.select_topk(want, cons, 'cost_per_token', 64)\n"
+        "    assert cnt == w_cnt and np.array_equal(idx, w_idx) and n == w_n and np.array_equal(f, w_f)\n"
+        "print('selections ok')\n")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    res = subprocess.run([sys.executable, "-c", code], cwd=root, env=dict(os.environ, GUIDE_NO_COOPERATIVE=value),
+                         capture_output=True, text=True, timeout=600)
+    assert res.returncode == 0 and "selections ok" in res.stdout, res.stdout[-2000:] + res.stderr[-2000:]
+
+
+@pytest.mark.parametrize("value", ["1", "refuse"])
+def test_selections_without_cooperative_launches(value):
+    """Taken to the other kernels from the start, or after CUDA has refused the launch (more blocks than fit): the
+    materialised selections to the accumulator kernels, the fused top-k to its bound in two kernels."""
+    without_cooperation(value)
