@@ -422,6 +422,7 @@ int trace_on_device(guide_trace *t, DTrace *out, cudaStream_t st) {
     d.view.sum_out = t->sum_out;
     d.view.sum_in = t->sum_in;
     d.view.n_zero = t->n_zero;
+    d.view.together = t->together;
     d.block.used_on(CudaDevice::stream_id(st));
     t->dev.push_back(d);
     *out = d.view;
@@ -641,6 +642,18 @@ int guide_trace_load(const double *arrival, const uint32_t *in_len, const uint32
             t->sum_out += out_len[i];
             t->sum_in += in_len[i];
         } else t->n_zero++;
+    }
+    if (!rc) {
+        std::vector<uint32_t> len;                             // output lengths: the largest group of equal ones
+        for (uint64_t i = 0; i < n; i++)
+            if (in_len[i]) len.push_back(out_len[i]);
+        std::sort(len.begin(), len.end());
+        uint64_t most = t->n_zero;                             // these all take the config's
+        for (size_t i = 0, run = 0; i < len.size(); i++) {
+            run = i && len[i] == len[i - 1] ? run + 1 : 1;
+            most = std::max<uint64_t>(most, run);
+        }
+        t->together = 2 * most >= n;
     }
     if (rc) { delete t; return rc; }
     *out = t;

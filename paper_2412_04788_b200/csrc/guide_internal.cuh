@@ -58,7 +58,7 @@ struct guide_space {
 struct guide_trace {
     std::vector<double> arrival;
     std::vector<uint32_t> in_len, out_len;
-    uint32_t max_in = 0, max_out = 0, max_tokens = 0, n_zero = 0;
+    uint32_t max_in = 0, max_out = 0, max_tokens = 0, n_zero = 0, together = 0;
     uint64_t sum_out = 0, sum_in = 0;
     std::mutex mu;
     std::vector<guide::DeviceTrace> dev;

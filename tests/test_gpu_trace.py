@@ -293,3 +293,35 @@ def test_single_request_and_single_config():
     got, *_ = run_simulate(sp, tr, per_request=True)
     assert_parity(got, want, fields=guide.F64_OUTPUTS + ("req_ttft", "req_tpot"))
     assert got["n_iters"][0] == 1 and got["thr_decode"][0] == 0.0 and np.isinf(got["cost_per_token"][0])
+
+
+@pytest.mark.parametrize("mix", ["config's lengths", "one length", "three quarters", "half", "just under half"])
+@pytest.mark.parametrize("kv_block", [1, 16, 48, 100])
+def test_requests_that_end_together(mix, kv_block):
+    """Equal output lengths admitted together end with one iteration, by the hundred: retired at once, next to requests
+    that stay; alone, in groups around the limit, and with evictions between (little memory)."""
+    rng = np.random.default_rng(len(mix) + kv_block)
+    n = 300
+    base = I.workload(1)["space"]
+    s = {k: np.array(v, copy=True) for k, v in base.items() if isinstance(v, np.ndarray)}
+    s["batch"] = np.array([1, 4, 5, 6, 7, 12, 31, 32, 33, 64, 100, 255, 256], dtype=np.uint32)
+    s["pairs"] = np.array([(40, 1), (40, 2), (100, 33), (17, 70)], dtype=np.uint32)
+    s["fw_i"][:, 1] = kv_block
+    in_len = rng.integers(20, 60, n).astype(np.uint32)
+    out_len = rng.integers(1, 90, n).astype(np.uint32)
+    if mix == "config's lengths":
+        in_len[:] = 0
+        out_len[:] = 0
+    else:
+        share = {"one length": n, "three quarters": 225, "half": 150, "just under half": 145}[mix]
+        out_len[rng.choice(n, share, replace=False)] = 37
+    for arrival in (np.zeros(n), np.sort(np.floor(rng.random(n) * 4.0) * 0.5)):
+        tr = {"arrival": arrival, "in_len": in_len, "out_len": out_len}
+        for mem in (None, 15 * 10 ** 9):
+            q = dict(s)
+            if mem:
+                q["hw_mem"] = np.full_like(s["hw_mem"], mem)
+            want = oracle.simulate(q, tr, per_request=True)
+            got, *_ = run_simulate(q, tr, per_request=True)
+            assert_parity(got, want, fields=guide.F64_OUTPUTS + ("req_ttft", "req_tpot"))
+            assert sum(bit_mismatches(got, want, guide.F64_OUTPUTS + ("req_ttft", "req_tpot")).values()) == 0
