@@ -22,6 +22,7 @@
 // Per-request results that outlive residency (tokens generated so far, first-token time, time per
 // output token) sit in a per-warp slice of the workspace.  The request trace is the same for every
 // config and is read through the read-only path, so it stays cache resident.
+#include <cstddef>
 #include <cstdlib>
 
 #include "guide_internal.cuh"
@@ -84,7 +85,7 @@ __device__ __forceinline__ double decode_time(double ctxd, double c_f9, double t
 }
 
 static_assert(sizeof(DModel) <= 128 && sizeof(DRate) <= 128, "a warp copies each of them with one word per lane");
-struct SlotArrays {
+struct alignas(16) SlotArrays {                // parts of it are read as double2 (an array of them keeps the alignment)
     double tbuf[32];    // times of the 32 iterations a run computes at once
     double dterm[32][4];   // decode terms (fixed tasks, all-reduce, head, activation bytes) of 32 neighbouring resident counts
     double task[7][16];    // what a prompt pass needs of each task, one per lane: see prompt_task (when the config's counts stay exact in doubles)
@@ -97,6 +98,8 @@ struct SlotArrays {
     u32 rm[SLOTS];      // request index (16 bits) << 8 | phase (6 bits) | first-ever prompt pass | waiting for its prompt pass
     u32 hist[HIST];     // residents per (cache - D) mod block
 };
+static_assert(sizeof(SlotArrays) % 16 == 0 && offsetof(SlotArrays, tbuf) % 16 == 0 && offsetof(SlotArrays, dterm) % 16 == 0, "16-byte loads");
+static_assert(SLOTS <= 256, "the search for the youngest packs the slot into eight bits beside the request index");
 
 // A prompt pass with one task per lane.  Every task time is F x ic against B x im (the sum of both for the
 // all-reduce) with F = p f and B = ((w + p a) / t + p r) m for a count p (new tokens; emitting requests
