@@ -30,10 +30,17 @@ __device__ __forceinline__ void store_metrics(const guide_outputs &o, u64 j, con
 // prompts 27.7 against 33.3 us, binary32 24.6 against 32.1, 537,922 of odd axes 16.6 against 22.7); 24
 // warps are as fast on the first and slower on the second (27.0, 26.5, 16.8).
 static constexpr u32 FLAT_THREADS = 128, FLAT_BLOCKS_PER_SM = 8;
+static constexpr u64 FLAT_MAX_CONFIGS = 0x7FFFFFFFull * 256;       // one launch; two rows of blocks from half of it on
+
+__device__ __forceinline__ u64 flat_index() { return ((u64)blockIdx.y * gridDim.x + blockIdx.x) * FLAT_THREADS + threadIdx.x; }
+static dim3 flat_grid(u64 count) {
+    const u64 blocks = (count + FLAT_THREADS - 1) / FLAT_THREADS, rows = (blocks + 0x7FFFFFFEull) / 0x7FFFFFFFull;
+    return dim3((u32)((blocks + rows - 1) / rows), (u32)rows);
+}
 
 template <int TIME_SUM>
 __global__ void __launch_bounds__(FLAT_THREADS, FLAT_BLOCKS_PER_SM) k_closed_form_flat(DSpace s, Range r, int tp_model, guide_outputs o) {
-    const u64 j = (u64)blockIdx.x * blockDim.x + threadIdx.x;
+    const u64 j = flat_index();
     if (j >= r.count) return;
     const Cfg c = decode_index(s, r.first + j);
     Metrics m;
@@ -44,7 +51,7 @@ __global__ void __launch_bounds__(FLAT_THREADS, FLAT_BLOCKS_PER_SM) k_closed_for
 // The same in binary32 (model_f32.cuh): the reduced-precision variant, values stored widened.
 template <int TIME_SUM>
 __global__ void __launch_bounds__(FLAT_THREADS, FLAT_BLOCKS_PER_SM) k_closed_form_flat_f32(DSpace s, Range r, int tp_model, guide_outputs o) {
-    const u64 j = (u64)blockIdx.x * blockDim.x + threadIdx.x;
+    const u64 j = flat_index();
     if (j >= r.count) return;
     const Cfg c = decode_index(s, r.first + j);
     Metrics m;
@@ -382,10 +389,10 @@ static int launch_split(const DSpace &s, int tp_model, const guide_outputs &o, c
 }
 
 int launch_closed_form_f32(const DSpace &s, Range r, int time_model, int tp_model, const guide_outputs &o, cudaStream_t st) {
-    const u64 blocks = (r.count + FLAT_THREADS - 1) / FLAT_THREADS;
-    if (blocks > 0x7FFFFFFFull) return fail(GUIDE_ERR_UNSUPPORTED, "range too large for one launch");
-    if (time_model) k_closed_form_flat_f32<1><<<(u32)blocks, FLAT_THREADS, 0, st>>>(s, r, tp_model, o);
-    else k_closed_form_flat_f32<0><<<(u32)blocks, FLAT_THREADS, 0, st>>>(s, r, tp_model, o);
+    if (r.count > FLAT_MAX_CONFIGS) return fail(GUIDE_ERR_UNSUPPORTED, "range too large for one launch");
+    const dim3 grid = flat_grid(r.count);
+    if (time_model) k_closed_form_flat_f32<1><<<grid, FLAT_THREADS, 0, st>>>(s, r, tp_model, o);
+    else k_closed_form_flat_f32<0><<<grid, FLAT_THREADS, 0, st>>>(s, r, tp_model, o);
     GUIDE_CUDA(cudaGetLastError());
     return GUIDE_OK;
 }
@@ -401,10 +408,10 @@ int launch_closed_form(const DSpace &s, Range r, int time_model, int tp_model, c
     TileGeom g;
     const bool tiled = r.count * 2 >= total && tiled_geometry(s, (u64)num_sms() * 16, 1ull << 30, &g);
     if (!tiled) {
-        const u64 blocks = (r.count + FLAT_THREADS - 1) / FLAT_THREADS;
-        if (blocks > 0x7FFFFFFFull) return fail(GUIDE_ERR_UNSUPPORTED, "range too large for one launch");
-        if (time_model) k_closed_form_flat<1><<<(u32)blocks, FLAT_THREADS, 0, st>>>(s, r, tp_model, o);
-        else k_closed_form_flat<0><<<(u32)blocks, FLAT_THREADS, 0, st>>>(s, r, tp_model, o);
+        if (r.count > FLAT_MAX_CONFIGS) return fail(GUIDE_ERR_UNSUPPORTED, "range too large for one launch");
+        const dim3 grid = flat_grid(r.count);
+        if (time_model) k_closed_form_flat<1><<<grid, FLAT_THREADS, 0, st>>>(s, r, tp_model, o);
+        else k_closed_form_flat<0><<<grid, FLAT_THREADS, 0, st>>>(s, r, tp_model, o);
     } else {
         const dim3 grid(g.gx, g.splits);
         if (time_model) k_closed_form_tiled<1><<<grid, g.threads, 0, st>>>(s, r, tp_model, g.hf_chunk, g.tiles_per_mb, o);

@@ -197,3 +197,28 @@ def test_full_size_sweep_sampled():
     assert bool((out["ttft"][ok] <= out["latency"][ok]).all())
     assert bool(torch.isinf(out["latency"][~ok]).all()) and bool(torch.isfinite(out["latency"][ok]).all())
     assert 0 < int(ok.sum()) < n
+
+
+def test_ranges_beyond_one_row_of_blocks():
+    """More configs than 2^31 - 1 blocks of the one-thread-per-config kernel hold are two rows of blocks (nothing is
+    written and nothing fits, so the call takes a second); past twice that the call is refused."""
+    import torch
+    n_m, n_h, n_f = 4096, 256, 256
+    base = I.workload(2, scale=0.0625)["space"]
+    rep = lambda v, n: np.resize(v, (n,) + v.shape[1:])
+    s = {"models": rep(base["models"], n_m), "hw": rep(base["hw"], n_h), "hw_mem": np.full(n_h, 10 ** 6, dtype=np.uint64),
+         "fw_f": rep(base["fw_f"], n_f), "fw_i": rep(base["fw_i"], n_f), "batch": np.arange(1, 65, dtype=np.uint32),
+         "tp": np.array([1, 2, 4, 8], dtype=np.uint32), "pairs": np.array([(64, k) for k in range(1, 10)], dtype=np.uint32)}
+    sp = guide.Space(s)
+    row, limit = 0x7FFFFFFF * 128, 0x7FFFFFFF * 256
+    assert sp.size > limit
+    guide.guide_simulate(sp, None, {}, first=5, count=row + 1000, precision=guide.PREC_F32)
+    torch.cuda.synchronize()
+    with pytest.raises(guide.GuideError) as e:
+        guide.guide_simulate(sp, None, {}, count=limit + 1, precision=guide.PREC_F32)
+    assert e.value.code == guide.GUIDE_ERR_UNSUPPORTED
+    # the last configs of a space this large, where the index needs 64 bits, through the same kernel
+    out = guide.alloc_outputs(100, 0, ("latency", "status"))
+    guide.guide_simulate(sp, None, out, first=sp.size - 100, count=100, precision=guide.PREC_F32)
+    torch.cuda.synchronize()
+    assert (out["status"] != 0).all() and torch.isinf(out["latency"]).all()
