@@ -58,13 +58,12 @@ template <int NA>
 struct Src {
     Arr a[NA];
     const uint8_t *status;
-    const u64 *row_base;   // null: entry j is config first + j.  Else the arrays hold sampled rows of 64 configs
-                           // back to back and row_base[j / 64] is the index of the row's first config.
+    const u64 *row_base;   // the arrays hold sampled rows of 64 configs back to back: index of a row's first config
 };
 
 template <int NA>
-__device__ __forceinline__ u64 cfg_index(const Src<NA> &s, u64 first, u64 j) {
-    return s.row_base ? __ldg(s.row_base + (j >> 6)) + (j & 63) : first + j;
+__device__ __forceinline__ u64 cfg_index(const Src<NA> &s, u64 j) {
+    return __ldg(s.row_base + (j >> 6)) + (j & 63);
 }
 
 // region layout, top-k: pairs minima[TK_SAMPLE_BLOCKS] | pairs spairs[TK_SKEYS_CAP] | KI cand[TK_CAND_CAP]
@@ -168,8 +167,7 @@ __device__ __forceinline__ void write_kth_pair(const ulonglong2 *sl, u32 n, u32 
 // Coarse bound: every block's smallest passing sample pair, then (last block) the k-th smallest of
 // those.  At least k passing configs, one per block, are within it.  All-ones (nothing excluded)
 // when fewer than k blocks saw a passing config.
-template <int NA>
-__global__ void __launch_bounds__(SEL_THREADS) k_topk_sample(Src<NA> s, Sample sm, u64 first, u32 k, u32 *header,
+__global__ void __launch_bounds__(SEL_THREADS) k_topk_sample(Src<1> s, Sample sm, u32 k, u32 *header,
                                                              ulonglong2 *minima) {
     __shared__ ulonglong2 sl[TK_SAMPLE_BLOCKS];
     __shared__ u32 last;
@@ -180,15 +178,15 @@ __global__ void __launch_bounds__(SEL_THREADS) k_topk_sample(Src<NA> s, Sample s
     const u64 stride = (u64)gridDim.x * n_warps;
     for (u64 c0 = (u64)warp * gridDim.x + blockIdx.x; c0 < sm.n_slots; c0 += SAMPLE_BATCH * stride) {
         u32 st[SAMPLE_BATCH];
-        double2 v[SAMPLE_BATCH][NA];
+        double2 v[SAMPLE_BATCH][1];
         u64 j[SAMPLE_BATCH];
         load_batch(s, sm, c0, stride, lane, st, v, j);
 #pragma unroll
         for (u32 u = 0; u < SAMPLE_BATCH; u++) {
             bool ok0, ok1;
             eval_pair(s, st[u], v[u], ok0, ok1);
-            if (j[u] != KEY_MAX && ok0) pair_min(bk, bi, metric_key(s.a[0], v[u][0].x), cfg_index(s, first, j[u]));
-            if (j[u] != KEY_MAX && ok1) pair_min(bk, bi, metric_key(s.a[0], v[u][0].y), cfg_index(s, first, j[u]) + 1);
+            if (j[u] != KEY_MAX && ok0) pair_min(bk, bi, metric_key(s.a[0], v[u][0].x), cfg_index(s, j[u]));
+            if (j[u] != KEY_MAX && ok1) pair_min(bk, bi, metric_key(s.a[0], v[u][0].y), cfg_index(s, j[u]) + 1);
         }
     }
     for (int d = 16; d > 0; d >>= 1)
@@ -218,8 +216,7 @@ __global__ void __launch_bounds__(SEL_THREADS) k_topk_sample(Src<NA> s, Sample s
 // Refinement: the sample's pairs within the coarse bound are gathered (few: the coarse bound is at
 // worst the k-th best row of the sample) and the last block replaces the bound by their k-th
 // smallest, the exact k-th pair of the sample (of the stored part of it, if they do not all fit).
-template <int NA>
-__global__ void __launch_bounds__(SEL_THREADS) k_topk_refine(Src<NA> s, Sample sm, u64 first, u32 k, u32 *header,
+__global__ void __launch_bounds__(SEL_THREADS) k_topk_refine(Src<1> s, Sample sm, u32 k, u32 *header,
                                                              ulonglong2 *spairs) {
     constexpr u32 PER = TK_SKEYS_SMEM / SEL_THREADS;
     __shared__ ulonglong2 sl[TK_SKEYS_SMEM];
@@ -233,7 +230,7 @@ __global__ void __launch_bounds__(SEL_THREADS) k_topk_refine(Src<NA> s, Sample s
     const u64 stride = (u64)gridDim.x * n_warps;
     for (u64 c0 = (u64)warp * gridDim.x + blockIdx.x; c0 < sm.n_slots; c0 += SAMPLE_BATCH * stride) {
         u32 st[SAMPLE_BATCH];
-        double2 v[SAMPLE_BATCH][NA];
+        double2 v[SAMPLE_BATCH][1];
         u64 j[SAMPLE_BATCH];
         load_batch(s, sm, c0, stride, lane, st, v, j);
 #pragma unroll
@@ -243,9 +240,9 @@ __global__ void __launch_bounds__(SEL_THREADS) k_topk_refine(Src<NA> s, Sample s
             const u64 key[2] = {metric_key(s.a[0], v[u][0].x), metric_key(s.a[0], v[u][0].y)};
 #pragma unroll
             for (u32 h = 0; h < 2; h++) {
-                if (j[u] != KEY_MAX && ok[h] && pair_le(key[h], cfg_index(s, first, j[u]) + h, bkey, bidx)) {
+                if (j[u] != KEY_MAX && ok[h] && pair_le(key[h], cfg_index(s, j[u]) + h, bkey, bidx)) {
                     const u32 p = atomicAdd(header + TK_SAMPLED, 1);
-                    if (p < TK_SKEYS_CAP) { ulonglong2 e; e.x = key[h]; e.y = cfg_index(s, first, j[u]) + h; spairs[p] = e; }
+                    if (p < TK_SKEYS_CAP) { ulonglong2 e; e.x = key[h]; e.y = cfg_index(s, j[u]) + h; spairs[p] = e; }
                 }
             }
         }
@@ -320,8 +317,7 @@ __global__ void __launch_bounds__(SEL_THREADS) k_topk_refine(Src<NA> s, Sample s
 // of the kernel boundary and of the "last block" selections, which here are spread over the whole
 // grid (one warp ranks one pair).  A dependent chain of short latencies, so every hand-over it
 // saves counts.  Used when the device supports cooperative launches.
-template <int NA>
-__global__ void __launch_bounds__(SEL_THREADS) k_topk_bound(Src<NA> s, Sample sm, u64 first, u32 k, u32 *header,
+__global__ void __launch_bounds__(SEL_THREADS) k_topk_bound(Src<1> s, Sample sm, u32 k, u32 *header,
                                                             ulonglong2 *minima, ulonglong2 *spairs) {
     namespace cg = cooperative_groups;
     cg::grid_group grid = cg::this_grid();
@@ -337,15 +333,15 @@ __global__ void __launch_bounds__(SEL_THREADS) k_topk_bound(Src<NA> s, Sample sm
     u64 bk = KEY_MAX, bi = KEY_MAX;
     for (u64 c0 = (u64)warp * gridDim.x + blockIdx.x; c0 < sm.n_slots; c0 += SAMPLE_BATCH * stride) {
         u32 st[SAMPLE_BATCH];
-        double2 v[SAMPLE_BATCH][NA];
+        double2 v[SAMPLE_BATCH][1];
         u64 j[SAMPLE_BATCH];
         load_batch(s, sm, c0, stride, lane, st, v, j);
 #pragma unroll
         for (u32 u = 0; u < SAMPLE_BATCH; u++) {
             bool ok0, ok1;
             eval_pair(s, st[u], v[u], ok0, ok1);
-            if (j[u] != KEY_MAX && ok0) pair_min(bk, bi, metric_key(s.a[0], v[u][0].x), cfg_index(s, first, j[u]));
-            if (j[u] != KEY_MAX && ok1) pair_min(bk, bi, metric_key(s.a[0], v[u][0].y), cfg_index(s, first, j[u]) + 1);
+            if (j[u] != KEY_MAX && ok0) pair_min(bk, bi, metric_key(s.a[0], v[u][0].x), cfg_index(s, j[u]));
+            if (j[u] != KEY_MAX && ok1) pair_min(bk, bi, metric_key(s.a[0], v[u][0].y), cfg_index(s, j[u]) + 1);
         }
     }
     for (int d = 16; d > 0; d >>= 1)
@@ -374,7 +370,7 @@ __global__ void __launch_bounds__(SEL_THREADS) k_topk_bound(Src<NA> s, Sample sm
     const u64 bkey = __ldcg(bound), bidx = __ldcg(bound + 1);
     for (u64 c0 = (u64)warp * gridDim.x + blockIdx.x; c0 < sm.n_slots; c0 += SAMPLE_BATCH * stride) {
         u32 st[SAMPLE_BATCH];
-        double2 v[SAMPLE_BATCH][NA];
+        double2 v[SAMPLE_BATCH][1];
         u64 j[SAMPLE_BATCH];
         load_batch(s, sm, c0, stride, lane, st, v, j);
 #pragma unroll
@@ -384,9 +380,9 @@ __global__ void __launch_bounds__(SEL_THREADS) k_topk_bound(Src<NA> s, Sample sm
             const u64 key[2] = {metric_key(s.a[0], v[u][0].x), metric_key(s.a[0], v[u][0].y)};
 #pragma unroll
             for (u32 h = 0; h < 2; h++) {
-                if (j[u] != KEY_MAX && ok[h] && pair_le(key[h], cfg_index(s, first, j[u]) + h, bkey, bidx)) {
+                if (j[u] != KEY_MAX && ok[h] && pair_le(key[h], cfg_index(s, j[u]) + h, bkey, bidx)) {
                     const u32 p = atomicAdd(header + TK_SAMPLED, 1);
-                    if (p < TK_SKEYS_CAP) { ulonglong2 e; e.x = key[h]; e.y = cfg_index(s, first, j[u]) + h; spairs[p] = e; }
+                    if (p < TK_SKEYS_CAP) { ulonglong2 e; e.x = key[h]; e.y = cfg_index(s, j[u]) + h; spairs[p] = e; }
                 }
             }
         }
@@ -481,8 +477,7 @@ __device__ __forceinline__ void block_lex_min(u64 &p, u64 &q, u64 (*scratch)[2])
 // seeds below) are gathered in shared memory and compared all against all; up to PA_PER_BLOCK of
 // the block's front, spread over it, go to the workspace.  The last block sorts the union and
 // sweeps it into the killer staircase: real points, ascending x, strictly falling y.
-template <int NA>
-__global__ void __launch_bounds__(SEL_THREADS) k_pareto_sample(Src<NA> s, Sample sm, u32 *header, P2 *local, u32 *local_n,
+__global__ void __launch_bounds__(SEL_THREADS) k_pareto_sample(Src<2> s, Sample sm, u32 *header, P2 *local, u32 *local_n,
                                                                P2 *killers) {
     constexpr u32 N_PTS = 2 * PA_ROWS_PER_WARP;
     __shared__ P2 list[PA_LOCAL_CAP];               // also the last block's sort buffer (PA_KILLERS entries)
@@ -499,7 +494,7 @@ __global__ void __launch_bounds__(SEL_THREADS) k_pareto_sample(Src<NA> s, Sample
 #pragma unroll
     for (u32 b = 0; b < PA_ROWS_PER_WARP / SAMPLE_BATCH; b++) {
         u32 st[SAMPLE_BATCH];
-        double2 v[SAMPLE_BATCH][NA];
+        double2 v[SAMPLE_BATCH][2];
         u64 j[SAMPLE_BATCH];
         load_batch(s, sm, (u64)warp * gridDim.x + blockIdx.x + (u64)b * SAMPLE_BATCH * stride, stride, lane, st, v, j);
 #pragma unroll
@@ -508,8 +503,8 @@ __global__ void __launch_bounds__(SEL_THREADS) k_pareto_sample(Src<NA> s, Sample
             bool ok0, ok1;
             eval_pair(s, st[u], v[u], ok0, ok1);
             px[i] = py[i] = px[i + 1] = py[i + 1] = KEY_MAX;            // "no point"
-            if (j[u] != KEY_MAX && ok0) { px[i] = metric_key(s.a[0], v[u][0].x); py[i] = metric_key(s.a[1 % NA], v[u][1 % NA].x); }
-            if (j[u] != KEY_MAX && ok1) { px[i + 1] = metric_key(s.a[0], v[u][0].y); py[i + 1] = metric_key(s.a[1 % NA], v[u][1 % NA].y); }
+            if (j[u] != KEY_MAX && ok0) { px[i] = metric_key(s.a[0], v[u][0].x); py[i] = metric_key(s.a[1], v[u][1].x); }
+            if (j[u] != KEY_MAX && ok1) { px[i + 1] = metric_key(s.a[0], v[u][0].y); py[i + 1] = metric_key(s.a[1], v[u][1].y); }
         }
     }
     // four seeds, all real points of this block: smallest (x, y), smallest (y, x), and between them
@@ -696,7 +691,6 @@ static Sample make_sample(u64 n_rows, u32 want_rows, u32 max_r) {
 
 // Can the bound kernel's grid (TK_SAMPLE_BLOCKS blocks of SEL_THREADS threads) be resident at once on
 // the current device, and does the device launch cooperatively?  Asked once per device.
-template <int NA>
 static bool cooperative_ok() {
     static std::atomic<int> cached[64] = {};         // 0 unknown, 1 yes, 2 no
     int dev = 0;
@@ -704,7 +698,7 @@ static bool cooperative_ok() {
     if (!cached[dev]) {
         int coop = 0, per_sm = 0;
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_topk_bound<NA>, SEL_THREADS, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_topk_bound, SEL_THREADS, 0);
         cached[dev] = (coop && !coop_disabled() && (u64)per_sm * num_sms() >= TK_SAMPLE_BLOCKS) ? 1 : 2;
     }
     return cached[dev] == 1;
@@ -851,13 +845,13 @@ static int topk_fused_t(const DSpace &s, int tp_model, const guide_constraints &
     src.status = f.pass;
     src.row_base = f.row_base;
     rc = COOP_REFUSED;
-    if (cooperative_ok<1>())
-        rc = launch_cooperative(k_topk_bound<1>, TK_SAMPLE_BLOCKS, SEL_THREADS, st, src, sm, (u64)0, k, header, minima, spairs);
+    if (cooperative_ok())
+        rc = launch_cooperative(k_topk_bound, TK_SAMPLE_BLOCKS, SEL_THREADS, st, src, sm, k, header, minima, spairs);
     if (rc == COOP_REFUSED) {
         GUIDE_CUDA(cudaMemsetAsync(header, 0, 256, st));
-        k_topk_sample<1><<<TK_SAMPLE_BLOCKS, SEL_THREADS, 0, st>>>(src, sm, (u64)0, k, header, minima);
+        k_topk_sample<<<TK_SAMPLE_BLOCKS, SEL_THREADS, 0, st>>>(src, sm, k, header, minima);
         GUIDE_CUDA(cudaGetLastError());
-        GUIDE_CUDA(launch_dependent(k_topk_refine<1>, TK_SAMPLE_BLOCKS, SEL_THREADS, 0, st, src, sm, (u64)0, k, header, spairs));
+        GUIDE_CUDA(launch_dependent(k_topk_refine, TK_SAMPLE_BLOCKS, SEL_THREADS, 0, st, src, sm, k, header, spairs));
     } else if (rc) {
         return rc;
     }
@@ -898,7 +892,7 @@ static int pareto_fused_t(const DSpace &s, int tp_model, const guide_constraints
     src.a[1] = Arr{f.a1, 0.0, 0, 0};
     src.status = f.pass;
     src.row_base = f.row_base;
-    k_pareto_sample<2><<<PA_SAMPLE_BLOCKS, SEL_THREADS, 0, st>>>(src, sm, header, local, local_n, killers);
+    k_pareto_sample<<<PA_SAMPLE_BLOCKS, SEL_THREADS, 0, st>>>(src, sm, header, local, local_n, killers);
     GUIDE_CUDA(cudaGetLastError());
     const u32 n_chunks = (s.n_h * s.n_f + MODEL_CHUNK - 1) / MODEL_CHUNK;
     cudaLaunchConfig_t cfg;
