@@ -7,7 +7,7 @@ A step is one pass of the whole closed-form path over the 16,777,216-config swee
 guide_simulate (memory check, task list, roofline, metrics -> 6 fp64 arrays + mask + B_max; a
 bandwidth-bound memory kernel and a model kernel for the configs that fit, side by side),
 guide_select_topk (constraint filter + top-64 by cost per token) and guide_pareto (latency vs $/h;
-both: a sampled bound, one filter pass at memory speed, an exact finish),
+each one cooperative launch: a sampled bound, one filter pass over the arrays, an exact finish),
 with the space tables already resident on the device; the two selections read the same metrics and
 run side by side on two streams.  `value` is configs per second over the K
 timed steps; the 0.89 GB of outputs a step writes and reads back exceed L2 several times over, so
@@ -432,9 +432,9 @@ def run_ours(args):
         path.fidx[:fr.numel()].copy_(fr)
         return found, fsize
 
-    # The two selections of a step read the same metrics and share nothing else: the Pareto front
-    # (the longer chain of kernels) runs on the step's stream, top-k beside it on a second one (both
-    # after guide_simulate; the next step's guide_simulate after both).
+    # The two selections of a step read the same metrics and share nothing else: the Pareto front (the
+    # longer one) runs on the step's stream, top-k beside it on a second one (both after guide_simulate;
+    # the next step's guide_simulate after both).
     main = torch.cuda.current_stream()
     side = torch.cuda.Stream()
     ev_sim = torch.cuda.Event()
@@ -495,8 +495,8 @@ def run_ours(args):
     t_topk = sum(e[1].elapsed_time(e[2]) for e in evt) * args.steps / n_turn
     t_par = sum(e[2].elapsed_time(e[3]) for e in evt) * args.steps / n_turn
     t_turn = sum(e[0].elapsed_time(e[3]) for e in evt) / n_turn
-    # the step as ONE call (guide_simulate_select: sampled bound and killers first, every config tested
-    # while its metrics are stored, survivors ranked), with the library's own events around the sweep kernels
+    # the step as ONE call (guide_simulate_select: the sweep, then both selections, on one stream), with the
+    # library's own events around the sweep kernels
     ev1 = [[torch.cuda.Event(enable_timing=True) for _ in range(4)] for _ in range(n_turn)]
     for e in ev1:
         e[1].record(); e[2].record()                  # the events handed to the library must exist
@@ -630,10 +630,9 @@ def run_ours(args):
         which = [int(x) for x in args.extras.split(",") if x]
         extras = extra_workloads(guide, torch, inputs, which, flush, hbm_peak, peak_kind, args.trace_fraction, oracle)
 
-    # simulate: memory + model kernel; top-k: bound, filter, rank and the two gated fallback kernels
-    # (scan, merge: they return at once); Pareto: sample, filter, rank and the gated general kernel;
-    # with several ranks the merge of the gathered lists (scan + merge, too short for the streaming path)
-    launches_per_step = 2 + 1 + 2 + (2 if world > 1 else 0)
+    # simulate: memory + line kernel; top-k: one launch; Pareto: one launch and the gated general kernel behind
+    # it; with several ranks the two selections over the gathered lists (one launch, one and a gated one)
+    launches_per_step = 2 + 1 + 2 + (3 if world > 1 else 0)
     line = {"metric": "configs/sec", "value": value, "unit": "configs/s", "n_gpus": world, "steps": args.steps,
             "warmup": max(args.warmup, 3), "ms_per_step": total_ms / args.steps, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",

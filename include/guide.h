@@ -227,7 +227,9 @@ const char *guide_last_error(void);
  * by n_heads, TP degrees powers of two, kv_block >= 1, reserve <= 1000, and that no FLOP or byte
  * count of the model can wrap 64 bits at the axis maxima (GUIDE_ERR_OVERFLOW).  Touches no GPU. */
 int guide_space_create(const guide_space_desc *desc, guide_space **out);
-void guide_space_destroy(guide_space *space);             /* frees host and device tables; NULL ok */
+/* Frees host and device tables; NULL ok.  Kernels of earlier calls may still be running: the device memory is
+ * freed, or kept for a later handle, so that they are not disturbed.  Allowed while a stream is being captured. */
+void guide_space_destroy(guide_space *space);
 uint64_t guide_space_size(const guide_space *space);      /* product of the axis lengths; 0 for NULL */
 /* Mixed-radix decode of a config index (host side, for reports). */
 int guide_space_decode(const guide_space *space, uint64_t idx, guide_config *out);
@@ -264,6 +266,8 @@ size_t guide_pareto_workspace_bytes(const guide_space *space);
  * the k passing configs that are smallest under (key value, config index), ascending.
  *   outputs != NULL: reads materialised metrics of configs [first, first+count) (opts gives the
  *     range the arrays cover; the metric arrays the key and the constraints need must be non-NULL).
+ *     k <= 128 is one cooperative launch whose blocks are all resident at once: beside a kernel that
+ *     fills the machine on another stream it starts when that one makes room.
  *   outputs == NULL: fused - evaluates the closed form on the fly, nothing is materialised;
  *     trace must be NULL (GUIDE_ERR_UNSUPPORTED otherwise).
  * idx_out_dev[k], key_out_dev[k], count_out_dev[1]: device.  Fewer than k passing configs is not
@@ -287,12 +291,10 @@ int guide_pareto(const guide_space *space, const guide_trace *trace, const guide
 
 /* guide_simulate (closed form), guide_select_topk and guide_pareto of the same space in one call:
  * the steps of Sec. 3.2 (memory check, performance model, selection under the constraints of Sec. 4.1)
- * as one pass.  out receives the metrics exactly as guide_simulate writes them; the two answers are
- * exactly those of the separate calls on those arrays.  What the call saves is the read-back: for a
- * whole space that goes through the line-wise kernels, a sample of configs evaluated first gives the
- * top-k bound and a set of dominating points, every config is tested against them while its metrics
- * are being stored, and only the few survivors are ranked.  Other spaces, sub-ranges and k above 128
- * run the three steps one after the other on the stream, with the same results.
+ * queued one after the other on the stream.  out receives the metrics exactly as guide_simulate writes
+ * them; the two answers are exactly those of the separate calls on those arrays.  What the call saves
+ * is the argument checks and launch preparation of two calls, and that every argument is checked before
+ * anything is queued.
  *   sel->topk_cons / pareto_cons, key, k, x_metric, y_metric: as for guide_select_topk / guide_pareto;
  *   both selections are required.  The metric arrays that the keys and the active constraints need
  *   must be present in out (as for a selection on materialised metrics).

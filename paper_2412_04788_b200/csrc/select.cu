@@ -603,13 +603,9 @@ __device__ __forceinline__ void topk_end(WarpTopK &acc, KI *smem, u32 block, u32
 }
 
 template <class Src, bool WARP>
-__global__ void __launch_bounds__(SEL_THREADS) k_topk_scan(Src src, Range r, u32 k, u32 *counts, KI *lists, u64 *gthr,
-                                                           const u32 *gate) {
+__global__ void __launch_bounds__(SEL_THREADS) k_topk_scan(Src src, Range r, u32 k, u32 *counts, KI *lists, u64 *gthr) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ u32 cnt;
-    grid_dep_launch();
-    grid_dep_wait();                            // a gated launch may have started before its predecessor finished
-    if (gate && __ldcg(gate) == 0) return;
     typename TopKPick<WARP>::type acc;
     topk_begin(acc, (KI *)smem_raw, &cnt, k, gthr);
     constexpr int ITEMS = Src::ITEMS;
@@ -900,7 +896,7 @@ k_pareto_tiled(DSpace s, Range r, int tp_model, u32 hf_chunk, u32 tiles_per_mb, 
 // top-k workspace: 256 B header | counts u32[max_blocks] | lists KI[max_blocks][k]
 static size_t topk_lists_offset(u32 max_blocks) { return 256 + ((size_t)max_blocks * 4 + 255) / 256 * 256; }
 
-// ... followed by the streaming path's region (sample results and survivor list)
+// ... followed by the region of the one-launch or of the fused form (sample results and survivor lists)
 static size_t topk_stream_offset(u32 k) {
     return (topk_lists_offset(SEL_MAX_BLOCKS) + (size_t)SEL_MAX_BLOCKS * k * sizeof(KI) + 255) / 256 * 256;
 }
@@ -954,30 +950,25 @@ static int topk_reset_header(unsigned char *ws, cudaStream_t st) {
 
 template <class Src, bool WARP>
 static int run_topk_scan_mode(const Src &src, Range r, u32 k, int negate, u32 max_blocks, unsigned char *ws, u64 *idx_out,
-                              double *key_out, u32 *count_out, const u32 *gate, cudaStream_t st) {
+                              double *key_out, u32 *count_out, cudaStream_t st) {
     u32 *counts = (u32 *)(ws + 256);
     KI *lists = (KI *)(ws + topk_lists_offset(max_blocks));
     const size_t smem = WARP ? (size_t)(SEL_THREADS / 32) * warp_seg_cap(k) * sizeof(KI) : (size_t)TOPK_CAP * sizeof(KI);
     int rc = allow_smem(k_topk_scan<Src, WARP>, smem);
     if (rc) return rc;
-    // a gated launch runs behind the streaming path, which has reset the header for the whole call
-    if (!gate && (rc = topk_reset_header(ws, st))) return rc;
-    const u32 grid = grid_for(r.count, Src::ITEMS, gate ? 1 : (WARP ? 4 : 3), max_blocks);   // gated: rarely runs, keep the launch small
-    if (gate) {
-        GUIDE_CUDA(launch_dependent(k_topk_scan<Src, WARP>, grid, SEL_THREADS, smem, st, src, r, k, counts, lists, (u64 *)ws, gate));
-    } else {
-        k_topk_scan<Src, WARP><<<grid, SEL_THREADS, smem, st>>>(src, r, k, counts, lists, (u64 *)ws, gate);
-        GUIDE_CUDA(cudaGetLastError());
-    }
-    return run_topk_merge(grid, k, negate, counts, lists, idx_out, key_out, count_out, gate, st);
+    if ((rc = topk_reset_header(ws, st))) return rc;
+    const u32 grid = grid_for(r.count, Src::ITEMS, WARP ? 4 : 3, max_blocks);
+    k_topk_scan<Src, WARP><<<grid, SEL_THREADS, smem, st>>>(src, r, k, counts, lists, (u64 *)ws);
+    GUIDE_CUDA(cudaGetLastError());
+    return run_topk_merge(grid, k, negate, counts, lists, idx_out, key_out, count_out, nullptr, st);
 }
 
 template <class Src>
 static int run_topk_scan(const Src &src, Range r, u32 k, int negate, u32 max_blocks, unsigned char *ws, u64 *idx_out,
-                         double *key_out, u32 *count_out, cudaStream_t st, const u32 *gate = nullptr) {
+                         double *key_out, u32 *count_out, cudaStream_t st) {
     return k <= TOPK_WARP_K
-               ? run_topk_scan_mode<Src, true>(src, r, k, negate, max_blocks, ws, idx_out, key_out, count_out, gate, st)
-               : run_topk_scan_mode<Src, false>(src, r, k, negate, max_blocks, ws, idx_out, key_out, count_out, gate, st);
+               ? run_topk_scan_mode<Src, true>(src, r, k, negate, max_blocks, ws, idx_out, key_out, count_out, st)
+               : run_topk_scan_mode<Src, false>(src, r, k, negate, max_blocks, ws, idx_out, key_out, count_out, st);
 }
 
 template <int TIME_SUM, bool WARP>

@@ -1,5 +1,5 @@
-// Shared by the selection kernels (select.cu: accumulator-based scans and the fused kernels;
-// select_stream.cu: the sampled-bound streaming path over materialised metrics).
+// Shared by the selection kernels (select.cu: accumulator-based scans and the tiled fused kernels;
+// select_coop.cu: one launch over materialised metrics; select_stream.cu: sampled bound and model walk, fused).
 #pragma once
 #include <cstdlib>
 #include <cstring>
@@ -160,9 +160,10 @@ inline int launch_cooperative(void (*kernel)(KArgs...), u32 grid, u32 block, cud
 
 // ---- workspace headers (first 256 bytes of a selection workspace, zeroed at the start of a call) ----
 // top-k:  u64 at word 0: complement of the grid-wide key bound of the per-warp accumulators (0 = none);
-//         words 2..: the streaming path's tickets, candidate and sample counts, redo flag and (two u64 at word 6) its bound pair.
+//         words 2..: tickets, candidate and sample counts, redo flag and (two u64 at word 6) the bound pair of the fused form;
+//         the one-launch form uses the tickets for the chunks of its passes over the arrays and two candidate counts.
 // Pareto: word 0 ticket of the per-warp kernel, word 1 redo flag, word 2 ticket of the general kernel;
-//         words 4..: the streaming path's tickets, survivor count, killer count and front count.
+//         words 4..: tickets, survivor counts, killer count and front count of the fused and the one-launch form.
 enum { TK_TICKET = 2, TK_COUNT = 3, TK_REDO = 4, TK_SAMPLED = 5, TK_BOUND = 6, TK_TICKET2 = 10, TK_COUNT2 = 11 };
 enum { PH_TICKET = 4, PH_COUNT = 5, PH_KILLERS = 6, PH_FRONT = 7, PH_TICKET2 = 8, PH_COUNT2 = 9 };
 

@@ -1,6 +1,6 @@
-// What a kernel needs in order to decide whether a selection can still want a config: the sampled bound
-// of a top-k call, the dominating points ("killers") of a Pareto call, and the lists the survivors go
-// to.  Shared by the one-launch selection (select_coop.cu) and the fused one (select_stream.cu).
+// What a kernel needs in order to decide whether a selection can still want a config.  The sizes of the lists
+// survivors go to and the two comparisons serve the one-launch selection (select_coop.cu) too; the dominating
+// points ("killers") of a Pareto sample and the appends are the fused one's (select_stream.cu).
 #pragma once
 #include "select.cuh"
 

@@ -311,7 +311,7 @@ def guide_simulate_select(space: Space, out: dict, topk_cons: dict | None, key: 
                           topk_workspace, pareto_cons: dict | None, x: str, y: str, front_idx, front_count, pareto_workspace,
                           first=0, count=0, time_model=TIME_MAX, tp_model=TP_EXPLICIT, stream=None, sweep_events=None):
     """guide_simulate (closed form) + guide_select_topk + guide_pareto in one call: the metrics go to
-    `out`, the two answers to their tensors; on whole spaces the selections cost no pass of their own.
+    `out`, the two answers to their tensors.
     sweep_events: optional pair of torch.cuda.Event (already recorded once, so that they exist) that the
     library records right before and after the kernels that evaluate and store the metrics."""
     o = _outputs_struct(out)

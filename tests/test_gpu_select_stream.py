@@ -1,5 +1,6 @@
-"""GPU parity of the streaming selection path (sample -> bound / killers -> one filter pass ->
-exact finish) that materialised metrics of 2^18 configs or more go through.
+"""GPU parity of the selections that work from a sample (sample -> bound / killers -> one filter pass ->
+exact finish): the one-launch kernels over materialised metrics, and the fused form of whole spaces of
+2^18 configs or more.
 
 The metric arrays are written by the test (seeded), not by the simulation, so that the cases the
 bound and the killers must survive can be built directly: ties on the key, fewer passing configs
@@ -17,7 +18,7 @@ from gpu_util import run_pareto, run_simulate, run_simulate_select, run_topk
 pytestmark = pytest.mark.gpu
 
 U64_MAX = np.iinfo(np.uint64).max
-N_MIN = 1 << 18                      # smallest range the streaming path takes
+N_MIN = 1 << 18                      # smallest whole space the fused form's sample and model walk take
 
 
 def synth(n, seed, pass_frac=0.3):
@@ -120,16 +121,28 @@ def test_topk_sorted_inputs_and_winners_in_one_corner(sp):
 
 
 def test_topk_bound_in_two_kernels():
-    """The top-k bound is one cooperative kernel where the device launches cooperatively, two
-    kernels otherwise; GUIDE_NO_COOPERATIVE forces the second form.  The library reads the variable
-    once per process, so the check runs in a child process: same cases, same oracle."""
+    """The bound of the fused top-k is one cooperative kernel where the device launches cooperatively, two
+    kernels otherwise; GUIDE_NO_COOPERATIVE forces the second form (and takes materialised calls to the
+    accumulator kernels).  The library reads the variable once per process, so the check runs in a child
+    process: same cases, same oracle."""
     import os
     import subprocess
     import sys
     code = (
         "import sys; sys.path.insert(0, 'tests')\n"
+        "import numpy as np, oracle\n"
         "import test_gpu_select_stream as t\n"
+        "from gpu_util import run_topk\n"
         "from paper_2412_04788_b200 import guide, inputs as I\n"
+        "w = I.workload(2, scale=0.5)\n"
+        "sp2 = guide.Space(w['space'])\n"
+        "assert sp2.size >= t.N_MIN\n"
+        "want = oracle.simulate(w['space'])\n"
+        "for cons in ({}, {'max_latency': float(np.median(want['latency'][want['status'] == 0]))}, {'max_latency': 0.0}):\n"
+        "    for key, k in (('cost_per_token', 64), ('cost_per_hr', 128), ('throughput', 1), ('latency', 100)):\n"
+        "        idx, val, cnt = run_topk(sp2, None, cons, key, k)\n"
+        "        w_idx, w_val, w_cnt = oracle.select_topk(want, cons, key, k)\n"
+        "        assert cnt == w_cnt and np.array_equal(idx, w_idx) and np.array_equal(val, w_val), (cons, key, k)\n"
         "sp = guide.Space(I.workload(5, scale=0.125)['space'])\n"
         "for n, seed in ((t.N_MIN + 1, 21), (5 * t.N_MIN + 65, 22)):\n"
         "    host = t.synth(n, seed); dev = t.to_dev(host)\n"
@@ -192,8 +205,8 @@ def test_pareto_duplicates_keep_the_lowest_index(sp):
 
 
 def test_pareto_wide_fronts(sp):
-    """Anti-correlated metrics on part of the range: 1500 front points go through the streaming
-    path's own finish, 2048 are the most a front may have, 2049 and 6000 report the overflow marker
+    """Anti-correlated metrics on part of the range: 1500 front points go through the one-launch
+    kernel's own finish, 2048 are the most a front may have, 2049 and 6000 report the overflow marker
     (6000 also overflows the survivor list, so the general kernel redoes the call)."""
     n = 2 * N_MIN + 9
     rng = np.random.default_rng(15)

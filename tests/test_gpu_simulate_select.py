@@ -1,9 +1,7 @@
 """GPU parity of guide_simulate_select: the closed-form sweep, a top-k and a Pareto selection in
-one call (Sec. 3.2 Steps 1-3 with the constraints of Sec. 4.1).  On whole spaces that go through
-the line-wise kernels the selections are a by-product of the sweep (sampled bound and killers first,
-every config tested while its metrics are stored); everything else runs the three steps in turn.
-Either way the metric arrays must equal the oracle's simulation bit for bit, and the two answers
-the oracle's selections on those arrays, index for index."""
+one call (Sec. 3.2 Steps 1-3 with the constraints of Sec. 4.1), the three steps in turn on the stream.
+The metric arrays must equal the oracle's simulation bit for bit, and the two answers the oracle's
+selections on those arrays, index for index."""
 import numpy as np
 import pytest
 
@@ -30,8 +28,8 @@ def check(space_np, want, cons_t, key, k, cons_p, x, y, **kw):
 
 @pytest.mark.parametrize("tm,tpm", [(0, 0), (1, 1)])
 def test_an_eighth_of_workload_5_through_the_line_kernels(tm, tpm):
-    """2,097,152 configs, length axis of 64: memory kernel + line kernel with both selections riding
-    along.  Keys with many ties (cost per hour), negated keys (throughput), k from 1 to 128,
+    """2,097,152 configs, length axis of 64: memory kernel + line kernel, then both selections on what they
+    wrote.  Keys with many ties (cost per hour), negated keys (throughput), k from 1 to 128,
     constraints that differ between the two selections, and constraints nothing meets."""
     w = I.workload(5, scale=0.125)
     want = oracle.simulate(w["space"], time_model=tm, tp_model=tpm)
