@@ -692,6 +692,14 @@ struct Killers8 {
         }
         return alive;
     }
+    // the same of one point
+    __device__ __forceinline__ bool kills_high(u64 x, u64 y) const {
+        const u32 X = (u32)(x >> 32), Y = (u32)(y >> 32);
+        bool dead = false;
+#pragma unroll
+        for (u32 q = 0; q < CO_DIRS; q++) { const uint2 h = hi[q]; dead |= h.x < X && h.y < Y; }
+        return dead;
+    }
     // strictly dominated by one of them?
     __device__ __forceinline__ bool kills(u64 x, u64 y) const {
         bool dead = false;
@@ -941,33 +949,23 @@ k_pareto_coop(CoopSrc<NA> s, Range r, Walk w, u32 *header, P2 *local, P3 *surv, 
     const Killers8 K = {ks, kh};
     const u32 lim = min(out_cap, GUIDE_PARETO_MAX);
     // ---- filter: the sample itself when it was everything; else it makes the staircase, and one pass over the arrays ----
-    auto sample_left = [&]() {
-        u32 X[N_PTS], Y[N_PTS], alive = 0;
-#pragma unroll
-        for (u32 i = 0; i < N_PTS; i++) {
-            X[i] = (u32)(px[i] >> 32); Y[i] = (u32)(py[i] >> 32);
-            alive |= (px[i] == KEY_MAX && py[i] == KEY_MAX ? 0u : 1u) << i;
-        }
-        return __any_sync(0xFFFFFFFFu, alive) ? K.left(X, Y, alive) : 0u;
-    };
     if (WHOLE) {
-        const u32 alive = sample_left();
 #pragma unroll
         for (u32 i = 0; i < N_PTS; i++) {
-            if (!__any_sync(0xFFFFFFFFu, (alive >> i) & 1u)) continue;
+            const bool real = !(px[i] == KEY_MAX && py[i] == KEY_MAX);
+            if (!__any_sync(0xFFFFFFFFu, real)) continue;
             P3 e; e.x = px[i]; e.y = py[i];
             e.idx = r.first + ((u64)(i >> 1) * total_warps + gwarp) * ROW + 2 * lane + (i & 1);
-            const bool take = ((alive >> i) & 1u) && !K.kills(px[i], py[i]);
+            const bool take = real && !K.kills_high(px[i], py[i]) && !K.kills(px[i], py[i]);
             if (gridDim.x == 1) warp_append(take, e, &s_n, sv, CO_P_CHUNK);
             else warp_append(take, e, header + PH_COUNT, surv, PA_SURV_CAP);
         }
     } else {
         Staircase S(K);
         if (w.r >= CO_STAIR_RATIO) {
-            const u32 alive = sample_left();
 #pragma unroll
             for (u32 i = 0; i < N_PTS; i++)
-                if ((alive >> i) & 1u) S.put(gsteps, px[i], py[i]);
+                if (!(px[i] == KEY_MAX && py[i] == KEY_MAX) && !K.kills_high(px[i], py[i])) S.put(gsteps, px[i], py[i]);
             grid_barrier();
             S.read(gsteps, steps, part);
         }
