@@ -222,15 +222,28 @@ struct CudaDevice {
     static void release(void *p) { cudaFree(p); }
     // an id of the stream that no later one gets; 0 while it is being captured
     static unsigned long long stream_id(cudaStream_t st) {
-        cudaStreamCaptureStatus cap;
+        if (capturing(st)) return 0;                           // asking for the id would end the capture
         unsigned long long id = 0;
-        if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) { (void)cudaGetLastError(); return 0; }
-        if (cap != cudaStreamCaptureStatusNone) return 0;      // asking for the id would end the capture
         if (cudaStreamGetId(st, &id) != cudaSuccess) { (void)cudaGetLastError(); return 0; }
         return id + 1;
     }
+    static bool capturing(cudaStream_t st) {
+        cudaStreamCaptureStatus cap;
+        if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) { (void)cudaGetLastError(); return true; }
+        return cap != cudaStreamCaptureStatusNone;
+    }
 };
 static TablePool<CudaDevice> g_tables;
+
+// A handle is about to be used on a stream.  The id is asked for when the stream is another one than last time.  (A new
+// stream may have an old one's address: its uses then go by the old id, for which no block is asked for any more.)
+template <class OnDevice>
+static void used_on(OnDevice &d, cudaStream_t st) {
+    if (CudaDevice::capturing(st)) { d.block.used_on(0); d.stream = nullptr; return; }
+    if (d.block.stream != 0 && d.stream == (void *)st) return;
+    d.block.used_on(CudaDevice::stream_id(st));
+    d.stream = (void *)st;
+}
 
 // Work orders for the closed-form model kernel.  They decide which thread evaluates what, never a
 // value: any permutation gives the same outputs.
@@ -314,7 +327,7 @@ int space_on_device(guide_space *s, DSpace *out, unsigned **ticket, cudaStream_t
     for (DeviceTables &d : s->dev)
         if (d.device == dev) {
             *out = d.view;
-            if (ticket) d.block.used_on(CudaDevice::stream_id(st));      // a selection on given metrics reads no tables
+            if (ticket) used_on(d, st);      // a selection on given metrics reads no tables
             return ticket ? ticket_for(d, st, ticket) : GUIDE_OK;
         }
 
@@ -388,7 +401,7 @@ int space_on_device(guide_space *s, DSpace *out, unsigned **ticket, cudaStream_t
     d.view.n_m = (u32)n_m; d.view.n_h = (u32)n_h; d.view.n_f = (u32)n_f;
     d.view.n_b = (u32)s->batch.size(); d.view.n_t = (u32)s->tp.size(); d.view.n_l = (u32)s->pairs.size();
     d.tickets = (unsigned *)(blob + o_tk);
-    if (ticket) d.block.used_on(CudaDevice::stream_id(st));
+    if (ticket) used_on(d, st);
     s->dev.push_back(d);
     *out = d.view;
     return ticket ? ticket_for(s->dev.back(), st, ticket) : GUIDE_OK;
@@ -399,7 +412,7 @@ int trace_on_device(guide_trace *t, DTrace *out, cudaStream_t st) {
     GUIDE_CUDA(cudaGetDevice(&dev));
     std::lock_guard<std::mutex> lock(t->mu);
     for (DeviceTrace &d : t->dev)
-        if (d.device == dev) { *out = d.view; d.block.used_on(CudaDevice::stream_id(st)); return GUIDE_OK; }
+        if (d.device == dev) { *out = d.view; used_on(d, st); return GUIDE_OK; }
     const size_t n = t->arrival.size();
     const size_t o_a = 0, o_i = align_up(n * 8, 256), o_o = o_i + align_up(n * 4, 256), total = o_o + align_up(n * 4, 256);
     TableBlock block;
@@ -423,7 +436,7 @@ int trace_on_device(guide_trace *t, DTrace *out, cudaStream_t st) {
     d.view.sum_in = t->sum_in;
     d.view.n_zero = t->n_zero;
     d.view.together = t->together;
-    d.block.used_on(CudaDevice::stream_id(st));
+    used_on(d, st);
     t->dev.push_back(d);
     *out = d.view;
     return GUIDE_OK;
@@ -644,16 +657,16 @@ int guide_trace_load(const double *arrival, const uint32_t *in_len, const uint32
         } else t->n_zero++;
     }
     if (!rc) {
-        std::vector<uint32_t> len;                             // output lengths: the largest group of equal ones
-        for (uint64_t i = 0; i < n; i++)
-            if (in_len[i]) len.push_back(out_len[i]);
-        std::sort(len.begin(), len.end());
-        uint64_t most = t->n_zero;                             // these all take the config's
-        for (size_t i = 0, run = 0; i < len.size(); i++) {
-            run = i && len[i] == len[i - 1] ? run + 1 : 1;
-            most = std::max<uint64_t>(most, run);
+        // the length that more than half have, if there is one (0: the config's): pairs of different ones cancel out
+        auto length = [&](uint64_t i) { return in_len[i] ? out_len[i] : 0u; };
+        uint32_t most = 0;
+        uint64_t lead = 0, have = 0;
+        for (uint64_t i = 0; i < n; i++) {
+            if (lead == 0) most = length(i);
+            lead = length(i) == most ? lead + 1 : lead - 1;
         }
-        t->together = 2 * most >= n;
+        for (uint64_t i = 0; i < n; i++) have += length(i) == most;
+        t->together = 2 * have > n;
     }
     if (rc) { delete t; return rc; }
     *out = t;

@@ -30,6 +30,7 @@ static constexpr unsigned TICKET_SLOTS = 64;
 struct DeviceTables {
     int device = -1;
     TableBlock block;
+    void *stream = nullptr;          // it was last used on
     DSpace view{};
     unsigned *tickets = nullptr;     // TICKET_SLOTS slots, 32 words apart
     std::vector<void *> ticket_streams;   // slot i belongs to the calls on ticket_streams[i]
@@ -38,6 +39,7 @@ struct DeviceTables {
 struct DeviceTrace {
     int device = -1;
     TableBlock block;
+    void *stream = nullptr;          // it was last used on
     DTrace view{};
 };
 

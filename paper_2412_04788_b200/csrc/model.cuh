@@ -80,7 +80,7 @@ struct DTrace {
     u64 sum_out;                 // sum of out_len over requests with explicit lengths
     u64 sum_in;                  // sum of in_len over the same requests
     u32 n_zero;                  // number of requests taking the config's lengths
-    u32 together;                // at least half of the requests share one output length: those admitted together end together
+    u32 together;                // more than half of the requests share one output length: those admitted together end together
 };
 
 struct Cfg { u32 m, h, f, b, t, l; };

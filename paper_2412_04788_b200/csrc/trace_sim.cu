@@ -386,7 +386,7 @@ __device__ __noinline__ u32 retire_many(SlotArrays &sl, u64 *left, u32 *gen, dou
     return kept;
 }
 
-// TOGETHER: see retire_many; for traces in which at least half of the requests share their output length.  The call alone
+// TOGETHER: see retire_many; for traces in which more than half of the requests share their output length.  The call alone
 // costs the others 2-3 % (8,192 configs x 2,048 requests of their own lengths 26.2 ms with it, 25.7 without).
 template <int TIME_SUM, bool TOGETHER>
 __global__ void __launch_bounds__(SIM_THREADS, SIM_MIN_BLOCKS)
