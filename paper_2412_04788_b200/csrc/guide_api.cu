@@ -2,6 +2,8 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <exception>
+#include <memory>
 #include <mutex>
 #include <new>
 
@@ -17,8 +19,14 @@ int fail(int code, const char *fmt, ...) {
     va_start(ap, fmt);
     vsnprintf(buf, sizeof buf, fmt, ap);
     va_end(ap);
-    g_err = buf;
+    try { g_err = buf; } catch (...) { g_err.clear(); }
     return code;
+}
+
+// Containers throw when host memory runs out; nothing may leave the C entries that way.
+template <class F>
+static int no_throw(F f) {
+    try { return f(); } catch (const std::exception &) { return fail(GUIDE_ERR_INVALID, "out of host memory"); }
 }
 
 int cuda_fail(cudaError_t e, const char *what) {
@@ -320,7 +328,7 @@ static int ticket_for(DeviceTables &d, cudaStream_t st, unsigned **ticket) {
     return GUIDE_OK;
 }
 
-int space_on_device(guide_space *s, DSpace *out, unsigned **ticket, cudaStream_t st) {
+static int space_tables(guide_space *s, DSpace *out, unsigned **ticket, cudaStream_t st) {
     int dev = 0;
     GUIDE_CUDA(cudaGetDevice(&dev));
     std::lock_guard<std::mutex> lock(s->mu);
@@ -358,6 +366,7 @@ int space_on_device(guide_space *s, DSpace *out, unsigned **ticket, cudaStream_t
     put(o_hs, hf_sorted.data(), hf_sorted.size() * sizeof(HfSorted));
     put(o_po, plane_order.data(), plane_order.size() * 4);
     put(o_lo, line_order.data(), line_order.size() * 4);
+    s->dev.reserve(s->dev.size() + 1);                         // nothing throws between taking the block and keeping it
     TableBlock block;
     GUIDE_CUDA((cudaError_t)g_tables.take(off, CudaDevice::stream_id(st), &block));
     char *const blob = (char *)block.p;
@@ -407,7 +416,11 @@ int space_on_device(guide_space *s, DSpace *out, unsigned **ticket, cudaStream_t
     return ticket ? ticket_for(s->dev.back(), st, ticket) : GUIDE_OK;
 }
 
-int trace_on_device(guide_trace *t, DTrace *out, cudaStream_t st) {
+int space_on_device(guide_space *s, DSpace *out, unsigned **ticket, cudaStream_t st) {
+    return no_throw([&] { return space_tables(s, out, ticket, st); });
+}
+
+static int trace_arrays(guide_trace *t, DTrace *out, cudaStream_t st) {
     int dev = 0;
     GUIDE_CUDA(cudaGetDevice(&dev));
     std::lock_guard<std::mutex> lock(t->mu);
@@ -415,6 +428,7 @@ int trace_on_device(guide_trace *t, DTrace *out, cudaStream_t st) {
         if (d.device == dev) { *out = d.view; used_on(d, st); return GUIDE_OK; }
     const size_t n = t->arrival.size();
     const size_t o_a = 0, o_i = align_up(n * 8, 256), o_o = o_i + align_up(n * 4, 256), total = o_o + align_up(n * 4, 256);
+    t->dev.reserve(t->dev.size() + 1);
     TableBlock block;
     GUIDE_CUDA((cudaError_t)g_tables.take(total, CudaDevice::stream_id(st), &block));
     char *const blob = (char *)block.p;
@@ -440,6 +454,10 @@ int trace_on_device(guide_trace *t, DTrace *out, cudaStream_t st) {
     t->dev.push_back(d);
     *out = d.view;
     return GUIDE_OK;
+}
+
+int trace_on_device(guide_trace *t, DTrace *out, cudaStream_t st) {
+    return no_throw([&] { return trace_arrays(t, out, st); });
 }
 
 static bool pow2(uint32_t v) { return v && !(v & (v - 1)); }
@@ -511,7 +529,7 @@ extern "C" {
 
 const char *guide_last_error(void) { return g_err.c_str(); }
 
-int guide_space_create(const guide_space_desc *d, guide_space **out) {
+static int space_create(const guide_space_desc *d, guide_space **out) {
     if (!d || !out) return fail(GUIDE_ERR_INVALID, "desc and out are required");
     *out = nullptr;
     if (!d->models || !d->hw || !d->fw || !d->batch || !d->tp || !d->pairs)
@@ -520,8 +538,7 @@ int guide_space_create(const guide_space_desc *d, guide_space **out) {
         return fail(GUIDE_ERR_INVALID, "an axis is empty");
     if (d->n_models > 4096 || (uint64_t)d->n_hw * d->n_fw > 65536)
         return fail(GUIDE_ERR_INVALID, "too many models (max 4096) or hardware x framework pairs (max 65536)");
-    guide_space *s = new (std::nothrow) guide_space;
-    if (!s) return fail(GUIDE_ERR_INVALID, "out of host memory");
+    std::unique_ptr<guide_space> s(new guide_space);
     s->models.assign(d->models, d->models + d->n_models);
     s->hw.assign(d->hw, d->hw + d->n_hw);
     s->fw.assign(d->fw, d->fw + d->n_fw);
@@ -596,9 +613,13 @@ int guide_space_create(const guide_space_desc *d, guide_space **out) {
     }
     if (!rc) rc = check_closed_form_overflow(*s);
     if (!rc) s->exact = closed_form_exact(*s);
-    if (rc) { delete s; return rc; }
-    *out = s;
+    if (rc) return rc;
+    *out = s.release();
     return GUIDE_OK;
+}
+
+int guide_space_create(const guide_space_desc *d, guide_space **out) {
+    return no_throw([&] { return space_create(d, out); });
 }
 
 void guide_space_destroy(guide_space *s) {
@@ -631,14 +652,13 @@ int guide_space_decode(const guide_space *s, uint64_t idx, guide_config *o) {
     return GUIDE_OK;
 }
 
-int guide_trace_load(const double *arrival, const uint32_t *in_len, const uint32_t *out_len, uint64_t n,
+static int trace_load(const double *arrival, const uint32_t *in_len, const uint32_t *out_len, uint64_t n,
                      guide_trace **out) {
     if (!out) return fail(GUIDE_ERR_INVALID, "out is required");
     *out = nullptr;
     if (!arrival || !in_len || !out_len) return fail(GUIDE_ERR_INVALID, "a trace array is NULL");
     if (n == 0 || n > 65536) return fail(GUIDE_ERR_INVALID, "n_req must be in 1..65536");
-    guide_trace *t = new (std::nothrow) guide_trace;
-    if (!t) return fail(GUIDE_ERR_INVALID, "out of host memory");
+    std::unique_ptr<guide_trace> t(new guide_trace);
     t->arrival.assign(arrival, arrival + n);
     t->in_len.assign(in_len, in_len + n);
     t->out_len.assign(out_len, out_len + n);
@@ -668,9 +688,14 @@ int guide_trace_load(const double *arrival, const uint32_t *in_len, const uint32
         for (uint64_t i = 0; i < n; i++) have += length(i) == most;
         t->together = 2 * have > n;
     }
-    if (rc) { delete t; return rc; }
-    *out = t;
+    if (rc) return rc;
+    *out = t.release();
     return GUIDE_OK;
+}
+
+int guide_trace_load(const double *arrival, const uint32_t *in_len, const uint32_t *out_len, uint64_t n,
+                     guide_trace **out) {
+    return no_throw([&] { return trace_load(arrival, in_len, out_len, n, out); });
 }
 
 void guide_trace_destroy(guide_trace *t) {

@@ -171,3 +171,27 @@ def test_simulate_select_refuses_bad_arguments_before_any_gpu_work():
     opts = guide.SimOpts(0, 0, 0, 0, 0, 1, 0)                          # clamp_seq: the separate calls only
     assert L.guide_simulate_select(sp.handle, C.byref(opts), C.byref(out), C.byref(sel), None, 0, None, 0, None) == guide.GUIDE_ERR_UNSUPPORTED
     assert guide.guide_last_error()
+
+
+def test_out_of_host_memory_is_an_error_not_an_abort():
+    """Four gigabytes of length pairs that cannot be copied under the process's limit: an error code with a message
+    (the pairs are pages that were never touched)."""
+    import subprocess
+    import sys
+    code = (
+        "import ctypes as C, mmap, resource\n"
+        "from paper_2412_04788_b200 import guide, inputs as I\n"
+        "L = guide.lib()\n"
+        "n = 1 << 29\n"
+        "m = mmap.mmap(-1, 8 * n, flags=mmap.MAP_PRIVATE | mmap.MAP_ANONYMOUS)\n"
+        "pairs = C.cast((C.c_char * 1).from_buffer(m), C.POINTER(guide.LenPair))\n"
+        "one = (C.c_uint32 * 1)(1)\n"
+        "desc = guide.SpaceDesc((guide.Model * 1)(), 1, (guide.Hw * 1)(), 1, (guide.Fw * 1)(), 1, one, 1, one, 1, pairs, n, None)\n"
+        "size = int(open('/proc/self/statm').read().split()[0]) * resource.getpagesize()\n"
+        "resource.setrlimit(resource.RLIMIT_AS, (size + (1 << 30), size + (1 << 30)))\n"
+        "h = C.c_void_p()\n"
+        "rc = L.guide_space_create(C.byref(desc), C.byref(h))\n"
+        "print('rc', rc, h.value, guide.guide_last_error())\n")
+    res = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=120)
+    assert res.returncode == 0, (res.returncode, res.stderr[-500:])
+    assert res.stdout.strip() == f"rc {guide.GUIDE_ERR_INVALID} None out of host memory", res.stdout
